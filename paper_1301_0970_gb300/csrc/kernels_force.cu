@@ -328,8 +328,21 @@ __global__ void __launch_bounds__(NT) k_force(ForceArgs a, int zchunk) {
 // forms the gradients, Eq. 7 and du, and the RMS-ID partials.  Pass 1 costs
 // 6 + 4k bytes per voxel of extra traffic (written, then read once), but
 // both passes keep all warps busy instead of waiting at per-plane barriers.
+//
+// Pass 1 marches a column along z and keeps the four corners of the cell's
+// high plane: where the next voxel's cell is the one above it (91 % of the
+// voxels at the end of a 512x512x160 registration: u is smooth) they are its
+// low plane and only four new corners are gathered.  The gathers are bound by
+// the L1's wavefronts (51 % of its peak with all eight, and most of the rest
+// waiting for them); half the gathers also take half the registers, so 5 CTAs
+// per SM stay resident (two planes' 16 gathers in flight took 64 registers, 4
+// CTAs).  512x512x160 inside a registration, contour terms on: 259 -> 220 us;
+// 4 or 6 CTAs per SM and the next plane's gathers issued ahead of the current
+// plane's interpolation measured slower (243, 250, 251 against 217 us alone).
+// The structure terms always come as texels here: a runtime choice between
+// texels and image + bits at each plane cost all of that gain.
 template <bool CONTOUR, typename IT>
-__global__ void __launch_bounds__(NT, 4) k_warp_pass(ForceArgs a, int zw) {
+__global__ void __launch_bounds__(NT, 5) k_warp_pass(ForceArgs a, int zw) {
     if (a.stop_flag && *a.stop_flag) return;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int x = blockIdx.x * TX + threadIdx.x, y = blockIdx.y * TY + threadIdx.y;
@@ -337,31 +350,31 @@ __global__ void __launch_bounds__(NT, 4) k_warp_pass(ForceArgs a, int zw) {
     const int nxy = nx * ny, N = nxy * nz;
     const int zb = blockIdx.z * zw, ze = min(zb + zw, nz);
     const float *__restrict__ u = a.u;
-    // two planes at a time: both points' 16 corner loads are in flight
-    // together, and the next two planes' displacements load meanwhile
     const int col = y * nx + x;
     auto disp = [&](int z, float &dx, float &dy, float &dz) {
         const int i = z * nxy + col;
         dx = __ldg(u + i); dy = __ldg(u + N + i); dz = __ldg(u + N + N + i);
     };
+    // displacements two planes ahead
     float ax = 0.f, ay = 0.f, az = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
     if (zb < ze) disp(zb, ax, ay, az);
     if (zb + 1 < ze) disp(zb + 1, bx, by, bz);
-    int z = zb;
-    for (; z + 1 < ze; z += 2) {
-        CornerSet<IT> c0, c1;
-        corner_load<CONTOUR, IT>(a, ax, ay, az, x, y, z, c0);
-        corner_load<CONTOUR, IT>(a, bx, by, bz, x, y, z + 1, c1);
-        if (z + 2 < ze) disp(z + 2, ax, ay, az);
-        if (z + 3 < ze) disp(z + 3, bx, by, bz);
-        corner_finish<CONTOUR, IT>(a, z * nxy + col, N, c0);
-        corner_finish<CONTOUR, IT>(a, (z + 1) * nxy + col, N, c1);
+    CornerQuad<IT> A = {}, B = {};
+    int held = -1, z = zb;             // low corner of the plane whose corners `lo` holds (-1: none)
+    auto step = [&](CornerQuad<IT> &lo, CornerQuad<IT> &hi, float &ux, float &uy, float &uz) {
+        const Cell w = corner_cell(a, ux, uy, uz, x, y, z);
+        corner_quad<CONTOUR, IT>(a, w.hi, w.dx, w.dy, hi);
+        if (w.lo != held) corner_quad<CONTOUR, IT>(a, w.lo, w.dx, w.dy, lo);
+        held = w.hi;
+        if (z + 2 < ze) disp(z + 2, ux, uy, uz);
+        corner_finish<CONTOUR, IT>(a, z * nxy + col, N, w, lo, hi);
+        ++z;
+    };
+    while (z + 1 < ze) {               // the two register sets swap roles: no copies
+        step(A, B, ax, ay, az);
+        step(B, A, bx, by, bz);
     }
-    if (z < ze) {
-        CornerSet<IT> c0;
-        corner_load<CONTOUR, IT>(a, ax, ay, az, x, y, z, c0);
-        corner_finish<CONTOUR, IT>(a, z * nxy + col, N, c0);
-    }
+    if (z < ze) step(A, B, ax, ay, az);
 }
 
 // Sums over a set m of structures (bit j = structure j), one table entry
@@ -1228,9 +1241,11 @@ __global__ void __launch_bounds__(NT, 2) k_level_coop(const __grid_constant__ Le
         // ---- pass 1: warp
         for (int i = gt; i < N; i += gs) {
             const int x = i % nx, y = (i / nx) % ny, z = i / nxy;
-            CornerSet<IT> cs;
-            corner_load<CONTOUR, IT>(a, __ldcg(u + i), __ldcg(u + N + i), __ldcg(u + N + N + i), x, y, z, cs);
-            corner_finish<CONTOUR, IT>(a, i, N, cs);
+            const Cell w = corner_cell(a, __ldcg(u + i), __ldcg(u + N + i), __ldcg(u + N + N + i), x, y, z);
+            CornerQuad<IT> lo, hi;
+            corner_quad<CONTOUR, IT>(a, w.lo, w.dx, w.dy, lo);
+            corner_quad<CONTOUR, IT>(a, w.hi, w.dx, w.dy, hi);
+            corner_finish<CONTOUR, IT>(a, i, N, w, lo, hi);
         }
         if (!grid_barrier(p.bar, nb, p.err)) return;
         // ---- pass 2: force and the RMS-ID sums
@@ -1477,7 +1492,7 @@ static cudaError_t launch_force_t(const ForceArgs &a, int zchunk, dim3 grid, dim
                                   int *err) {
     const bool contour = a.contour && a.k > 0;
     const size_t N = (size_t)a.nx * a.ny * a.nz;
-    if (a.wfield != nullptr && N < (size_t)1 << 31) {
+    if (a.wfield != nullptr && N < (size_t)1 << 31 && (!contour || a.mtex != nullptr)) {
         const int zc = two_pass_zchunk(a.nx, a.ny, a.nz);
         dim3 g(grid.x, grid.y, (a.nz + zc - 1) / zc);
         // pass 2 marches the caller's (longer) z chunks: fewer CTAs, so fewer

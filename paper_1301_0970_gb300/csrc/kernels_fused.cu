@@ -368,7 +368,8 @@ __global__ void __launch_bounds__(FT) k_fused_smooth_warp(const __grid_constant_
     if (!tile_smooth<R>(&tin, use_tma != 0, in, t, nx, ny, nz, x0, y0, z0, sm.S, sm.X, sm.bar, err, tid)) return;
     const float *Z = sm.X;
     const int nxy = nx * ny, N = nxy * nz;
-    CornerSet<IT> cs[kVoxPerThread];
+    Cell cell[kVoxPerThread];
+    CornerQuad<IT> lo[kVoxPerThread], hi[kVoxPerThread];
     int iv[kVoxPerThread];
 #pragma unroll
     for (int v = 0; v < kVoxPerThread; ++v) {
@@ -382,11 +383,13 @@ __global__ void __launch_bounds__(FT) k_fused_smooth_warp(const __grid_constant_
         u[i] = sx;
         u[N + i] = sy;
         u[N + N + i] = sz;
-        corner_load<CONTOUR, IT>(a, sx, sy, sz, x, y, z, cs[v]);
+        cell[v] = corner_cell(a, sx, sy, sz, x, y, z);
+        corner_quad<CONTOUR, IT>(a, cell[v].lo, cell[v].dx, cell[v].dy, lo[v]);
+        corner_quad<CONTOUR, IT>(a, cell[v].hi, cell[v].dx, cell[v].dy, hi[v]);
     }
 #pragma unroll
     for (int v = 0; v < kVoxPerThread; ++v)
-        if (iv[v] >= 0) corner_finish<CONTOUR, IT>(a, iv[v], N, cs[v]);
+        if (iv[v] >= 0) corner_finish<CONTOUR, IT>(a, iv[v], N, cell[v], lo[v], hi[v]);
 }
 
 // Tensor map of a [3][nz][ny][nx] field for the tile box; false if TMA
@@ -447,7 +450,8 @@ cudaError_t warp_r(const float *in, const Taps &t, float *u, const ForceArgs &a,
 }  // namespace
 
 bool fused_schedule_ok(const ForceArgs &a) {
-    return a.wfield != nullptr && (size_t)a.nx * a.ny * a.nz < (size_t)1 << 31;
+    return a.wfield != nullptr && (!(a.contour && a.k > 0) || a.mtex != nullptr) &&
+           (size_t)a.nx * a.ny * a.nz < (size_t)1 << 31;
 }
 
 cudaError_t launch_fused_smooth_compose(const float *du, const float *u, int mode, float sigma, int nx, int ny,

@@ -10,27 +10,25 @@
 
 namespace cgdir {
 
-// The eight corners of one interpolation point, loaded (pass 1).  Values of
-// 16-bit images stay raw until corner_finish converts them: a conversion at
-// the load would wait for the load there, before the other gathers of the
-// thread are issued.
-//   c  values (float images)
-//   h  raw 16-bit values (16-bit images without texels)
-//   m  words whose bits sh .. sh + 7 are the corners' moving-mask bits
-//      (mask_shift): for 16-bit texels the whole texel word (value in the
-//      low half, sh = 16), otherwise the bits alone (sh = 0)
-template <typename IT>
-struct CornerSet {
-    float c[8];
-    unsigned short h[8];
-    unsigned m[8];
+// One interpolation point: the weights and the linear indices of the low
+// corners of its two planes (lo, hi; equal at the last plane), and the index
+// steps to the high corners in x and y (0 at the border).
+struct Cell {
     float wx, wy, wz;
+    int lo, hi, dx, dy;
 };
 
-template <bool CONTOUR, typename IT>
-__device__ __forceinline__ int mask_shift(const ForceArgs &a) {
-    return (CONTOUR && sizeof(IT) == 2 && a.mtex != nullptr) ? 16 : 0;
-}
+// The four corners of one plane of a cell, loaded.  Values of 16-bit images
+// stay raw until corner_finish converts them: a conversion at the load would
+// wait for the load there, before the other gathers of the thread are issued.
+//   c  values (float images)
+//   m  float images: the corners' moving-mask bits; 16-bit images: the raw
+//      value in the low half, mask bits in bits 16-23 (the texel word)
+template <typename IT>
+struct CornerQuad {
+    float c[4];
+    unsigned m[4];
+};
 
 // The float value of a raw 16-bit image value (the low half of w).
 template <typename IT>
@@ -44,69 +42,69 @@ __device__ __forceinline__ float from_raw16<__nv_bfloat16>(unsigned w) {
 template <>
 __device__ __forceinline__ float from_raw16<float>(unsigned w) { return __uint_as_float(w); }   // not used
 
-// Clamp x + u, find the corners and issue their loads (texels when the
-// structure terms are on and texels exist, else image values and mask bits).
-template <bool CONTOUR, typename IT>
-__device__ __forceinline__ void corner_load(const ForceArgs &a, float ux, float uy, float uz, int x, int y, int z,
-                                            CornerSet<IT> &cs) {
-    using TT = typename TexOf<IT>::type;
+// Clamp x + u and find the corners.
+__device__ __forceinline__ Cell corner_cell(const ForceArgs &a, float ux, float uy, float uz, int x, int y, int z) {
     const int nx = a.nx, ny = a.ny, nz = a.nz, nxy = nx * ny;
     const float px = fminf(fmaxf((float)x + ux, 0.f), (float)(nx - 1));
     const float py = fminf(fmaxf((float)y + uy, 0.f), (float)(ny - 1));
     const float pz = fminf(fmaxf((float)z + uz, 0.f), (float)(nz - 1));
     const float fx = floorf(px), fy = floorf(py), fz = floorf(pz);
     const int ix = (int)fx, iy = (int)fy, iz = (int)fz;
-    cs.wx = px - fx; cs.wy = py - fy; cs.wz = pz - fz;
-    const int dx = ix < nx - 1 ? 1 : 0, dy = iy < ny - 1 ? nx : 0, dz = iz < nz - 1 ? nxy : 0;
-    const int b0 = iz * nxy + iy * nx + ix;
-    const int o[8] = {0, dx, dy, dy + dx, dz, dz + dx, dz + dy, dz + dy + dx};
-    if (CONTOUR && a.mtex != nullptr) {
-        const TT *__restrict__ q0 = static_cast<const TT *>(a.mtex) + b0;
+    Cell w;
+    w.wx = px - fx; w.wy = py - fy; w.wz = pz - fz;
+    w.dx = ix < nx - 1 ? 1 : 0; w.dy = iy < ny - 1 ? nx : 0;
+    w.lo = iz * nxy + iy * nx + ix;
+    w.hi = w.lo + (iz < nz - 1 ? nxy : 0);
+    return w;
+}
+
+// Issue the loads of the four corners b, b + dx, b + dy, b + dy + dx of one
+// plane (texels when the structure terms are on, else image values).
+template <bool CONTOUR, typename IT>
+__device__ __forceinline__ void corner_quad(const ForceArgs &a, int b, int dx, int dy, CornerQuad<IT> &cs) {
+    const int o[4] = {0, dx, dy, dy + dx};
+    const void *base = CONTOUR ? a.mtex : a.I0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
         if (sizeof(IT) == 2) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) cs.m[q] = (unsigned)__ldg(reinterpret_cast<const uint32_t *>(q0 + o[q]));
+            cs.m[q] = CONTOUR ? (unsigned)__ldg(static_cast<const uint32_t *>(base) + b + o[q])
+                              : (unsigned)__ldg(static_cast<const unsigned short *>(base) + b + o[q]);
+        } else if (CONTOUR) {
+            const float2 t = __ldg(static_cast<const float2 *>(base) + b + o[q]);
+            cs.c[q] = t.x;
+            cs.m[q] = __float_as_uint(t.y);
         } else {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float2 t = __ldg(reinterpret_cast<const float2 *>(q0 + o[q]));
-                cs.c[q] = t.x;
-                cs.m[q] = __float_as_uint(t.y);
-            }
-        }
-    } else {
-        const IT *__restrict__ q0 = static_cast<const IT *>(a.I0) + b0;
-        if (sizeof(IT) == 2) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) cs.h[q] = __ldg(reinterpret_cast<const unsigned short *>(q0 + o[q]));
-        } else {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) cs.c[q] = __ldg(reinterpret_cast<const float *>(q0 + o[q]));
-        }
-        if (CONTOUR) {
-            const uint8_t *__restrict__ r0 = a.mbits + b0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) cs.m[q] = __ldg(r0 + o[q]);
+            cs.c[q] = __ldg(static_cast<const float *>(base) + b + o[q]);
         }
     }
 }
 
-// Interpolate I0~ from the loaded corners, write it, the corner bits'
-// AND / OR and, where they disagree, P_j.
+template <typename IT>
+__device__ __forceinline__ float corner_value(const CornerQuad<IT> &cs, int q) {
+    return sizeof(IT) == 4 ? cs.c[q] : from_raw16<IT>(cs.m[q]);
+}
+
+// Interpolate I0~ at voxel i from the loaded corners of the cell's low and
+// high plane, write it, the corner bits' AND / OR and, where they disagree, P_j.
 template <bool CONTOUR, typename IT>
-__device__ __forceinline__ void corner_finish(const ForceArgs &a, int i, int N, const CornerSet<IT> &cs) {
-    const float wx = cs.wx, wy = cs.wy, wz = cs.wz;
+__device__ __forceinline__ void corner_finish(const ForceArgs &a, int i, int N, const Cell &w,
+                                              const CornerQuad<IT> &lo, const CornerQuad<IT> &hi) {
+    const float wx = w.wx, wy = w.wy, wz = w.wz;
     float c[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q)
-        c[q] = sizeof(IT) == 4 ? cs.c[q]
-                               : (CONTOUR && a.mtex != nullptr ? from_raw16<IT>(cs.m[q]) : from_raw16<IT>(cs.h[q]));
+    for (int q = 0; q < 4; ++q) {
+        c[q] = corner_value<IT>(lo, q);
+        c[4 + q] = corner_value<IT>(hi, q);
+    }
     const float e00 = fmaf(wx, c[1] - c[0], c[0]), e10 = fmaf(wx, c[3] - c[2], c[2]);
     const float e01 = fmaf(wx, c[5] - c[4], c[4]), e11 = fmaf(wx, c[7] - c[6], c[6]);
     const float f0 = fmaf(wy, e10 - e00, e00), f1 = fmaf(wy, e11 - e01, e01);
     a.wfield[i] = fmaf(wz, f1 - f0, f0);
     if (CONTOUR) {
-        const unsigned *m = cs.m;
-        const int sh = mask_shift<CONTOUR, IT>(a);
+        unsigned m[8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) { m[q] = lo.m[q]; m[4 + q] = hi.m[q]; }
+        constexpr int sh = sizeof(IT) == 2 ? 16 : 0;      // where the mask bits lie in m
         // the words hold nothing above the mask bits (texel bits 24-31 are zero)
         const unsigned andb = (m[0] & m[1] & m[2] & m[3] & m[4] & m[5] & m[6] & m[7]) >> sh;
         const unsigned orb = (m[0] | m[1] | m[2] | m[3] | m[4] | m[5] | m[6] | m[7]) >> sh;

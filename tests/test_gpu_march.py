@@ -1,0 +1,62 @@
+"""Kernels that march along z and keep values between planes, at the sizes and
+displacements where that can go wrong, against the FP64 oracle.
+
+Tolerance: as in the parity tests, 1e-5 of the reference's scale for values
+that a few dozen FP32 operations form (about 6e-8 relative rounding each).
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - CPU container
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_1301_0970_gb300 as cg  # noqa: E402
+
+DEV = torch.device("cuda:0")
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    with cg.Context(0) as c:
+        yield c
+
+
+def field(kind, shape, rng):
+    """Displacements [3][nz][ny][nx]: slowly varying (the cell moves up by one
+    plane from voxel to voxel), jumping (it does not), or beyond the border."""
+    nz, ny, nx = shape
+    z, y, x = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")
+    if kind == "smooth":
+        u = np.stack([1.3 * np.sin(0.21 * x + 0.13 * z), 0.9 * np.cos(0.17 * y) + 0.4, -0.7 + 0.05 * z])
+    elif kind == "jumping":
+        u = rng.uniform(-2.5, 2.5, (3, nz, ny, nx))
+    else:
+        u = np.stack([np.full(shape, 2.0 * nx), np.full(shape, -3.0), np.where(z % 2 == 0, 1.5 * nz, -1.5 * nz)])
+    return u.astype(np.float32)
+
+
+@pytest.mark.parametrize("kind", ["smooth", "jumping", "outside"])
+@pytest.mark.parametrize("shape", [(1, 5, 36), (2, 9, 33), (3, 8, 32), (9, 10, 65), (70, 6, 40)])
+def test_force_warp_pass(ctx, shape, kind):
+    """I0~ of the force step (its `warped` output), structure terms on and off."""
+    rng = np.random.default_rng(hash_of(shape))
+    img = rng.uniform(-1000, 700, shape).astype(np.float32)
+    u = field(kind, shape, rng)
+    bits = rng.integers(0, 4, shape, dtype=np.uint8)
+    ref = oracle.warp(img, u)
+    d = [torch.from_numpy(a).to(DEV) for a in (img, u, bits)]
+    for contour in (False, True):
+        out = torch.empty_like(d[0])
+        ctx.force(d[0], d[0], d[2], d[2], [1e-3] * 2, [1, -1], d[1], contour=contour, warped=out)
+        torch.cuda.synchronize()
+        err = np.abs(out.cpu().numpy().astype(np.float64) - ref).max()
+        assert err <= 1e-5 * np.abs(img).max(), (contour, err)
+
+
+def hash_of(shape):
+    return shape[0] * 10007 + shape[1] * 101 + shape[2]
