@@ -193,7 +193,7 @@ void cgdir_default_params(cgdir_params *p);
                                  cgdir_register when no other request is
                                  running at submission, else the throughput one)
      CGDIR_SHARED_WIDE_CAP=n     z-march smoothing CTAs per SM in batched and
-                                 shared served registrations (default 2; 0: no cap) */
+                                 shared served registrations (default 4; 0: no cap) */
 int cgdir_create(cgdir_ctx **out, const cgdir_config *cfg);
 
 /* Release every device buffer, cached graph and (if owned) stream of ctx.
@@ -337,7 +337,7 @@ int cgdir_compose(cgdir_ctx *ctx, const float *u, const float *du, int mode, flo
    (CGDIR_ADDITIVE), G the Gaussian of sigma voxels (0 <= sigma <= 2; 0 is
    no smoothing).  The kernels are the context's forced smoothing variant
    (CGDIR_SMOOTH at creation; under CGDIR_SMOOTH=fused one 3-D tile kernel
-   for both steps), else chosen by size; every choice gives the same bits.
+   for both steps), else the z-march; every choice gives the same bits.
    Fields [3][nz][ny][nx] FP32 in device memory; out must not alias u or
    du.  Errors: EINVAL, ENOMEM, ECUDA. */
 int cgdir_smooth_compose(cgdir_ctx *ctx, const float *du, const float *u, int mode, float sigma,
@@ -466,7 +466,7 @@ int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us);
  * shape shaped like a registration's, the candidate configurations of the
  * force stencil pass (four z-chunk lengths, four or two voxels per thread)
  * and of the smoothing with the composite update (steps 2-4 of an
- * iteration, timed behind a force step: the 64 x 16 TMA z-march with the
+ * iteration, timed behind a force step: the 32 x 32 z-march with the
  * volume in 1 to 16 z chunks, the 32 x 16 one with 2, 4 and 8, 3-D
  * shared-memory tile, split xy + z kernels with the update in the z pass)
  * on ctx's stream and keeps the fastest, then times the fused schedule
@@ -484,7 +484,7 @@ int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us);
                                   smooth_ms / force_ms are then those kernels' times (the
                                   per-step alternative is kept but not reported; a loaded
                                   table that says FUSED picks the per-step kernels by size) */
-#define CGDIR_SMOOTH_MARCH32 5 /* the 32 x 16 z-march where the 64 x 16 one would apply */
+#define CGDIR_SMOOTH_MARCH32 5 /* the z-march on 32 x 16 instead of 32 x 32 tiles */
 typedef struct {
     int   nx, ny, nz;           /* level shape                                   */
     int   contour;              /* structure terms on at this level               */

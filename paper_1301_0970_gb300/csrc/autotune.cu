@@ -3,10 +3,10 @@
 // data of that shape, the candidate launch configurations of the two
 // kernels whose best configuration depends on the shape:
 //   smoothing (with the composite update, i.e. steps 2-4 of an iteration):
-//              the TMA z-march with its default z chunk, half, double and
-//              four times that chunk (plus the separate update kernel), the 3-D
-//              shared-memory tile kernel (idem), and the split xy + z
-//              kernels with the update fused into the z pass;
+//              the z-march with its estimated z chunk and the volume in 1 to
+//              16 chunks, on 32 x 32 and 32 x 16 tiles (plus the separate
+//              update kernel), the 3-D shared-memory tile kernel (idem), and
+//              the split xy + z kernels with the update fused into the z pass;
 //   force:     the stencil pass with the default z chunk, half, a quarter
 //              and double;
 // then the fused schedule (force stencil pass alone, 3-D tiles of G(du)
@@ -77,9 +77,9 @@ static const TunedLevel *find_tuned(const cgdir_ctx *ctx, int nx, int ny, int nz
 
 SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt, bool allow_fused) {
     SmoothChoice ch;
-    // registrations that share the GPU (batched, served) cap the wide z-march
-    // at two CTAs per SM: three fill an SM's shared memory and registers and
-    // starve the other registrations' kernels
+    // registrations that share the GPU (batched, served) cap the z-march's
+    // CTAs per SM: uncapped they fill an SM's registers and starve the other
+    // registrations' kernels
     if (!allow_fused) ch.ctas_per_sm = ctx->shared_wide_cap;
     if (ctx->smooth_variant != SMOOTH_AUTO || ctx->smooth_zchunk > 0) {
         ch.variant = ctx->smooth_variant;
@@ -220,7 +220,7 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
     }
     if (rc == CGDIR_OK) {
         float bt = 1e30f;
-        const int d = smooth_default_zchunk(nx, ny, nz, 3);
+        const int d = smooth_default_zchunk(nx, ny, nz, 3, sigma);
         SmoothChoice cand[16];
         int nc = 0;
         auto add = [&](int variant, int zc) {
@@ -229,21 +229,16 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
             cand[nc].variant = variant;
             cand[nc++].zchunk = zc;
         };
-        if (nx % 4 == 0) {
-            // z chunks: the default and the volume cut into 1 .. 16 chunks
-            // (longer chunks reload fewer halo planes; more chunks fill more
-            // SMs, and the count of CTAs against whole waves decides which
-            // wins); the 32 x 16 z-march with 2, 4 and 8 chunks where the
-            // 64 x 16 one applies (more CTAs per chunk on small levels)
-            add(SMOOTH_MARCH, d);
-            const int nch[7] = {1, 2, 3, 4, 6, 8, 16};
-            for (int q = 0; q < 7; ++q) add(SMOOTH_MARCH, (nz + nch[q] - 1) / nch[q]);
-            if (nx % 8 == 0)
-                for (int c = 2; c <= 8; c *= 2) add(SMOOTH_MARCH_NARROW, (nz + c - 1) / c);
-        }
+        // z chunks: the estimated best and the volume cut into 1 .. 16 chunks
+        // (longer chunks reload fewer halo planes; more chunks fill more SMs);
+        // the 32 x 16 z-march with 2, 4 and 8 chunks (more CTAs per chunk on
+        // small levels)
+        add(SMOOTH_MARCH, d);
+        const int nch[7] = {1, 2, 3, 4, 6, 8, 16};
+        for (int q = 0; q < 7; ++q) add(SMOOTH_MARCH, (nz + nch[q] - 1) / nch[q]);
+        for (int c = 2; c <= 8; c *= 2) add(SMOOTH_MARCH_NARROW, (nz + c - 1) / c);
         cand[nc].variant = SMOOTH_TILE; cand[nc++].zchunk = 0;
         cand[nc].variant = SMOOTH_SPLIT; cand[nc++].zchunk = 0;
-        const SmoothChoice dflt{smooth_auto_variant(nx, ny, nz), 0};
         for (int ci = 0; ci < nc && rc == CGDIR_OK; ++ci) {
             float ms = 0.f;
             // one iteration: the force step (so du and the caches are as in a
@@ -259,9 +254,7 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 return launch_smooth(out, 3, sigma, nx, ny, nz, du, nullptr, st, kerr(ctx), cand[ci], sscr);
             });
             ms = std::max(ms - best.force_ms, 0.f);
-            const bool is_default = cand[ci].variant == dflt.variant &&
-                                    (cand[ci].variant == SMOOTH_TILE || cand[ci].zchunk == d);
-            if (is_default) best.default_smooth_ms = ms;
+            if (ci == 0) best.default_smooth_ms = ms;      // the untuned choice
             if (rc == CGDIR_OK && ms < bt) {
                 bt = ms;
                 best.smooth_variant = cand[ci].variant;

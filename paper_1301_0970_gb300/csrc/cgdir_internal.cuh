@@ -181,23 +181,22 @@ cudaError_t launch_finalize(const double *partial, int nblocks, LevelState st, i
 // fused iteration schedule (3-D tiles of all three components with the
 // composite update fused into the du pass and the next warp into the u
 // pass; a standalone smoothing takes the tile kernel), or chosen by size.
-// SMOOTH_MARCH takes the wide-tile z-march (64 x 16 tiles, nx % 8 == 0, R <= 4)
-// where it applies, else the 32 x 16 one; SMOOTH_MARCH_NARROW always the
-// 32 x 16 one (same bits; a context setting for comparisons, never tuned).
+// SMOOTH_AUTO takes the z-march at every size (its z chunks fill the SMs also
+// on small levels: 64x64x32 5 us against 11 for the tile kernel);
+// SMOOTH_MARCH_NARROW is its 32 x 16 tile (same bits).
 enum { SMOOTH_AUTO = 0, SMOOTH_MARCH = 1, SMOOTH_TILE = 2, SMOOTH_SPLIT = 3, SMOOTH_FUSED = 4,
        SMOOTH_MARCH_NARROW = 5 };
 static_assert(SMOOTH_MARCH == CGDIR_SMOOTH_MARCH && SMOOTH_TILE == CGDIR_SMOOTH_TILE &&
                   SMOOTH_SPLIT == CGDIR_SMOOTH_SPLIT && SMOOTH_FUSED == CGDIR_SMOOTH_FUSED &&
                   SMOOTH_MARCH_NARROW == CGDIR_SMOOTH_MARCH32,
               "internal smoothing variants are the public tuning codes");
-int smooth_auto_variant(int nx, int ny, int nz);
 // Kernel choice for one smoothing launch: variant and (z-march) z chunk, 0 = default.
 struct SmoothChoice {
     int variant = SMOOTH_AUTO;
     int zchunk = 0;
-    int ctas_per_sm = 0;          // at most this many wide z-march CTAs per SM (0: no cap)
+    int ctas_per_sm = 0;          // at most this many z-march CTAs per SM (0: no cap)
 };
-int smooth_default_zchunk(int nx, int ny, int nz, int ncomp);
+int smooth_default_zchunk(int nx, int ny, int nz, int ncomp, float sigma);
 // err: device word set to 1 if a bounded wait inside the kernel ran out;
 // nullptr selects the plain-load kernel (no waits).
 cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int ny, int nz,

@@ -4,21 +4,18 @@
 //
 // Smoothing: the 3-D Gaussian is applied as x, y and z passes (the
 // separability the paper uses) inside ONE kernel, so each component is read
-// once and written once.  A CTA owns a 32 x 8 column in x-y and marches
-// along z: every input plane of the column plus an R-voxel halo goes to
-// shared memory, the x pass and the y pass run there, and each thread keeps
-// the last 2R+1 xy-filtered values of its column in registers for the z
-// pass.  Halo indices are clamped (clamp-to-edge).  All three components of
-// a displacement field are filtered by the same CTA.
+// once and written once.  A CTA owns a column in x-y and marches along z:
+// every input plane of the column plus an R-voxel halo goes to shared memory,
+// the x pass and the y pass run there, and each thread keeps the last 2R+1
+// xy-filtered values of its outputs in registers for the z pass.  The borders
+// are clamped (clamp-to-edge).
 //
-// Two versions of the smoothing kernel share that structure.  The TMA one
-// (used whenever the field satisfies the tensor-map rules: nx a multiple of
-// 4, 16-byte aligned base) streams each input plane of the column into a
-// 4-stage shared-memory ring with cp.async.bulk.tensor, so the loads of the
-// next planes are in flight while the current one is filtered; clamping at
-// the volume border is done by index remapping in the x and y passes (the
-// TMA box itself zero-fills outside the volume).  The plain one loads the
-// halo with ordinary clamped loads.
+// Where the field satisfies the tensor-map rules (nx a multiple of 4, 16-byte
+// aligned base) the planes come by cp.async.bulk.tensor, otherwise by
+// cp.async with clamped indices, into a ring of shared-memory stages, so the
+// loads of the next planes are in flight while the current one is filtered.
+// The plain kernel family (no waits inside kernels) loads the halo with
+// ordinary clamped loads.
 //
 // Every kernel here returns at once when the level's stop flag is set, so a
 // level that converged early leaves its fields untouched.
@@ -121,28 +118,26 @@ __global__ void __launch_bounds__(NT) k_smooth(const float *__restrict__ in,
     }
 }
 
-// ---- TMA-fed version ---------------------------------------------------
-// A CTA (32 x 8 threads) filters NC components (NC = 1: one component per
-// CTA; NC = 3: the three components of a DVF, needed by the composite-update
-// epilogue) of a 32 x 16 column; each thread owns two adjacent output rows.
-// Per input plane one TMA box (x from x0 - ML, ML = R rounded up to 4 so the
-// start is 16-byte aligned; y from y0 - R) lands in a 4-stage ring.
-// x pass: each task filters 4 adjacent outputs of one row from 16-byte
-// shared loads; y pass: two rows from 2R+2 loads; z pass: a (2R+1)-deep
-// register ring whose slots are fixed at compile time by unrolling the
-// plane loop 2R+1 times.  One barrier per plane.
-//
-// COMPOSE (NC = 3): the z-pass result is the smoothed du at (x, y, z); the
+// ---- one-pass G(du) + composite update (the fused kernel family) ----------
+// A CTA (32 x 8 threads) filters the three components of a DVF over a 32 x 16
+// column; each thread owns two adjacent output rows.  Per input plane one TMA
+// box (x from x0 - ML, ML = R rounded up to 4 so the start is 16-byte
+// aligned; y from y0 - R) lands in a 6-stage ring.  x pass: each task
+// filters 4 adjacent outputs of one row from 16-byte shared loads; y pass:
+// two rows from 2R+2 loads; z pass: a (2R+1)-deep register ring whose slots
+// are fixed at compile time by unrolling the plane loop 2R+1 times.  One
+// barrier per plane.  The z-pass result is the smoothed du at (x, y, z); the
 // epilogue applies Algorithm A step 3 there, u_new = du + u(x + du), so the
 // smoothed du never goes back to memory.
 constexpr int SY = 16;                 // output rows per CTA (2 per thread)
 
-template <int R, int NC>
+template <int R>
 struct SmoothGeom {
+    static constexpr int NC = 3;
     static constexpr int ML = (R + 3) / 4 * 4;
     static constexpr int BXW = TX + 2 * ML;
     static constexpr int BY = SY + 2 * R;
-    static constexpr int ST = NC == 1 ? 8 : 6;                      // pipeline stages
+    static constexpr int ST = 6;                                    // pipeline stages
     static constexpr int STAGE = (NC * BY * BXW + 31) / 32 * 32;   // floats per stage
     static constexpr int NV = (4 + R + ML + 3) / 4;                // float4 per x task
     static constexpr int XB = NC * BY * TX;                          // floats per X buffer
@@ -164,14 +159,14 @@ __device__ __forceinline__ float trilinear_at(const float *__restrict__ f, size_
     return fmaf(wz, f1 - f0, f0);
 }
 
-template <int R, int NC, bool COMPOSE>
-__global__ void __launch_bounds__(NT) k_smooth_tma(const __grid_constant__ CUtensorMap tin,
-                                                   const float *__restrict__ ucomp, int mode,
-                                                   float *__restrict__ out, int ncomp, Taps taps,
-                                                   int nx, int ny, int nz, int zchunk,
-                                                   const int *stop_flag, int *err) {
+template <int R>
+__global__ void __launch_bounds__(NT) k_smooth_compose_tma(const __grid_constant__ CUtensorMap tin,
+                                                           const float *__restrict__ ucomp, int mode,
+                                                           float *__restrict__ out, Taps taps, int nx, int ny,
+                                                           int nz, int zchunk, const int *stop_flag, int *err) {
     if (stop_flag && *stop_flag) return;
-    using G = SmoothGeom<R, NC>;
+    using G = SmoothGeom<R>;
+    constexpr int NC = G::NC;
     constexpr int BY = G::BY, BXW = G::BXW, ML = G::ML, STAGE = G::STAGE, NV = G::NV, K = 2 * R + 1;
     constexpr int ST = G::ST, TPT = G::TPT;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -183,16 +178,12 @@ __global__ void __launch_bounds__(NT) k_smooth_tma(const __grid_constant__ CUten
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
     const size_t N = (size_t)nx * ny * nz, nxy = (size_t)nx * ny;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * SY;
-    const int nchunks = (nz + zchunk - 1) / zchunk;
-    const int chunk = (int)blockIdx.z % nchunks;
-    const int comp = NC == 1 ? (int)blockIdx.z / nchunks : 0;      // component of an NC=1 CTA
-    const int zb = chunk * zchunk, ze = min(zb + zchunk, nz);
+    const int zb = (int)blockIdx.z * zchunk, ze = min(zb + zchunk, nz);
     const int P = (ze - zb) + 2 * R;
     const int x = x0 + tx, ya = y0 + 2 * ty;                        // rows ya, ya + 1
     const bool acta = x < nx && ya < ny, actb = x < nx && ya + 1 < ny;
     const bool xin = (x0 - R >= 0) && (x0 + TX + R <= nx);
     const uint32_t tx_bytes = (uint32_t)(NC * BY * BXW * sizeof(float));
-    (void)ncomp;
 
     float2 w2[K];
 #pragma unroll
@@ -210,7 +201,7 @@ __global__ void __launch_bounds__(NT) k_smooth_tma(const __grid_constant__ CUten
     for (int q = 0; q < TPT; ++q) {
         const int task = tid + q * NT;
         const int g = task & (TX / 4 - 1), row = task >> 3;         // row = c * BY + hy
-        const int c = NC == 1 ? 0 : row / BY, hy = row - c * BY;
+        const int c = row / BY, hy = row - c * BY;
         const int ly = clampi(y0 - R + hy, 0, ny - 1) - (y0 - R);
         t_row[q] = task < G::NTASK ? (c * BY + ly) * BXW : -1;
         t_g4[q] = 4 * g;
@@ -219,13 +210,13 @@ __global__ void __launch_bounds__(NT) k_smooth_tma(const __grid_constant__ CUten
     const int xlim = nx - x0 + ML;        // first local column beyond the volume's last x
     float *outp[NC];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) outp[c] = out + (size_t)(comp + c) * N + (size_t)ya * nx + x;
+    for (int c = 0; c < NC; ++c) outp[c] = out + (size_t)c * N + (size_t)ya * nx + x;
 
     auto issue = [&](int q) {
         const int sidx = q % ST;
         const int z = clampi(zb - R + q, 0, nz - 1);
         mbar_expect_tx(&bar[sidx], tx_bytes);
-        tma_load_4d(stage + sidx * STAGE, &tin, x0 - ML, y0 - R, z, comp, &bar[sidx]);
+        tma_load_4d(stage + sidx * STAGE, &tin, x0 - ML, y0 - R, z, 0, &bar[sidx]);
     };
     if (tid == 0) {
         for (int q = 0; q < ST; ++q) mbar_init(&bar[q], 1);
@@ -328,30 +319,24 @@ __global__ void __launch_bounds__(NT) k_smooth_tma(const __grid_constant__ CUten
                 for (int h = 0; h < 2; ++h) {
                     if (!(h == 0 ? acta : actb)) continue;
                     const size_t off = zoff + (size_t)h * nx;
-                    if (COMPOSE) {
-                        const int y = ya + h;
-                        const size_t i = off + (size_t)ya * nx + x;
-                        const float dx = h ? res[0].y : res[0].x;
-                        const float dy = NC > 1 ? (h ? res[NC > 1 ? 1 : 0].y : res[NC > 1 ? 1 : 0].x) : 0.f;
-                        const float dz = NC > 2 ? (h ? res[NC > 2 ? 2 : 0].y : res[NC > 2 ? 2 : 0].x) : 0.f;
-                        float ax, ay, az;
-                        if (mode == CGDIR_ADDITIVE) {
-                            ax = __ldg(ucomp + i); ay = __ldg(ucomp + N + i); az = __ldg(ucomp + 2 * N + i);
-                        } else {
-                            const Corners cc = corners((float)x + dx, (float)y + dy, (float)zo + dz, nx, ny, nz);
-                            const int ddx = cc.x1 - cc.x0, ddy = (cc.y1 - cc.y0) * nx, ddz = (cc.z1 - cc.z0) * nx * ny;
-                            const size_t b0 = ((size_t)cc.z0 * ny + cc.y0) * nx + cc.x0;
-                            ax = trilinear_at(ucomp, b0, ddx, ddy, ddz, cc.wx, cc.wy, cc.wz);
-                            ay = trilinear_at(ucomp + N, b0, ddx, ddy, ddz, cc.wx, cc.wy, cc.wz);
-                            az = trilinear_at(ucomp + 2 * N, b0, ddx, ddy, ddz, cc.wx, cc.wy, cc.wz);
-                        }
-                        outp[0][off] = dx + ax;
-                        outp[0][N + off] = dy + ay;
-                        outp[0][2 * N + off] = dz + az;
+                    const int y = ya + h;
+                    const size_t i = off + (size_t)ya * nx + x;
+                    const float dx = h ? res[0].y : res[0].x, dy = h ? res[1].y : res[1].x,
+                                dz = h ? res[2].y : res[2].x;
+                    float ax, ay, az;
+                    if (mode == CGDIR_ADDITIVE) {
+                        ax = __ldg(ucomp + i); ay = __ldg(ucomp + N + i); az = __ldg(ucomp + 2 * N + i);
                     } else {
-#pragma unroll
-                        for (int c = 0; c < NC; ++c) outp[c][off] = h ? res[c].y : res[c].x;
+                        const Corners cc = corners((float)x + dx, (float)y + dy, (float)zo + dz, nx, ny, nz);
+                        const int ddx = cc.x1 - cc.x0, ddy = (cc.y1 - cc.y0) * nx, ddz = (cc.z1 - cc.z0) * nx * ny;
+                        const size_t b0 = ((size_t)cc.z0 * ny + cc.y0) * nx + cc.x0;
+                        ax = trilinear_at(ucomp, b0, ddx, ddy, ddz, cc.wx, cc.wy, cc.wz);
+                        ay = trilinear_at(ucomp + N, b0, ddx, ddy, ddz, cc.wx, cc.wy, cc.wz);
+                        az = trilinear_at(ucomp + 2 * N, b0, ddx, ddy, ddz, cc.wx, cc.wy, cc.wz);
                     }
+                    outp[0][off] = dx + ax;
+                    outp[0][N + off] = dy + ay;
+                    outp[0][2 * N + off] = dz + az;
                 }
             }
         }
@@ -367,216 +352,280 @@ __global__ void __launch_bounds__(NT) k_smooth_tma(const __grid_constant__ CUten
     }
 }
 
-// ---- wide-tile z-march (one component per CTA, nx % 8 == 0, R <= 4) -----
-// The same passes and the same order of operations as k_smooth_tma (so the
-// same bits), on a 64 x 16 output tile with less work per output:
-//  * per input plane one TMA box (x from x0 - 4, 72 wide; y from y0 - R)
-//    lands in a ring of stages; the ring and the x-pass buffers are indexed
-//    from the kernel's own shared array, so every access is a shared-memory
-//    load or store;
-//  * x pass: a task is 8 adjacent outputs of one box row (four 16-byte
-//    loads, 56 FMAs, half of them paired); the clamp at the volume's x
-//    borders is a select on the loaded values (the box is zero-filled
-//    there), the clamp in y a remapped row, in z a clamped plane;
-//  * y pass: a thread takes a column pair and two rows: 8-byte loads of the
-//    pair, paired FMAs only;
-//  * z pass: the last 2R+1 y-pass results of those four outputs stay in
+// ---- z-march (one component per CTA) ---------------------------------------
+// A CTA of 128 threads filters a 32-wide, 8 RY-high column of one component
+// and marches along z, one barrier per plane:
+//  * the input plane of the column plus its halo lands in a ring of ST
+//    stages: one TMA box (x from x0 - ML, ML = R rounded up to 4 so that the
+//    start is 16-byte aligned; y from y0 - R), or, where no tensor map is
+//    possible (nx % 4 != 0, a misaligned field), 4-byte cp.async copies with
+//    clamped indices that arrive on the same mbarrier;
+//  * x pass: a task is 8 adjacent outputs of one box row (16-byte loads,
+//    56 FMAs at R = 3, the register-aligned half of them paired); the clamp
+//    at the volume's x borders is a select on the loaded values taken by the
+//    CTAs there (the TMA box is zero-filled outside), the clamp in y a
+//    remapped row, in z a clamped plane;
+//  * y pass: a thread takes a column pair and RY rows: 2R + RY 8-byte loads
+//    of the pair, paired FMAs only;
+//  * z pass: the last 2R + 1 y-pass results of those 2 RY outputs stay in
 //    registers (slots fixed at compile time by unrolling the plane loop
-//    2R+1 times), paired FMAs; 8-byte stores.
-// One barrier per PB planes (PB x-pass buffers, double-buffered); the
-// launcher takes PB = 1 (two to four planes per barrier measured slower:
-// 262-332 against 218 us at 512 x 512 x 160).  The plane count of a step is
-// the runtime min(PB, planes left) even for PB = 1: written with a
-// compile-time 1 instead (same bits), the kernel took 265 us.
-// Box rows are 76 floats wide (x0 - 4 .. x0 + 71; the last 4 columns are
-// not used) and so are the x-pass buffer's rows: 19 16-byte units, so the
-// x-pass tasks below (task q: box row q % BY, column group q / BY) hit
-// distinct bank groups in every quarter-warp, for their 16-byte loads and
-// stores alike (unit 19 row + 2 group = 3 q mod 8 when BY = 6 mod 8).
-constexpr int WX = 64, WY = 16, WML = 4, WBX = 76;
-
-template <int R>
-struct WideGeom {
-    static constexpr int BY = WY + 2 * R;                       // box rows
-    static constexpr int ST = 8;                                // pipeline stages
-    static constexpr int STAGE = (BY * WBX + 31) / 32 * 32;     // floats per stage (128-byte multiple)
-    static constexpr int XB = BY * WBX;                         // floats per x-pass buffer
-    static constexpr int NTASK = BY * (WX / 8);                 // x-pass tasks per plane
-    static constexpr size_t bytes(int pb) {
-        return sizeof(float) * ((size_t)ST * STAGE + 2 * (size_t)pb * XB) + ST * sizeof(uint64_t) + 128;
+//    2R + 1 times), paired FMAs, one 8-byte store per row.
+// The taps are symmetric, so R + 1 pairs of them are held.  Box rows and
+// x-pass rows are an odd number of 16-byte units wide and consecutive tasks
+// take consecutive rows, so the 16-byte accesses of every quarter-warp fall
+// in distinct bank groups.
+//
+// Bound by shared-memory bandwidth, issue and the per-plane chain together
+// (512x512x160, sigma 1: DRAM 69 %, shared memory 65 %, issue 0.61), so the
+// tile is chosen to cut all three: four rows per thread need 10 instead of 16
+// loads in the y pass per 8 outputs and a 38 / 32 instead of 22 / 16 x-pass
+// halo (28 instead of 38 thread instructions per output), and five small CTAs
+// per SM (94 registers, 40 KB of shared memory) have five independent
+// barriers to wait at.  Per three-component field, against the 64 x 16 tile
+// with two rows per thread and 256 threads that it replaces (z chunks each
+// side's best): 512x512x160 215 -> 172 us, 256x256x96 43 -> 33, 240x160x70
+// 24.6 -> 20.5.  Also measured at 512x512x160: 64 x 32 tiles of 256 threads 183 us
+// (2 CTAs per SM), 64 x 32 at 3 CTAs (80 registers, spills) 251, 32 x 24 172 but
+// slower at 256x256x96, 32 x 16 194, a fifth warp for the x pass 189, the x pass
+// one plane ahead of the y / z passes 189.
+// RY = 2 is the 32 x 16 tile: radii 5 and 6, whose z ring would not fit four
+// rows' registers, and the MARCH32 variant.
+constexpr int MT = 128;                // threads
+constexpr int MX = 32;                 // tile width
+template <int R, int RY>
+struct MarchGeom {
+    static constexpr int K = 2 * R + 1;
+    static constexpr int WY = 8 * RY, BY = WY + 2 * R;          // tile height, box rows
+    static constexpr int ML = (R + 3) / 4 * 4;                  // x margin of the box
+    static constexpr int W = MX + 2 * ML + 4;                   // box and x-pass row: 11 or 13 units of 16 bytes
+    static constexpr int ST = RY == 4 ? 4 : 6;                  // stages
+    static constexpr int STAGE = (BY * W + 31) / 32 * 32;       // floats per stage (128-byte multiple)
+    static constexpr int XB = BY * W;                           // floats per x-pass buffer
+    static constexpr int NTASK = BY * (MX / 8);                 // x-pass tasks per plane
+    static constexpr int TPT = (NTASK + MT - 1) / MT;
+    static constexpr int CTAS = RY == 4 ? (R <= 3 ? 5 : 4) : (R <= 4 ? 6 : 4);   // resident per SM (registers)
+    static constexpr size_t bytes() {
+        return sizeof(float) * ((size_t)ST * STAGE + 2 * (size_t)XB) + ST * sizeof(uint64_t) + 128;
     }
+    static_assert(W / 4 % 2 == 1, "odd number of 16-byte units per row");
 };
 
-template <int R, int PB>
-__global__ void __launch_bounds__(NT, 2) k_smooth_wide(const __grid_constant__ CUtensorMap tin,
-                                                       float *__restrict__ out, Taps taps, int nx, int ny,
-                                                       int nz, int zchunk, const int *stop_flag, int *err) {
+template <int R, int RY, bool ASYNC>
+__global__ void __launch_bounds__(MT, RY == 4 ? 4 : MarchGeom<R, RY>::CTAS)
+    k_smooth_march(const __grid_constant__ CUtensorMap tin, const float *__restrict__ in, float *__restrict__ out,
+                   Taps taps, int nx, int ny, int nz, int zchunk, const int *stop_flag, int *err) {
     if (stop_flag && *stop_flag) return;
-    using G = WideGeom<R>;
-    constexpr int K = 2 * R + 1, BY = G::BY, ST = G::ST, STAGE = G::STAGE, XB = G::XB;
-    static_assert(R >= 1 && R <= 4, "8-output x tasks read 16 loaded values");
-    static_assert(PB >= 1 && PB <= 4, "planes per barrier");
+    using G = MarchGeom<R, RY>;
+    constexpr int K = G::K, BY = G::BY, ML = G::ML, W = G::W, ST = G::ST, STAGE = G::STAGE, XB = G::XB, TPT = G::TPT;
+    constexpr int NV = 8 + 2 * ML;                               // loaded values of an x task
     extern __shared__ __align__(128) float wsm[];
     // 128-byte aligned base for the TMA stages, still a shared-memory pointer
     const int pad = (int)(((128u - (smem_u32(wsm) & 127u)) & 127u) >> 2);
     float *stage0 = wsm + pad;                                   // [ST][STAGE]
-    float *xbuf = stage0 + ST * STAGE;                           // [2][PB][BY][WBX]
-    uint64_t *bar = reinterpret_cast<uint64_t *>(xbuf + 2 * PB * XB);
+    float *xbuf = stage0 + ST * STAGE;                           // [2][BY][W]
+    uint64_t *bar = reinterpret_cast<uint64_t *>(xbuf + 2 * XB);
 
-    const int tid = threadIdx.y * TX + threadIdx.x;
-    const int x0 = blockIdx.x * WX, y0 = blockIdx.y * WY;
+    const int tid = threadIdx.x;
+    const int x0 = blockIdx.x * MX, y0 = blockIdx.y * G::WY;
     const int nchunks = (nz + zchunk - 1) / zchunk;
     const int chunk = (int)blockIdx.z % nchunks, comp = (int)blockIdx.z / nchunks;
     const int zb = chunk * zchunk, ze = min(zb + zchunk, nz);
     const int P = (ze - zb) + 2 * R;
-    const uint32_t tx_bytes = (uint32_t)(BY * WBX * sizeof(float));
-
-    float2 w2[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) w2[j] = make_float2(taps.w[j], taps.w[j]);
-
-    // x-pass task of this thread (fixed for every plane): box row and column group
-    const bool xtask = tid < G::NTASK;
-    const int xrow = tid % BY, xg = tid / BY;
-    const int srow = clampi(y0 - R + xrow, 0, ny - 1) - (y0 - R);    // clamped source row in the box
-    const int xsrc = srow * WBX + 8 * xg;                            // first loaded float
-    const int xdst = xrow * WBX + 8 * xg;
-    const bool pleft = x0 == 0 && xg == 0;                            // taps left of x = 0
-    const bool pright = x0 + 8 * xg + 8 == nx;                        // taps right of x = nx - 1
-    const bool xedge = x0 == 0 || x0 + WX >= nx;                      // the same for the whole CTA
-    // y / z pass: column pair (x, x + 1) and rows (y, y + 1) of this thread
-    const int yc = 2 * (tid & 31), yr = 2 * (tid >> 5);
-    const int gx = x0 + yc, gy = y0 + yr;
-    const bool act0 = gx < nx && gy < ny, act1 = gx < nx && gy + 1 < ny;
     const size_t nxy = (size_t)nx * ny;
+
+    float2 w2[R + 1];
+#pragma unroll
+    for (int j = 0; j <= R; ++j) w2[j] = make_float2(taps.w[j], taps.w[j]);
+    auto tap = [&](int j) { return w2[j <= R ? j : 2 * R - j]; };
+
+    // x-pass tasks of this thread (fixed for every plane)
+    int xsrc[TPT], xdst[TPT];
+    bool xt[TPT];
+#pragma unroll
+    for (int q = 0; q < TPT; ++q) {
+        const int task = tid + q * MT, row = task % BY, g = task / BY;
+        xt[q] = task < G::NTASK;
+        // the clamped source row (the asynchronous copies are clamped themselves)
+        const int srow = ASYNC ? row : clampi(y0 - R + row, 0, ny - 1) - (y0 - R);
+        xsrc[q] = srow * W + 8 * g;
+        xdst[q] = row * W + 8 * g;
+    }
+    const bool xedge = !ASYNC && (x0 == 0 || x0 + MX + R > nx); // the same for the whole CTA
+    // y / z pass: column pair and RY rows of this thread
+    const int yc = 2 * (tid % (MX / 2)), yr = RY * (tid / (MX / 2));
+    const int gx = x0 + yc, gy = y0 + yr;
+    const int nact = gx < nx ? min(max(ny - gy, 0), RY) : 0;     // rows inside the volume
     float *optr = out + (size_t)comp * nxy * nz + (size_t)zb * nxy + (size_t)gy * nx + gx;
 
-    auto issue = [&](int q) {
-        const int sidx = q % ST;
+    // issue the loads of plane q into the stage at offset so, completing on b
+    // (one thread; with ASYNC every thread)
+    auto issue = [&](int q, int so, uint64_t *b) {
         const int z = clampi(zb - R + q, 0, nz - 1);
-        mbar_expect_tx(&bar[sidx], tx_bytes);
-        tma_load_4d(stage0 + sidx * STAGE, &tin, x0 - WML, y0 - R, z, comp, &bar[sidx]);
+        if (!ASYNC) {
+            mbar_expect_tx(b, (uint32_t)(BY * W * sizeof(float)));
+            tma_load_4d(stage0 + so, &tin, x0 - ML, y0 - R, z, comp, b);
+            return;
+        }
+        // warp w takes rows w, w + 4, ...: lane l the columns l and, for the
+        // 2R further ones, 32 + l
+        const int lane = tid & 31, r0 = tid >> 5;
+        const float *src = in + (size_t)comp * nxy * nz + (size_t)z * nxy;
+        const int ca = clampi(x0 - R + lane, 0, nx - 1), cb = clampi(x0 - R + MX + lane, 0, nx - 1);
+        const uint32_t d0 = smem_u32(stage0 + so + r0 * W + ML - R + lane);
+        if (y0 >= R && y0 + G::WY + R <= ny) {
+            const float *pa = src + (size_t)(y0 - R + r0) * nx;
+            const size_t step = (size_t)4 * nx;
+#pragma unroll 5
+            for (int i = 0; i < (BY + 3) / 4; ++i, pa += step) {
+                if (4 * i + r0 >= BY) break;
+                cp_async4(d0 + i * 16 * W, pa + ca);
+                if (lane < 2 * R) cp_async4(d0 + i * 16 * W + 128, pa + cb);
+            }
+        } else {
+            for (int i = 0; 4 * i + r0 < BY; ++i) {
+                const float *pa = src + (size_t)clampi(y0 - R + r0 + 4 * i, 0, ny - 1) * nx;
+                cp_async4(d0 + i * 16 * W, pa + ca);
+                if (lane < 2 * R) cp_async4(d0 + i * 16 * W + 128, pa + cb);
+            }
+        }
+        cp_async_arrive(b);
     };
-    if (tid == 0) {
-        for (int q = 0; q < ST; ++q) mbar_init(&bar[q], 1);
+    // the issuing thread: the last one that waits for every plane itself
+    constexpr int kIssuer = (G::NTASK < MT ? G::NTASK : MT) - 1;
+    if (tid == kIssuer) {
+        for (int q = 0; q < ST; ++q) mbar_init(&bar[q], ASYNC ? MT : 1);
         fence_mbar_init();
     }
     __syncthreads();
-    if (tid == 0)
-        for (int q = 0; q < ST && q < P; ++q) issue(q);
+    if (ASYNC || tid == kIssuer)
+        for (int q = 0; q < ST && q < P; ++q) issue(q, q * STAGE, bar + q);
 
-    float2 ring[2][K];
+    float2 ring[RY][K];
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < RY; ++h)
 #pragma unroll
         for (int j = 0; j < K; ++j) ring[h][j] = make_float2(0.f, 0.f);
 
-    // x pass of the plane in stage sidx into x-pass buffer dst
-    auto xpass = [&](int sidx, float *dst) {
-        const float *src = stage0 + sidx * STAGE + xsrc;
-        float v[16];
+    // x pass of one task; xend: outputs of it inside the volume
+    auto xpass = [&](const float *src, float *d, bool left, int xend) {
+        float v[NV];
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
+        for (int h = 0; h < NV / 4; ++h) {
             const float4 f = *reinterpret_cast<const float4 *>(src + 4 * h);
             v[4 * h] = f.x; v[4 * h + 1] = f.y; v[4 * h + 2] = f.z; v[4 * h + 3] = f.w;
         }
-        if (xedge) {                   // CTAs at an x border of the volume only
+        if (xedge) {                   // CTAs at an x border of the volume only (nx % 4 == 0)
 #pragma unroll
-            for (int k = WML - R; k < WML; ++k) v[k] = pleft ? v[WML] : v[k];
+            for (int k = ML - R; k < ML; ++k) v[k] = left ? v[ML] : v[k];
 #pragma unroll
-            for (int k = 8 + WML; k < 8 + WML + R; ++k) v[k] = pright ? v[7 + WML] : v[k];
+            for (int k = 4 + ML; k < 8 + ML + R; ++k) v[k] = xend == 4 ? v[3 + ML] : v[k];
+#pragma unroll
+            for (int k = 8 + ML; k < 8 + ML + R; ++k) v[k] = xend == 8 ? v[7 + ML] : v[k];
+            if (ML > 4) {              // radii above 4 reach past the next group's first half
+#pragma unroll
+                for (int k = 12 + ML; k < 8 + ML + R; ++k) v[k] = xend == 12 ? v[11 + ML] : v[k];
+            }
         }
         float2 o[4];
 #pragma unroll
         for (int m = 0; m < 4; ++m) o[m] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            constexpr int B = WML - R;
+            constexpr int B = ML - R;
             if ((B + j) % 2 == 0) {            // operand pairs register-aligned
 #pragma unroll
                 for (int m = 0; m < 4; ++m)
-                    o[m] = __ffma2_rn(w2[j], make_float2(v[B + j + 2 * m], v[B + j + 2 * m + 1]), o[m]);
-            } else {
+                    o[m] = __ffma2_rn(tap(j), make_float2(v[B + j + 2 * m], v[B + j + 2 * m + 1]), o[m]);
+            } else {                           // odd offset: scalar FMAs (same rounding, no moves)
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    o[m].x = fmaf(w2[j].x, v[B + j + 2 * m], o[m].x);
-                    o[m].y = fmaf(w2[j].x, v[B + j + 2 * m + 1], o[m].y);
+                    o[m].x = fmaf(tap(j).x, v[B + j + 2 * m], o[m].x);
+                    o[m].y = fmaf(tap(j).x, v[B + j + 2 * m + 1], o[m].y);
                 }
             }
         }
-        float *d = dst + xdst;
         *reinterpret_cast<float4 *>(d) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
         *reinterpret_cast<float4 *>(d + 4) = make_float4(o[2].x, o[2].y, o[3].x, o[3].y);
     };
 
-    int tw = -1;                        // plane whose wait ran out (-1: none)
-    int sidx = 0, xo = 0;               // stage of plane t, x-pass buffer offset
-    uint32_t par = 0;                   // phase parity of that stage
-    for (int t0 = 0; t0 < P && tw < 0; t0 += PB * K) {
+    // tw: the plane whose wait ran out in this thread (-1: none); it skips the
+    // later waits, and the CTA leaves at the next turn of the plane loop,
+    // where its threads agree on it
+    int tw = -1;
+    bool leave = false;
+    uint32_t par = 0;                   // phase parity of the current stage
+    int so = 0, xo = 0;                 // offsets of the current stage and x-pass buffer
+    uint64_t *bcur = bar;
+    int t0 = 0;
+    for (; t0 < P; t0 += K) {
 #pragma unroll
-        for (int rr = 0; rr < PB * K; rr += PB) {
-            const int t = t0 + rr;
+        for (int r = 0; r < K; ++r) {
+            const int t = t0 + r;
             if (t >= P) break;
-            const int np = min(PB, P - t);                // planes this step (the same for every thread)
-            bool ok = true;
-            if (xtask) {
-                int si = sidx;
-                uint32_t pa = par;
+            if (xt[0] && tw < 0 && !mbar_wait_bounded(bcur, par)) tw = t;
 #pragma unroll
-                for (int e = 0; e < PB; ++e) {
-                    if (e >= np) break;
-                    ok = ok && mbar_wait_bounded(&bar[si], pa);
-                    xpass(si, xbuf + xo + e * XB);
-                    if (++si == ST) { si = 0; pa ^= 1u; }
+            for (int q = 0; q < TPT; ++q) {
+                const int xg = xdst[q] % W;
+                if (xt[q]) xpass(stage0 + so + xsrc[q], xbuf + xo + xdst[q], x0 == 0 && xg == 0, nx - x0 - xg);
+            }
+            if (r == 0) {
+                if (__syncthreads_or(tw >= 0)) { leave = true; break; }
+            } else {
+                __syncthreads();
+            }
+            if (t + ST < P) {           // the stage just consumed takes plane t + ST
+                if (ASYNC) {
+                    issue(t + ST, so, bcur);
+                } else if (tid == kIssuer && tw < 0) {
+                    fence_proxy_async();
+                    issue(t + ST, so, bcur);
                 }
             }
-            if (__syncthreads_or(!ok)) { tw = t; break; }
-            if (tid == 0) {                    // the stages just consumed take planes t + e + ST
-                fence_proxy_async();
-                for (int e = 0; e < np; ++e)
-                    if (t + e + ST < P) issue(t + e + ST);
+            so += STAGE; ++bcur;
+            if (so == ST * STAGE) { so = 0; bcur = bar; par ^= 1u; }
+            // y pass into the plane's ring slot, z pass for plane t - 2R
+            const float *col = xbuf + xo + yr * W + yc;
+            float2 yin[2 * R + RY];
+#pragma unroll
+            for (int j = 0; j < 2 * R + RY; ++j) yin[j] = *reinterpret_cast<const float2 *>(col + j * W);
+#pragma unroll
+            for (int h = 0; h < RY; ++h) {
+                float2 a = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int j = 0; j < K; ++j) a = __ffma2_rn(tap(j), yin[h + j], a);
+                ring[h][r] = a;
             }
-            for (int e = 0; e < np; ++e)
-                if (++sidx == ST) { sidx = 0; par ^= 1u; }
-            // y pass into the planes' ring slots, z pass for planes t + e - 2R
+            if (t >= 2 * R) {
 #pragma unroll
-            for (int e = 0; e < PB; ++e) {
-                if (e >= np) break;
-                const int te = t + e, re = (rr + e) % K;
-                const float *col = xbuf + xo + e * XB + yr * WBX + yc;
-                float2 yin[K + 1];
+                for (int h = 0; h < RY; ++h) {
+                    float2 o = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int j = 0; j <= K; ++j) yin[j] = *reinterpret_cast<const float2 *>(col + j * WBX);
-                float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int j = 0; j < K; ++j) {
-                    a0 = __ffma2_rn(w2[j], yin[j], a0);
-                    a1 = __ffma2_rn(w2[j], yin[j + 1], a1);
-                }
-                ring[0][re] = a0;
-                ring[1][re] = a1;
-                if (te >= 2 * R) {
-                    float2 o0 = make_float2(0.f, 0.f), o1 = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int j = 0; j < K; ++j) {
-                        o0 = __ffma2_rn(w2[j], ring[0][(re + 1 + j) % K], o0);
-                        o1 = __ffma2_rn(w2[j], ring[1][(re + 1 + j) % K], o1);
+                    for (int j = 0; j < K; ++j) o = __ffma2_rn(tap(j), ring[h][(r + 1 + j) % K], o);
+                    if (h < nact) {
+                        float *d = optr + (size_t)h * nx;
+                        if (ASYNC) {              // odd rows are not 8-byte aligned
+                            d[0] = o.x;
+                            if (gx + 1 < nx) d[1] = o.y;
+                        } else {
+                            *reinterpret_cast<float2 *>(d) = o;
+                        }
                     }
-                    if (act0) *reinterpret_cast<float2 *>(optr) = o0;
-                    if (act1) *reinterpret_cast<float2 *>(optr + nx) = o1;
-                    optr += nxy;
                 }
+                optr += nxy;
             }
-            xo ^= PB * XB;
+            xo ^= XB;
         }
+        if (leave) break;
     }
-    if (tw >= 0) {
-        // a wait ran out: record it, drain the loads still in flight (planes
-        // tw .. tw + ST + PB - 2 were issued at most; bounded waits), leave
-        if (tid == 0) {
+    if (leave) {
+        // record it, let the loads in flight land (bounded waits), leave
+        if (ASYNC) {
+            cp_async_wait_all();
+            if (tid == 0) atomicExch(err, 1);
+        } else if (tid == kIssuer) {
             atomicExch(err, 1);
-            for (int q = tw; q < min(tw + ST + PB - 1, P); ++q)
-                mbar_wait_bounded(&bar[q % ST], (uint32_t)((q / ST) & 1));
+            const int q0 = tw >= 0 ? tw : t0 + 1, q1 = min((tw >= 0 ? tw : t0) + ST, P);
+            for (int q = q0; q < q1; ++q) mbar_wait_bounded(&bar[q % ST], (uint32_t)((q / ST) & 1));
         }
         __syncthreads();
     }
@@ -955,12 +1004,6 @@ __global__ void k_copy(const float *__restrict__ in, float *__restrict__ out, si
         out[i] = in[i];
 }
 
-// z chunk of the smoothing kernels: about two waves of resident CTAs (4 per
-// SM for one component per CTA, 2 for the three-component compose variant).
-int smooth_zchunk(int nx, int ny, int nz, int rows, int comp_ctas, int resident) {
-    return pick_zchunk(nz, (long)((nx + TX - 1) / TX) * ((ny + rows - 1) / rows) * comp_ctas, resident, 2);
-}
-
 unsigned flat_grid(size_t n) {
     size_t g = (n + 255) / 256;
     if (g > 152 * 16) g = 152 * 16;
@@ -969,87 +1012,109 @@ unsigned flat_grid(size_t n) {
 
 }  // namespace
 
-template <int R, int NC, bool COMPOSE>
-static cudaError_t smooth_tma_r(const float *in, const float *ucomp, int mode, float *out, int ncomp,
-                                const Taps &t, int nx, int ny, int nz, const int *stop_flag, int *err,
-                                cudaStream_t s, bool *launched, int zc_override) {
-    using G = SmoothGeom<R, NC>;
-    CUtensorMap m;
-    const uint64_t dims[4] = {(uint64_t)nx, (uint64_t)ny, (uint64_t)nz, (uint64_t)ncomp};
-    const uint32_t box[4] = {(uint32_t)G::BXW, (uint32_t)G::BY, 1u, (uint32_t)NC};
-    *launched = false;
-    if (!encode_tensor_map(&m, in, 4, dims, box, 4)) return cudaSuccess;
-    const int zc = zc_override > 0 ? std::min(zc_override, nz)
-                                   : smooth_zchunk(nx, ny, nz, SY, NC == 1 ? ncomp : 1, NC == 1 ? 4 : 2);
-    const int nchunks = (nz + zc - 1) / zc;
-    dim3 grid((nx + TX - 1) / TX, (ny + SY - 1) / SY, nchunks * (NC == 1 ? ncomp : 1)), block(TX, TY);
-    const size_t smem = G::bytes();
-    cudaError_t e = ensure_smem((const void *)k_smooth_tma<R, NC, COMPOSE>, smem);
-    if (e != cudaSuccess) return e;
-    k_smooth_tma<R, NC, COMPOSE><<<grid, block, smem, s>>>(m, ucomp, mode, out, ncomp, t, nx, ny, nz, zc,
-                                                          stop_flag, err);
-    *launched = true;
-    note_launch();
-    return cudaGetLastError();
-}
-
-// z chunk of the wide-tile z-march: about four waves of 3 resident CTAs per SM.
-static int wide_default_zchunk(int nx, int ny, int nz, int ncomp) {
-    return pick_zchunk(nz, (long)((nx + WX - 1) / WX) * ((ny + WY - 1) / WY) * ncomp, 3, 4);
-}
-
-// The wide-tile z-march for one component per CTA (nx % 8 == 0, R <= 4).
 template <int R>
-static cudaError_t smooth_wide_r(const float *in, float *out, int ncomp, const Taps &t, int nx, int ny, int nz,
-                                 const int *stop_flag, int *err, cudaStream_t s, bool *launched, int zc_override,
-                                 int cap) {
-    using G = WideGeom<R>;
+static cudaError_t smooth_compose_tma_r(const float *in, const float *ucomp, int mode, float *out, const Taps &t, int nx,
+                                        int ny, int nz, const int *stop_flag, int *err, cudaStream_t s,
+                                        bool *launched) {
+    using G = SmoothGeom<R>;
     CUtensorMap m;
-    const uint64_t dims[4] = {(uint64_t)nx, (uint64_t)ny, (uint64_t)nz, (uint64_t)ncomp};
-    const uint32_t box[4] = {(uint32_t)WBX, (uint32_t)G::BY, 1u, 1u};
+    const uint64_t dims[4] = {(uint64_t)nx, (uint64_t)ny, (uint64_t)nz, 3};
+    const uint32_t box[4] = {(uint32_t)G::BXW, (uint32_t)G::BY, 1u, 3u};
     *launched = false;
     if (!encode_tensor_map(&m, in, 4, dims, box, 4)) return cudaSuccess;
-    const int zc = zc_override > 0 ? std::min(zc_override, nz) : wide_default_zchunk(nx, ny, nz, ncomp);
-    const int nchunks = (nz + zc - 1) / zc;
-    dim3 grid((nx + WX - 1) / WX, (ny + WY - 1) / WY, nchunks * ncomp), block(TX, TY);
-    constexpr int PB = 1;       // planes per barrier: 2 to 4 measured slower (more x-pass buffers)
-    // a cap on CTAs per SM is a shared-memory request above 1/(cap+1) of the SM's 228 KB
-    const size_t smem = std::max(G::bytes(PB), cap > 0 ? (size_t)(228 << 10) / (cap + 1) + 1024 : (size_t)0);
-    cudaError_t e = ensure_smem((const void *)k_smooth_wide<R, PB>, smem);
+    const int zc = pick_zchunk(nz, (long)((nx + TX - 1) / TX) * ((ny + SY - 1) / SY), 2, 2);
+    dim3 grid((nx + TX - 1) / TX, (ny + SY - 1) / SY, (nz + zc - 1) / zc), block(TX, TY);
+    const size_t smem = G::bytes();
+    cudaError_t e = ensure_smem((const void *)k_smooth_compose_tma<R>, smem);
     if (e != cudaSuccess) return e;
-    k_smooth_wide<R, PB><<<grid, block, smem, s>>>(m, out, t, nx, ny, nz, zc, stop_flag, err);
+    k_smooth_compose_tma<R><<<grid, block, smem, s>>>(m, ucomp, mode, out, t, nx, ny, nz, zc, stop_flag, err);
     *launched = true;
     note_launch();
     return cudaGetLastError();
 }
 
-static cudaError_t smooth_wide(const float *in, float *out, int ncomp, const Taps &t, int nx, int ny, int nz,
-                               const int *stop_flag, int *err, cudaStream_t s, bool *launched, int zc = 0,
-                               int cap = 0) {
-    *launched = false;
-    if (nx % 8 != 0) return cudaSuccess;
+static cudaError_t smooth_compose_tma(const float *in, const float *ucomp, int mode, float *out, const Taps &t, int nx,
+                                      int ny, int nz, const int *stop_flag, int *err, cudaStream_t s,
+                                      bool *launched) {
     switch (t.r) {
-        case 1: return smooth_wide_r<1>(in, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc, cap);
-        case 2: return smooth_wide_r<2>(in, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc, cap);
-        case 3: return smooth_wide_r<3>(in, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc, cap);
-        case 4: return smooth_wide_r<4>(in, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc, cap);
-        default: return cudaSuccess;
-    }
-}
-
-template <int NC, bool COMPOSE>
-static cudaError_t smooth_tma(const float *in, const float *ucomp, int mode, float *out, int ncomp,
-                              const Taps &t, int nx, int ny, int nz, const int *stop_flag, int *err,
-                              cudaStream_t s, bool *launched, int zc = 0) {
-    switch (t.r) {
-        case 1: return smooth_tma_r<1, NC, COMPOSE>(in, ucomp, mode, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc);
-        case 2: return smooth_tma_r<2, NC, COMPOSE>(in, ucomp, mode, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc);
-        case 3: return smooth_tma_r<3, NC, COMPOSE>(in, ucomp, mode, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc);
-        case 4: return smooth_tma_r<4, NC, COMPOSE>(in, ucomp, mode, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc);
-        case 5: return smooth_tma_r<5, NC, COMPOSE>(in, ucomp, mode, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc);
-        case 6: return smooth_tma_r<6, NC, COMPOSE>(in, ucomp, mode, out, ncomp, t, nx, ny, nz, stop_flag, err, s, launched, zc);
+        case 1: return smooth_compose_tma_r<1>(in, ucomp, mode, out, t, nx, ny, nz, stop_flag, err, s, launched);
+        case 2: return smooth_compose_tma_r<2>(in, ucomp, mode, out, t, nx, ny, nz, stop_flag, err, s, launched);
+        case 3: return smooth_compose_tma_r<3>(in, ucomp, mode, out, t, nx, ny, nz, stop_flag, err, s, launched);
+        case 4: return smooth_compose_tma_r<4>(in, ucomp, mode, out, t, nx, ny, nz, stop_flag, err, s, launched);
+        case 5: return smooth_compose_tma_r<5>(in, ucomp, mode, out, t, nx, ny, nz, stop_flag, err, s, launched);
+        case 6: return smooth_compose_tma_r<6>(in, ucomp, mode, out, t, nx, ny, nz, stop_flag, err, s, launched);
         default: *launched = false; return cudaErrorInvalidValue;
     }
+}
+
+// z chunk of the z-march for `tiles` columns (all components) with `res`
+// CTAs resident per SM: the chunk count with the least estimated time.  A
+// CTA marches zc + 2r planes; a plane takes it 0.3 + 0.14 m (in units of a
+// full SM's plane) with m CTAs on its SM, fitted to 256x256x96 (192 columns,
+// 5 resident: 1, 2, 3, 4, 6, 8, 12 chunks estimated 59, 39, 33, 43, 38, 44, 47
+// us, measured 60, 39, 33, 41, 37, 41, 44); whole waves add up and the last one
+// counts with the CTAs it has.  At 512x512x160 it takes the measured best too
+// (4 chunks, 172 us; 1 chunk 230, 12 chunks 197).
+static int march_zchunk_r(int nz, long tiles, int res, int r) {
+    const long sms = sm_count(), wave = (long)res * sms;
+    auto plane = [](long m) { return 0.3 + 0.14 * (double)m; };
+    int best = nz;
+    double bt = 0.0;
+    for (int k = 1; k <= nz && k <= 128; ++k) {
+        const int zc = (nz + k - 1) / k;
+        const long n = tiles * ((nz + zc - 1) / zc), rem = n % wave;
+        const double t = (zc + 2 * r) * ((double)(n / wave) * plane(res) + (rem ? plane((rem + sms - 1) / sms) : 0.0));
+        if (k == 1 || t < bt) { bt = t; best = zc; }
+    }
+    return best;
+}
+
+template <int R, int RY>
+static cudaError_t smooth_march_r(const float *in, float *out, int ncomp, const Taps &t, int nx, int ny, int nz,
+                                  const int *stop_flag, int *err, cudaStream_t s, int zc_override, int cap) {
+    using G = MarchGeom<R, RY>;
+    const int tx = (nx + MX - 1) / MX, ty = (ny + G::WY - 1) / G::WY;
+    CUtensorMap m{};
+    const uint64_t dims[4] = {(uint64_t)nx, (uint64_t)ny, (uint64_t)nz, (uint64_t)ncomp};
+    const uint32_t box[4] = {(uint32_t)G::W, (uint32_t)G::BY, 1u, 1u};
+    const bool tma = nx % 4 == 0 && ((uintptr_t)out & 7) == 0 && encode_tensor_map(&m, in, 4, dims, box, 4);
+    const int full = tma ? G::CTAS : 4;      // the asynchronous-copy form holds more registers
+    const int res = cap > 0 ? std::min(cap, full) : full;
+    const int zc = zc_override > 0 ? std::min(zc_override, nz) : march_zchunk_r(nz, (long)tx * ty * ncomp, res, R);
+    const dim3 grid(tx, ty, (nz + zc - 1) / zc * ncomp);
+    // a cap on CTAs per SM is a shared-memory request above 1/(cap+1) of the SM's 228 KB
+    const size_t smem = std::max(G::bytes(), cap > 0 ? (size_t)(228 << 10) / (cap + 1) + 1024 : (size_t)0);
+    const void *f = tma ? (const void *)k_smooth_march<R, RY, false> : (const void *)k_smooth_march<R, RY, true>;
+    cudaError_t e = ensure_smem(f, smem);
+    if (e != cudaSuccess) return e;
+    if (tma)
+        k_smooth_march<R, RY, false><<<grid, MT, smem, s>>>(m, in, out, t, nx, ny, nz, zc, stop_flag, err);
+    else
+        k_smooth_march<R, RY, true><<<grid, MT, smem, s>>>(m, in, out, t, nx, ny, nz, zc, stop_flag, err);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// The z-march: 32 x 32 tiles for radii up to 4, else (and when `narrow`) 32 x 16.
+static cudaError_t smooth_march(const float *in, float *out, int ncomp, const Taps &t, int nx, int ny, int nz,
+                                bool narrow, const int *stop_flag, int *err, cudaStream_t s, int zc, int cap) {
+#define CGDIR_MARCH(R, RY) return smooth_march_r<R, RY>(in, out, ncomp, t, nx, ny, nz, stop_flag, err, s, zc, cap)
+    switch (t.r) {
+        case 1: if (narrow) CGDIR_MARCH(1, 2); else CGDIR_MARCH(1, 4);
+        case 2: if (narrow) CGDIR_MARCH(2, 2); else CGDIR_MARCH(2, 4);
+        case 3: if (narrow) CGDIR_MARCH(3, 2); else CGDIR_MARCH(3, 4);
+        case 4: if (narrow) CGDIR_MARCH(4, 2); else CGDIR_MARCH(4, 4);
+        case 5: CGDIR_MARCH(5, 2);
+        case 6: CGDIR_MARCH(6, 2);
+        default: return cudaErrorInvalidValue;
+    }
+#undef CGDIR_MARCH
+}
+
+int smooth_default_zchunk(int nx, int ny, int nz, int ncomp, float sigma) {
+    const int r = std::max(gauss_radius(sigma), 1), wy = r <= 4 ? 32 : 16;
+    const int res = r <= 3 ? 5 : 4;          // MarchGeom::CTAS
+    return march_zchunk_r(nz, (long)((nx + MX - 1) / MX) * ((ny + wy - 1) / wy) * ncomp, res, r);
 }
 
 template <int R>
@@ -1080,7 +1145,7 @@ static cudaError_t smooth_tile(const float *in, int ncomp, const Taps &t, int nx
 
 static cudaError_t smooth_plain(const float *in, int ncomp, const Taps &t, int nx, int ny, int nz,
                                 float *out, const int *stop_flag, cudaStream_t s) {
-    const int zc = smooth_zchunk(nx, ny, nz, TY, 1, 4);
+    const int zc = pick_zchunk(nz, (long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY), 4, 2);
     dim3 grid((nx + TX - 1) / TX, (ny + TY - 1) / TY, (nz + zc - 1) / zc), block(TX, TY);
     switch (t.r) {
         case 1: k_smooth<1><<<grid, block, 0, s>>>(in, out, ncomp, t, nx, ny, nz, zc, stop_flag); break;
@@ -1093,10 +1158,6 @@ static cudaError_t smooth_plain(const float *in, int ncomp, const Taps &t, int n
     }
     note_launch();
     return cudaGetLastError();
-}
-
-int smooth_auto_variant(int nx, int ny, int nz) {
-    return (size_t)nx * ny * nz < ((size_t)2 << 20) ? SMOOTH_TILE : SMOOTH_MARCH;
 }
 
 template <int R>
@@ -1137,11 +1198,6 @@ static cudaError_t smooth_split(const float *in, const float *u, int mode, bool 
     }
 }
 
-int smooth_default_zchunk(int nx, int ny, int nz, int ncomp) {
-    if (nx % 8 == 0) return wide_default_zchunk(nx, ny, nz, ncomp);
-    return smooth_zchunk(nx, ny, nz, SY, ncomp, 4);
-}
-
 cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int ny, int nz,
                           float *out, const int *stop_flag, cudaStream_t s, int *err, SmoothChoice ch, float *scratch) {
     int variant = ch.variant;
@@ -1153,22 +1209,12 @@ cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int n
         return cudaGetLastError();
     }
     if (err != nullptr) {
-        // small volumes: the 3-D tile kernel (one short wave); large: the
-        // TMA z-march, whose plane pipeline needs long chunks to pay off
-        if (variant == SMOOTH_AUTO) variant = smooth_auto_variant(nx, ny, nz);
         if (variant == SMOOTH_FUSED) variant = SMOOTH_TILE;     // nothing to fuse with here
         if (variant == SMOOTH_TILE) return smooth_tile(in, ncomp, t, nx, ny, nz, out, stop_flag, s);
         if (variant == SMOOTH_SPLIT && scratch != nullptr && scratch != in && scratch != out)
             return smooth_split(in, nullptr, 0, false, ncomp, t, nx, ny, nz, out, scratch, ch.zchunk, stop_flag, s);
-        bool launched = false;
-        if (variant != SMOOTH_MARCH_NARROW) {      // the wide-tile z-march where it applies
-            cudaError_t e = smooth_wide(in, out, ncomp, t, nx, ny, nz, stop_flag, err, s, &launched, ch.zchunk,
-                                        ch.ctas_per_sm);
-            if (e != cudaSuccess || launched) return e;
-        }
-        cudaError_t e =
-            smooth_tma<1, false>(in, nullptr, 0, out, ncomp, t, nx, ny, nz, stop_flag, err, s, &launched, ch.zchunk);
-        if (e != cudaSuccess || launched) return e;
+        return smooth_march(in, out, ncomp, t, nx, ny, nz, variant == SMOOTH_MARCH_NARROW, stop_flag, err, s, ch.zchunk,
+                            ch.ctas_per_sm);
     }
     return smooth_plain(in, ncomp, t, nx, ny, nz, out, stop_flag, s);
 }
@@ -1178,15 +1224,14 @@ cudaError_t launch_smooth_compose(const float *du, const float *u, int mode, flo
                                   int *err, bool one_pass, SmoothChoice ch) {
     const Taps t = gauss_taps(sigma);
     if (!one_pass && t.r > 0 && err != nullptr) {
-        int variant = ch.variant == SMOOTH_AUTO ? smooth_auto_variant(nx, ny, nz) : ch.variant;
-        if (variant == SMOOTH_SPLIT)   // x/y pass, then the z pass with the composite update fused
+        if (ch.variant == SMOOTH_SPLIT)   // x/y pass, then the z pass with the composite update fused
             return smooth_split(du, u, mode, true, 3, t, nx, ny, nz, out, tmp, ch.zchunk, stop_flag, s);
-        if (variant == SMOOTH_FUSED && (size_t)nx * ny * nz < (size_t)1 << 31)   // one 3-D tile kernel
+        if (ch.variant == SMOOTH_FUSED && (size_t)nx * ny * nz < (size_t)1 << 31)   // one 3-D tile kernel
             return launch_fused_smooth_compose(du, u, mode, sigma, nx, ny, nz, out, stop_flag, err, s);
     }
     if (one_pass && t.r > 0 && err != nullptr) {
         bool launched = false;
-        cudaError_t e = smooth_tma<3, true>(du, u, mode, out, 3, t, nx, ny, nz, stop_flag, err, s, &launched);
+        cudaError_t e = smooth_compose_tma(du, u, mode, out, t, nx, ny, nz, stop_flag, err, s, &launched);
         if (e != cudaSuccess || launched) return e;
     }
     // smooth du into tmp, then compose

@@ -105,7 +105,11 @@ struct cgdir_ctx {
     bool serve_priority = true;   // served requests' streams ranked by age (CGDIR_SERVE_PRIORITY=0: off)
     int serve_schedule = 2;       // served requests' schedule (CGDIR_SERVE_SCHEDULE=shared|alone|auto:
                                   // 0|1|2): auto takes the latency one when nothing else is running
-    int shared_wide_cap = 2;      // CGDIR_SHARED_WIDE_CAP=n: wide z-march CTAs per SM in batches (0: no cap)
+    // CGDIR_SHARED_WIDE_CAP=n: z-march CTAs per SM in batches (0: no cap).  4
+    // of the 5 that fit leave registers for the other registrations' kernels:
+    // six cases of uneven sizes, FP16 images, 100.2 ms uncapped, 83.9 / 86.6 /
+    // 92.2 / 114.8 ms at 4 / 3 / 2 / 1
+    int shared_wide_cap = 4;
     int force_width = 0;          // CGDIR_FORCE_WIDTH=1|2: force pass 2 voxels per thread (0: widest)
     int force_zchunk = 0;         // CGDIR_FORCE_ZCHUNK: force-pass z chunk for every level (0 = tuned / default)
     int smooth_zchunk = 0;        // CGDIR_SMOOTH_ZCHUNK: z-march smoothing z chunk (0 = tuned / default)

@@ -79,6 +79,17 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
         : "memory");
 }
 
+// 4-byte asynchronous copies (no alignment rule beyond 4 bytes): cp_async4
+// copies one float, cp_async_arrive lets the thread's copies so far arrive on
+// `bar` (counted as one arrival of its expected count).
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // ---- host side -------------------------------------------------------------
 // Encode a tiled tensor map of a dense x-fastest array with `rank` dims
 // (dims[0] = x extent) of `elem` bytes per element.  Returns false when the

@@ -58,5 +58,40 @@ def test_force_warp_pass(ctx, shape, kind):
         assert err <= 1e-5 * np.abs(img).max(), (contour, err)
 
 
+def smooth_ctx(variant):
+    import os
+    old = os.environ.get("CGDIR_SMOOTH")
+    os.environ["CGDIR_SMOOTH"] = variant
+    try:
+        return cg.Context(0)
+    finally:
+        if old is None:
+            del os.environ["CGDIR_SMOOTH"]
+        else:
+            os.environ["CGDIR_SMOOTH"] = old
+
+
+@pytest.mark.parametrize("sigma", [0.3, 0.6, 1.0, 1.3, 1.6, 2.0])      # radii 1 .. 6
+@pytest.mark.parametrize("shape", [(1, 1, 1), (3, 2, 4), (2, 33, 12), (9, 32, 32), (5, 65, 36), (17, 31, 64),
+                                   (40, 70, 100), (9, 34, 33), (23, 67, 45), (6, 5, 130)])
+def test_smooth_march_equals_tile_kernel(shape, sigma):
+    """The z-march (32 x 32 and 32 x 16 tiles; TMA where nx % 4 == 0, else
+    4-byte copies) has the tile kernel's order of operations, so the same
+    bits: partial tiles in every axis, volumes thinner than the filter, one
+    component and three, and a field that is not 16-byte aligned."""
+    rng = np.random.default_rng(hash_of(shape))
+    f = torch.from_numpy(rng.normal(0, 3, (3,) + shape).astype(np.float32)).to(DEV)
+    off = torch.empty(f.numel() + 1, device=DEV)[1:].view(f.shape)
+    off.copy_(f)
+    got = {}
+    for variant in ("tile", "march", "march32"):
+        with smooth_ctx(variant) as c:
+            got[variant] = [c.smooth(f, sigma), c.smooth(f[1].contiguous(), sigma), c.smooth(off, sigma)]
+            c.sync()
+    for variant in ("march", "march32"):
+        for a, b in zip(got["tile"], got[variant]):
+            assert torch.equal(a, b)
+
+
 def hash_of(shape):
     return shape[0] * 10007 + shape[1] * 101 + shape[2]
