@@ -242,11 +242,10 @@ cudaError_t launch_prolong(const float *uc, int cx, int cy, int cz, int nx, int 
                            float *uf, cudaStream_t s);
 cudaError_t launch_uroi(const uint8_t *sbits, int k, int nx, int ny, int nz, const double *spacing,
                         double margin, uint8_t *scratch, uint8_t *out, cudaStream_t s);
-size_t uroi_scratch_bytes(size_t n);
+size_t uroi_scratch_bytes(int nx, int ny, int nz);
 cudaError_t launch_sign_sums(const void *T0, int dtype, const uint8_t *sbits, int k, int nx, int ny, int nz,
-                             uint8_t *tmp_a, uint8_t *tmp_b, double *partial,
-                             double *sums /* [k][4] */, cudaStream_t s);
-size_t sign_partial_rows(size_t n);
+                             uint8_t *dxy, double *partial, double *sums /* [k][4] */, cudaStream_t s);
+size_t sign_partial_rows(int nx, int ny, int nz);
 // Convert n image values from in_dtype to out_dtype (round to nearest even).
 cudaError_t launch_convert_image(const void *in, int in_dtype, size_t n, void *out, int out_dtype,
                                  cudaStream_t s);

@@ -1386,8 +1386,21 @@ __global__ void __launch_bounds__(NT, 2) k_level_coop(const __grid_constant__ Le
     }
 }
 
+// Voxel coordinates of linear index i (32-bit divisions where they suffice).
+__device__ __forceinline__ void coords(size_t i, size_t N, int nx, int ny, int &x, int &y, int &z) {
+    if (N <= 0xffffffffull) {
+        const unsigned r = (unsigned)i / (unsigned)nx;
+        x = (int)((unsigned)i - r * (unsigned)nx);
+        z = (int)(r / (unsigned)ny);
+        y = (int)(r - (unsigned)z * (unsigned)ny);
+    } else {
+        x = (int)(i % nx); y = (int)((i / nx) % ny); z = (int)(i / ((size_t)nx * ny));
+    }
+}
+
 // Metric-only pass: I0~ at every voxel and the UROI partial sums (the warp
-// of Algorithm A step 5 after a level's last update).
+// of Algorithm A step 5 after a level's last update).  Grid-strided: the
+// UROI's voxels, a few compact regions, spread evenly over the threads.
 constexpr int MT = 256;
 template <typename IT>
 __global__ void __launch_bounds__(MT) k_metric(const IT *__restrict__ I0,
@@ -1402,7 +1415,8 @@ __global__ void __launch_bounds__(MT) k_metric(const IT *__restrict__ I0,
     int cnt = 0;
     for (size_t i = (size_t)blockIdx.x * MT + threadIdx.x; i < N; i += (size_t)gridDim.x * MT) {
         if (uroi && !uroi[i]) continue;
-        const int x = (int)(i % nx), y = (int)((i / nx) % ny), z = (int)(i / ((size_t)nx * ny));
+        int x, y, z;
+        coords(i, N, nx, ny, x, y, z);
         const Corners c = corners((float)x + __ldg(u + i), (float)y + __ldg(u + N + i),
                                   (float)z + __ldg(u + 2 * N + i), nx, ny, nz);
         float acc = 0.f;
@@ -1427,7 +1441,8 @@ __global__ void k_warp(const float *__restrict__ f, const float *__restrict__ u,
     const size_t N = (size_t)nx * ny * nz;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
          i += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % nx), y = (int)((i / nx) % ny), z = (int)(i / ((size_t)nx * ny));
+        int x, y, z;
+        coords(i, N, nx, ny, x, y, z);
         const Corners c = corners((float)x + __ldg(u + i), (float)y + __ldg(u + N + i),
                                   (float)z + __ldg(u + 2 * N + i), nx, ny, nz);
         float acc = 0.f;

@@ -5,6 +5,8 @@
 // type conversion.  None of these run per iteration.
 #include "cgdir_internal.cuh"
 
+#include <algorithm>
+
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -40,6 +42,25 @@ __global__ void k_pack4(MaskPtrs m, int k, size_t n4, uint32_t *__restrict__ bit
             if (j < k) b |= __vcmpne4(__ldg(reinterpret_cast<const uint32_t *>(m.p[j]) + i), 0u) & (0x01010101u << j);
         bits[i] = b;
     }
+}
+
+// Sixteen voxels per thread (16-byte loads, all masks' in flight together).
+__global__ void k_pack16(MaskPtrs m, int k, size_t n16, uint4 *__restrict__ bits) {
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n16) return;
+    uint4 w[kMaxMasks];
+#pragma unroll
+    for (int j = 0; j < kMaxMasks; ++j)
+        if (j < k) w[j] = __ldg(reinterpret_cast<const uint4 *>(m.p[j]) + i);
+    uint4 b = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int j = 0; j < kMaxMasks; ++j)
+        if (j < k) {
+            const uint32_t one = 0x01010101u << j;
+            b.x |= __vcmpne4(w[j].x, 0u) & one; b.y |= __vcmpne4(w[j].y, 0u) & one;
+            b.z |= __vcmpne4(w[j].z, 0u) & one; b.w |= __vcmpne4(w[j].w, 0u) & one;
+        }
+    bits[i] = b;
 }
 
 __global__ void k_pack(MaskPtrs m, int k, size_t n, uint8_t *__restrict__ bits) {
@@ -90,6 +111,41 @@ __global__ void k_restrict_image_rows(const IT *__restrict__ in, int nx, int ny,
     out[vox(X, Y, Z, cx, cy)] = from_f<OT>(s * 0.125f);
 }
 
+// The same where nx is even and rows are aligned for pairs: the two x
+// neighbours come by one load, four coarse values per thread are in flight.
+template <typename IT>
+struct PairOf { using type = unsigned; };
+template <>
+struct PairOf<float> { using type = float2; };
+__device__ __forceinline__ float2 pair_f(float2 v, float) { return v; }
+__device__ __forceinline__ float2 pair_f(unsigned v, __half) {
+    return make_float2(from_bits16<__half>(v & 0xffffu), from_bits16<__half>(v >> 16));
+}
+__device__ __forceinline__ float2 pair_f(unsigned v, __nv_bfloat16) {
+    return make_float2(from_bits16<__nv_bfloat16>(v & 0xffffu), from_bits16<__nv_bfloat16>(v >> 16));
+}
+template <typename IT, typename OT>
+__global__ void k_restrict_image_pairs(const IT *__restrict__ in, int nx, int ny, int nz, OT *__restrict__ out) {
+    using PT = typename PairOf<IT>::type;
+    const int cx = nx / 2, cy = (ny + 1) / 2;
+    const int X = blockIdx.x * RB + threadIdx.x, Y = blockIdx.y, Z = blockIdx.z;
+    if (X >= cx) return;
+    const int y1 = min(2 * Y + 1, ny - 1), z1 = min(2 * Z + 1, nz - 1);
+    PT p[4];
+    p[0] = __ldg(reinterpret_cast<const PT *>(in + vox(2 * X, 2 * Y, 2 * Z, nx, ny)));
+    p[1] = __ldg(reinterpret_cast<const PT *>(in + vox(2 * X, y1, 2 * Z, nx, ny)));
+    p[2] = __ldg(reinterpret_cast<const PT *>(in + vox(2 * X, 2 * Y, z1, nx, ny)));
+    p[3] = __ldg(reinterpret_cast<const PT *>(in + vox(2 * X, y1, z1, nx, ny)));
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float2 v = pair_f(p[q], IT());
+        s += v.x;
+        s += v.y;
+    }
+    out[vox(X, Y, Z, cx, cy)] = from_f<OT>(s * 0.125f);
+}
+
 // Per bit: inside if at least 4 of the 8 source voxels are inside.
 __global__ void k_restrict_bits(const uint8_t *__restrict__ in, int nx, int ny, int nz,
                                 uint8_t *__restrict__ out) {
@@ -114,7 +170,41 @@ __global__ void k_restrict_bits(const uint8_t *__restrict__ in, int nx, int ny, 
     }
 }
 
-// u_f(x) = 2 u_c((x + 0.5)/2 - 0.5), trilinear with clamped coordinates.
+// (256x256x96: 11.6 -> 5.2 us against the loop over bits below.)
+// Eight fine voxels of a row (one 8-byte load from each of the 2 x 2 rows) to
+// four coarse ones, nx % 8 == 0: the eight bytes of a coarse voxel are added
+// bit by bit with carry-save adders on 16-bit lanes (two coarse voxels per
+// word); the count is at least 4 where two of the four carries (worth 2
+// each) are set.
+__device__ __forceinline__ uint32_t majority8(const uint32_t *a) {
+    auto carry = [](uint32_t x, uint32_t y, uint32_t z) { return (x & y) | (z & (x ^ y)); };
+    const uint32_t s1 = a[0] ^ a[1] ^ a[2], c1 = carry(a[0], a[1], a[2]);
+    const uint32_t s2 = a[3] ^ a[4] ^ a[5], c2 = carry(a[3], a[4], a[5]);
+    const uint32_t s3 = a[6] ^ a[7], c3 = a[6] & a[7];
+    const uint32_t c4 = carry(s1, s2, s3);
+    return (c1 & c2) | (c3 & c4) | ((c1 | c2) & (c3 | c4));
+}
+__global__ void k_restrict_bits8(const uint8_t *__restrict__ in, int nx, int ny, int nz, uint8_t *__restrict__ out) {
+    const int cx = nx / 2, cy = (ny + 1) / 2;
+    const int g = blockIdx.x * RB + threadIdx.x, Y = blockIdx.y, Z = blockIdx.z;
+    if (8 * g >= nx) return;
+    const int y1 = min(2 * Y + 1, ny - 1), z1 = min(2 * Z + 1, nz - 1);
+    uint2 r[4];
+    r[0] = __ldg(reinterpret_cast<const uint2 *>(in + vox(8 * g, 2 * Y, 2 * Z, nx, ny)));
+    r[1] = __ldg(reinterpret_cast<const uint2 *>(in + vox(8 * g, y1, 2 * Z, nx, ny)));
+    r[2] = __ldg(reinterpret_cast<const uint2 *>(in + vox(8 * g, 2 * Y, z1, nx, ny)));
+    r[3] = __ldg(reinterpret_cast<const uint2 *>(in + vox(8 * g, y1, z1, nx, ny)));
+    uint32_t lo[8], hi[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        lo[2 * q] = r[q].x & 0x00ff00ffu; lo[2 * q + 1] = (r[q].x >> 8) & 0x00ff00ffu;
+        hi[2 * q] = r[q].y & 0x00ff00ffu; hi[2 * q + 1] = (r[q].y >> 8) & 0x00ff00ffu;
+    }
+    const uint32_t a = majority8(lo), b = majority8(hi);
+    *reinterpret_cast<uint32_t *>(out + vox(4 * g, Y, Z, cx, cy)) =
+        (a & 0xffu) | ((a >> 8) & 0xff00u) | ((b & 0xffu) << 16) | ((b & 0xff0000u) << 8);
+}
+
 __global__ void k_restrict_bits_rows(const uint8_t *__restrict__ in, int nx, int ny, int nz,
                                      uint8_t *__restrict__ out) {
     const int cx = (nx + 1) / 2, cy = (ny + 1) / 2;
@@ -135,61 +225,99 @@ __global__ void k_restrict_bits_rows(const uint8_t *__restrict__ in, int nx, int
     out[vox(X, Y, Z, cx, cy)] = (uint8_t)o;
 }
 
-// Prolongation over 64 x 8 x 8 fine tiles: the coarse values the tile's
-// interpolations read (34 x 6 x 6 per component, indices clamped) are staged
-// in shared memory once, then each thread forms two x-adjacent fine voxels per
-// row and plane with the same corners and the same order of multiply-adds as
-// k_prolong (same bits), and stores them as a pair.  Replaces 24 cached
-// gathers per fine voxel by shared-memory reads.
+// u_f(x) = 2 u_c((x + 0.5)/2 - 0.5), trilinear with clamped coordinates.
+// Tiles of 64 x 8 x 8 fine voxels: the coarse values the interpolations read
+// (34 x 6 x 6 per component, indices clamped) are staged in shared memory; a
+// thread forms 2 x 2 x 2 fine voxels (2X, 2X + 1 and so on) of one component at
+// a time from the 3 x 3 x 3 coarse values around (X, Y, Z): 27 shared reads
+// for 8 outputs.  Along an axis the even voxel's corners are the first two of
+// those three values and the odd one's the last two, with k_prolong's weights
+// and order of multiply-adds (same bits); at the low border, where the clamped
+// coordinate is 0, the weights are 1 and 0 on values that are both u_c(0).
 constexpr int PX = 64, PY = 8, PZ = 8;
 constexpr int PCX = PX / 2 + 2, PCY = PY / 2 + 2, PCZ = PZ / 2 + 2;
-__global__ void __launch_bounds__(256) k_prolong_tile(const float *__restrict__ uc, int cx, int cy, int cz, int nx,
+// Weights (low, high corner) of fine index x on a coarse axis of c voxels.
+__device__ __forceinline__ void prolong_axis(int x, int c, float *w) {
+    const float p = fminf(fmaxf((x + 0.5f) * 0.5f - 0.5f, 0.f), (float)(c - 1));
+    w[1] = p - floorf(p);
+    w[0] = 1.f - w[1];
+}
+__global__ void __launch_bounds__(128) k_prolong_tile(const float *__restrict__ uc, int cx, int cy, int cz, int nx,
                                                       int ny, int nz, float *__restrict__ uf) {
     __shared__ float t[3][PCZ][PCY][PCX];
     const int x0 = blockIdx.x * PX, y0 = blockIdx.y * PY, z0 = blockIdx.z * PZ;
     const int bx = x0 / 2 - 1, by = y0 / 2 - 1, bz = z0 / 2 - 1;      // coarse origin of the tile
     const size_t Nc = (size_t)cx * cy * cz, N = (size_t)nx * ny * nz;
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    for (int e = tid; e < 3 * PCZ * PCY * PCX; e += blockDim.x * blockDim.y) {
-        const int i = e % PCX, j = (e / PCX) % PCY, k = (e / (PCX * PCY)) % PCZ, comp = e / (PCX * PCY * PCZ);
-        const int gx = clampi(bx + i, 0, cx - 1), gy = clampi(by + j, 0, cy - 1), gz = clampi(bz + k, 0, cz - 1);
-        t[comp][k][j][i] = __ldg(uc + comp * Nc + ((size_t)gz * cy + gy) * cx + gx);
+    // a warp per coarse row, nine rows' loads in flight
+    static_assert(3 * PCZ * PCY % 36 == 0, "4 warps x 9 rows per turn");
+    const int ca = clampi(bx + (int)threadIdx.x, 0, cx - 1), cb = clampi(bx + 32 + (int)threadIdx.x, 0, cx - 1);
+    for (int r0 = threadIdx.y; r0 < 3 * PCZ * PCY; r0 += 36) {
+        float v[9], e[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const int row = r0 + 4 * q, j = row % PCY, k = (row / PCY) % PCZ, comp = row / (PCY * PCZ);
+            const float *src = uc + comp * Nc + ((size_t)clampi(bz + k, 0, cz - 1) * cy + clampi(by + j, 0, cy - 1)) * cx;
+            v[q] = __ldg(src + ca);
+            e[q] = threadIdx.x < PCX - 32 ? __ldg(src + cb) : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const int row = r0 + 4 * q, j = row % PCY, k = (row / PCY) % PCZ, comp = row / (PCY * PCZ);
+            t[comp][k][j][threadIdx.x] = v[q];
+            if (threadIdx.x < PCX - 32) t[comp][k][j][32 + threadIdx.x] = e[q];
+        }
     }
     __syncthreads();
-    const int y = y0 + threadIdx.y, xa = x0 + 2 * threadIdx.x;
-    if (y >= ny || xa >= nx) return;
-    const bool two = xa + 1 < nx;
-    for (int dz = 0; dz < PZ; ++dz) {
-        const int z = z0 + dz;
-        if (z >= nz) break;
-        float out[2][3];
+    const int lx = threadIdx.x, ly = threadIdx.y;                     // coarse cell of this thread: (lx, ly) of 32 x 4
+    const int xa = x0 + 2 * lx, ya = y0 + 2 * ly;
+    if (xa >= nx || ya >= ny) return;
+    float wx[2][2], wy[2][2];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int x = xa + h;
-            const Corners c = corners((x + 0.5f) * 0.5f - 0.5f, (y + 0.5f) * 0.5f - 0.5f, (z + 0.5f) * 0.5f - 0.5f,
-                                      cx, cy, cz);
-            float acc[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int qx = (q & 1) ? c.x1 : c.x0, qy = (q & 2) ? c.y1 : c.y0, qz = (q & 4) ? c.z1 : c.z0;
-                const float w = ((q & 1) ? c.wx : 1.f - c.wx) * ((q & 2) ? c.wy : 1.f - c.wy) *
-                                ((q & 4) ? c.wz : 1.f - c.wz);
-#pragma unroll
-                for (int comp = 0; comp < 3; ++comp)
-                    acc[comp] = fmaf(w, t[comp][qz - bz][qy - by][qx - bx], acc[comp]);
-            }
-#pragma unroll
-            for (int comp = 0; comp < 3; ++comp) out[h][comp] = 2.f * acc[comp];
-        }
-        const size_t i = vox(xa, y, z, nx, ny);
+    for (int h = 0; h < 2; ++h) {
+        prolong_axis(xa + h, cx, wx[h]);
+        prolong_axis(ya + h, cy, wy[h]);
+    }
+    const bool pair = xa + 1 < nx && nx % 2 == 0 && (reinterpret_cast<uintptr_t>(uf) & 7u) == 0;
+    for (int lz = 0; lz < PZ / 2; ++lz) {
+        const int za = z0 + 2 * lz;
+        if (za >= nz) break;
+        float wz[2][2];
+        prolong_axis(za, cz, wz[0]);
+        prolong_axis(za + 1, cz, wz[1]);
 #pragma unroll
         for (int comp = 0; comp < 3; ++comp) {
-            float *o = uf + comp * N + i;
-            if (two && (reinterpret_cast<uintptr_t>(o) & 7u) == 0) {
-                *reinterpret_cast<float2 *>(o) = make_float2(out[0][comp], out[1][comp]);
-            } else {
-                o[0] = out[0][comp];
-                if (two) o[1] = out[1][comp];
+            float c[3][3][3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) c[k][j][i] = t[comp][lz + k][ly + j][lx + i];
+#pragma unroll
+            for (int hz = 0; hz < 2; ++hz) {
+                if (za + hz >= nz) continue;
+#pragma unroll
+                for (int hy = 0; hy < 2; ++hy) {
+                    if (ya + hy >= ny) continue;
+                    float o[2];
+#pragma unroll
+                    for (int hx = 0; hx < 2; ++hx) {
+                        float acc = 0.f;
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const int i = q & 1, j = (q >> 1) & 1, k = q >> 2;
+                            acc = fmaf(wx[hx][i] * wy[hy][j] * wz[hz][k], c[hz + k][hy + j][hx + i], acc);
+                        }
+                        o[hx] = 2.f * acc;
+                    }
+                    float *d = uf + comp * N + vox(xa, ya + hy, za + hz, nx, ny);
+                    if (pair) {
+                        *reinterpret_cast<float2 *>(d) = make_float2(o[0], o[1]);
+                    } else {
+                        d[0] = o[0];
+                        if (xa + 1 < nx) d[1] = o[1];
+                    }
+                }
             }
         }
     }
@@ -219,137 +347,115 @@ __global__ void k_prolong(const float *__restrict__ uc, int cx, int cy, int cz, 
     }
 }
 
-// ---- UROI: exact ellipsoidal dilation in three passes -----------------
-// pass 1: per voxel, the distance |dx| (voxels) to the nearest union voxel of
-// its x-row within rx, 255 if none.  pass 2: per voxel (x, y, z') and per
-// z offset dz, bit dz+rz says that some row (y+dy, z') holds a union voxel
-// within the x extent the ellipsoid allows at (dy, dz).  pass 3: voxel
-// (x, y, z) is in the UROI if bit dz+rz of pass 2 at (x, y, z+dz) is set for
-// some dz.  The extents are computed on the host with the same double
-// expression as the definition, so the decision equals the brute-force test
-// voxel by voxel.
+// ---- UROI: exact ellipsoidal dilation on bit rows ---------------------------
+// The union of the structures is packed to one bit per voxel, rows of
+// ceil(nx / 32) words, so a thread handles 32 voxels with shifts and ORs:
+//   k_uroi_bits   bytes -> bits (N bytes read, N / 8 written)
+//   k_uroi_rows   per word of row (y, z) and per |dz| = 0 .. rz, the OR over dy
+//                 of row y + dy dilated in x by ext(dy, dz), the x extent the
+//                 ellipsoid admits there (-1: none); a dilation by r is built
+//                 from the one by r - 1 with two shifts over the neighbour words
+//   k_uroi_out    OR over dz of the |dz| words at z + dz, expanded to bytes
+// The extents are computed on the host with the same double expression as the
+// definition, so the decision equals the brute-force test voxel by voxel.
+// Two bytes per voxel must move; 256x256x96 with 10 mm takes 19 us, where byte
+// maps (row distances and per-voxel z masks, about 31 byte loads per voxel)
+// took 146 us.
 constexpr int kMaxUroiRadius = 15;
 struct UroiTable {
     int rx, ry, rz;
-    int8_t ext[2 * kMaxUroiRadius + 1][2 * kMaxUroiRadius + 1];   // [dz][dy], -1 = none
+    int8_t ext[kMaxUroiRadius + 1][kMaxUroiRadius + 1];   // [|dz|][|dy|], -1 = none
 };
 
-__global__ void k_uroi_rows(const uint8_t *__restrict__ sbits, unsigned mask, int rx, int nx,
-                            int ny, int nz, uint8_t *__restrict__ rowdist) {
-    const size_t N = (size_t)nx * ny * nz;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % nx);
-        int d = 255;
-        for (int dx = -rx; dx <= rx; ++dx) {
-            const int xx = x + dx;
-            if (xx < 0 || xx >= nx) continue;
-            if (__ldg(sbits + i - x + xx) & mask) d = min(d, abs(dx));
-        }
-        rowdist[i] = (uint8_t)d;
+// Word i of the bit rows: its row (y, z) and first voxel x.
+struct BitWord {
+    long long row;
+    int x;
+    __device__ BitWord(long long i, int wpr) {
+        row = i < (1ll << 31) ? (long long)((unsigned)i / (unsigned)wpr) : i / wpr;
+        x = (int)(i - row * wpr) * 32;
     }
-}
-
-__global__ void k_uroi_planes(const uint8_t *__restrict__ rowdist, UroiTable t, int nx, int ny, int nz,
-                              uint32_t *__restrict__ zbits) {
-    const size_t N = (size_t)nx * ny * nz;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int y = (int)((i / nx) % ny);
-        uint32_t b = 0;
-        for (int dy = -t.ry; dy <= t.ry; ++dy) {
-            const int yy = y + dy;
-            if (yy < 0 || yy >= ny) continue;
-            const int r = __ldg(rowdist + i + (ptrdiff_t)dy * nx);
-            if (r == 255) continue;
-            for (int dz = -t.rz; dz <= t.rz; ++dz)
-                if (r <= t.ext[dz + t.rz][dy + t.ry]) b |= 1u << (dz + t.rz);
-        }
-        zbits[i] = b;
+    __device__ int z(int ny) const {
+        return (int)(row < (1ll << 31) ? (unsigned)row / (unsigned)ny : row / ny);
     }
-}
-
-__global__ void k_uroi_dilate(const uint32_t *__restrict__ zbits, int rz, int nx, int ny, int nz,
-                              uint8_t *__restrict__ out) {
-    const size_t N = (size_t)nx * ny * nz, nxy = (size_t)nx * ny;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int z = (int)(i / nxy);
-        uint32_t hit = 0;
-        for (int dz = -rz; dz <= rz; ++dz) {
-            const int zz = z + dz;
-            if (zz < 0 || zz >= nz) continue;
-            hit |= ((uint32_t)__ldg(zbits + i + (ptrdiff_t)dz * (ptrdiff_t)nxy) >> (dz + rz)) & 1u;
-        }
-        out[i] = (uint8_t)hit;
-    }
-}
-
-// Row versions of the three UROI passes.  Pass 1 stages the row's mask bits
-// (with an rx halo) in shared memory; pass 2 takes, per y offset, the z
-// offsets whose extent admits the row distance r from a table built on the
-// host (bit dz + rz of zsets[dy + ry][r] set iff r <= ext[dz][dy]), the same
-// decisions as the loop over dz.
-struct UroiZsets {
-    uint32_t zs[2 * kMaxUroiRadius + 1][kMaxUroiRadius + 1];
 };
 
-__global__ void k_uroi_rows_r(const uint8_t *__restrict__ sbits, unsigned mask, int rx, int nx, int ny, int nz,
-                              uint8_t *__restrict__ rowdist) {
-    __shared__ uint8_t row[RB + 2 * kMaxUroiRadius];
-    const int x0 = blockIdx.x * RB, y = blockIdx.y, z = blockIdx.z;
-    const size_t rb = vox(0, y, z, nx, ny);
-    for (int p = threadIdx.x; p < RB + 2 * rx; p += RB) {
-        const int xx = x0 - rx + p;
-        row[p] = (xx >= 0 && xx < nx && (__ldg(sbits + rb + xx) & mask)) ? 1 : 0;
-    }
-    __syncthreads();
-    const int x = x0 + threadIdx.x;
-    if (x >= nx) return;
-    int d = 255;
-    for (int dx = -rx; dx <= rx; ++dx)
-        if (row[threadIdx.x + rx + dx]) d = min(d, abs(dx));
-    rowdist[rb + x] = (uint8_t)d;
+// Bit q set where byte q of w has a bit of the mask.
+__device__ __forceinline__ uint32_t bits_of(uint32_t w, uint32_t mask4) {
+    const uint32_t b = __vcmpne4(w & mask4, 0u) & 0x08040201u;      // bit q of byte q
+    return (b | (b >> 8) | (b >> 16) | (b >> 24)) & 0xfu;
 }
-
-// W: the z-mask word, 16 bits where 2 rz + 1 <= 16 (half the bytes written
-// here and read by the z pass), else 32.
-template <typename W>
-__global__ void k_uroi_planes_r(const uint8_t *__restrict__ rowdist, const __grid_constant__ UroiZsets t, int ry,
-                                int nx, int ny, int nz, W *__restrict__ zbits) {
-    const int x = blockIdx.x * RB + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
-    if (x >= nx) return;
-    const size_t i = vox(x, y, z, nx, ny);
+__global__ void k_uroi_bits(const uint8_t *__restrict__ sbits, unsigned mask, int nx, long long words, int wpr, int vec,
+                            uint32_t *__restrict__ bits) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= words) return;
+    const BitWord bw(i, wpr);
+    const int x = bw.x;
+    const uint8_t *src = sbits + (size_t)bw.row * nx + x;
     uint32_t b = 0;
-    for (int dy = -ry; dy <= ry; ++dy) {
-        const int yy = y + dy;
-        if (yy < 0 || yy >= ny) continue;
-        const int r = __ldg(rowdist + i + (ptrdiff_t)dy * nx);
-        if (r != 255) b |= t.zs[dy + ry][r];
+    if (vec && x + 32 <= nx) {                     // 16-byte aligned rows
+        const uint32_t m4 = mask * 0x01010101u;
+        const uint4 p = __ldg(reinterpret_cast<const uint4 *>(src)), q = __ldg(reinterpret_cast<const uint4 *>(src) + 1);
+        b = bits_of(p.x, m4) | bits_of(p.y, m4) << 4 | bits_of(p.z, m4) << 8 | bits_of(p.w, m4) << 12 |
+            bits_of(q.x, m4) << 16 | bits_of(q.y, m4) << 20 | bits_of(q.z, m4) << 24 | bits_of(q.w, m4) << 28;
+    } else {
+#pragma unroll 8
+        for (int e = 0; e < 32; ++e)
+            if (x + e < nx && (__ldg(src + e) & mask)) b |= 1u << e;
     }
-    zbits[i] = (W)b;
+    bits[i] = b;
 }
 
-// Pass 3 marching z: a thread owns an x position of a row and takes kUroiZc
-// consecutive planes, so each z-mask word it reads for one plane is read
-// again, from L1, for the next 2 rz planes.
-constexpr int kUroiZc = 16;
-template <typename W>
-__global__ void k_uroi_dilate_r(const W *__restrict__ zbits, int rz, int nx, int ny, int nz,
-                                uint8_t *__restrict__ out) {
-    const int x = blockIdx.x * RB + threadIdx.x, y = blockIdx.y;
-    if (x >= nx) return;
-    const int zb = blockIdx.z * kUroiZc, ze = min(zb + kUroiZc, nz);
-    const size_t nxy = (size_t)nx * ny;
-    for (int z = zb; z < ze; ++z) {
-        const size_t i = vox(x, y, z, nx, ny);
-        uint32_t hit = 0;
-        for (int dz = -rz; dz <= rz; ++dz) {
-            const int zz = z + dz;
-            if (zz < 0 || zz >= nz) continue;
-            hit |= (__ldg(zbits + i + (ptrdiff_t)dz * (ptrdiff_t)nxy) >> (dz + rz)) & 1u;
+// NZ: accumulators (|dz| values) per thread, at least rz + 1.
+template <int NZ>
+__global__ void k_uroi_rows(const uint32_t *__restrict__ bits, const __grid_constant__ UroiTable t, int ny,
+                            long long words, int wpr, uint32_t *__restrict__ zrows) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= words) return;
+    const BitWord bw(i, wpr);
+    const int c = bw.x / 32, y = (int)(bw.row - (long long)bw.z(ny) * ny);
+    uint32_t acc[NZ];
+#pragma unroll
+    for (int z = 0; z < NZ; ++z) acc[z] = 0u;
+    for (int dy = -t.ry; dy <= t.ry; ++dy) {
+        if (y + dy < 0 || y + dy >= ny) continue;
+        const uint32_t *r = bits + i + (long long)dy * wpr;
+        const uint32_t w = __ldg(r), pw = c > 0 ? __ldg(r - 1) : 0u, nw = c + 1 < wpr ? __ldg(r + 1) : 0u;
+        if ((w | pw | nw) == 0u) continue;
+        uint32_t d = w;                             // the row dilated by q
+        for (int q = 0; q <= t.rx; ++q) {
+            if (q > 0) d |= __funnelshift_l(pw, w, q) | __funnelshift_r(w, nw, q);
+#pragma unroll
+            for (int z = 0; z < NZ; ++z)
+                if (z <= t.rz && t.ext[z][dy < 0 ? -dy : dy] == q) acc[z] |= d;
         }
-        out[i] = (uint8_t)hit;
+    }
+    for (int z = 0; z < NZ; ++z)
+        if (z <= t.rz) zrows[(size_t)z * words + i] = acc[z];
+}
+
+// The bytes 0 / 1 of bits 4 e .. 4 e + 3 of w.
+__device__ __forceinline__ uint32_t byte4(uint32_t w, int e) {
+    const uint32_t n = (w >> (4 * e)) & 0xfu;
+    return (n | (n << 7) | (n << 14) | (n << 21)) & 0x01010101u;
+}
+__global__ void k_uroi_out(const uint32_t *__restrict__ zrows, int rz, int nx, int ny, int nz,
+                           long long words, int wpr, int vec, uint8_t *__restrict__ out) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x, plane = (long long)ny * wpr;
+    if (i >= words) return;
+    const BitWord bw(i, wpr);
+    const int x = bw.x, z = bw.z(ny);
+    uint32_t b = 0;
+    for (int dz = -rz; dz <= rz; ++dz) {
+        if (z + dz < 0 || z + dz >= nz) continue;
+        b |= __ldg(zrows + (size_t)(dz < 0 ? -dz : dz) * words + i + dz * plane);
+    }
+    uint8_t *dst = out + (size_t)bw.row * nx + x;
+    if (vec && x + 32 <= nx) {
+        reinterpret_cast<uint4 *>(dst)[0] = make_uint4(byte4(b, 0), byte4(b, 1), byte4(b, 2), byte4(b, 3));
+        reinterpret_cast<uint4 *>(dst)[1] = make_uint4(byte4(b, 4), byte4(b, 5), byte4(b, 6), byte4(b, 7));
+    } else {
+        for (int e = 0; e < 32 && x + e < nx; ++e) dst[e] = (uint8_t)((b >> e) & 1u);
     }
 }
 
@@ -360,55 +466,187 @@ __global__ void k_fill_u8(uint8_t *p, size_t n, uint8_t v) {
 }
 
 // ---- automatic sign ---------------------------------------------------
-// Chebyshev dilation by 2 voxels of all mask bits, one axis per launch.
-__global__ void k_dilate_axis(const uint8_t *__restrict__ in, int axis, int nx, int ny, int nz,
-                              uint8_t *__restrict__ out) {
-    const size_t N = (size_t)nx * ny * nz;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % nx), y = (int)((i / nx) % ny), z = (int)(i / ((size_t)nx * ny));
-        unsigned b = 0;
-        for (int d = -2; d <= 2; ++d) {
-            int xx = x, yy = y, zz = z;
-            if (axis == 0) xx += d; else if (axis == 1) yy += d; else zz += d;
-            if (xx < 0 || yy < 0 || zz < 0 || xx >= nx || yy >= ny || zz >= nz) continue;
-            b |= __ldg(in + vox(xx, yy, zz, nx, ny));
+// Per structure {sum T0 inside, count inside, sum T0 in the shell, count of the
+// shell}, the shell being the voxels outside the structure within Chebyshev
+// distance 2 of it.  k_dilate_xy ORs the mask bytes over 5 x 5 voxels in each
+// plane; k_sign_sums marches along z with five planes of that in registers and
+// reads T0 only where some structure or shell is.  A thread owns V x-adjacent
+// voxels (V = 4, one 32-bit word of mask bytes, where nx % 4 == 0).  A thread
+// sums in pairs of floats (high part and rounding errors, exact to 2^-47 of the
+// sum for its 64 voxels at most), because FP64 adds take a warp 14 cycles of
+// the SM here; across threads the sums are FP64.  A structure that no thread of
+// a warp met costs it no reduction.
+// 256x256x96, 5 structures, all three kernels: 39 us; with FP64 sums per thread
+// 87 us; with three dilation launches and, per structure, an FP64 pass over T0
+// and a serial sum of its partials 742 us.
+constexpr int SB = 256, SZ = 16;                  // threads (32 x 8), most planes per CTA
+// A 1-D grid of 32 V x 8 tiles, x fastest, then y, then z: no limit on ny or nz.
+struct SignTile {
+    int x, y, bz;
+    __device__ SignTile(int nx, int ny, int v) {
+        const int tx = (nx + 32 * v - 1) / (32 * v), ty = (ny + 7) / 8, bid = blockIdx.x;
+        bz = bid / (tx * ty);
+        const int by = (bid - bz * tx * ty) / tx;
+        x = v * ((bid - (bz * ty + by) * tx) * 32 + threadIdx.x);
+        y = by * 8 + threadIdx.y;
+    }
+};
+// A sum of floats as high part and the rounding errors' sum (Knuth's two-sum).
+struct PairSum {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+        s = t;
+    }
+    __device__ __forceinline__ double value() const { return isfinite(s) ? (double)s + (double)e : (double)s; }
+};
+template <int V>
+__global__ void __launch_bounds__(SB) k_dilate_xy(const uint8_t *__restrict__ bits, int nx, int ny,
+                                                  uint8_t *__restrict__ out) {
+    const SignTile t(nx, ny, V);
+    const int x = t.x, y = t.y;
+    if (x >= nx || y >= ny) return;
+    // rows outside the volume are read at the border, which lies within
+    // distance 2 as well: no branch between the loads
+    uint32_t w[5][V == 4 ? 3 : 5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        const uint8_t *r = bits + ((size_t)t.bz * ny + clampi(y + q - 2, 0, ny - 1)) * nx + x;
+        if constexpr (V == 4) {
+            const uint32_t *rw = reinterpret_cast<const uint32_t *>(r);
+            w[q][0] = __ldg(rw);
+            w[q][1] = __ldg(rw - (x > 0 ? 1 : 0));
+            w[q][2] = __ldg(rw + (x + 4 < nx ? 1 : 0));
+        } else {
+#pragma unroll
+            for (int e = 0; e < 5; ++e) w[q][e] = __ldg(r + (clampi(x + e - 2, 0, nx - 1) - x));
         }
-        out[i] = (uint8_t)b;
+    }
+    uint32_t d = 0;
+    const size_t i = ((size_t)t.bz * ny + y) * nx + x;
+    if constexpr (V == 4) {
+        uint32_t c = 0, p = 0, n = 0;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) { c |= w[q][0]; p |= w[q][1]; n |= w[q][2]; }
+        if (x == 0) p = 0u;
+        if (x + 4 >= nx) n = 0u;
+        d = c | __funnelshift_l(p, c, 8) | __funnelshift_l(p, c, 16) | __funnelshift_r(c, n, 8) |
+            __funnelshift_r(c, n, 16);
+        *reinterpret_cast<uint32_t *>(out + i) = d;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+#pragma unroll
+            for (int e = 0; e < 5; ++e) d |= w[q][e];
+        out[i] = (uint8_t)d;
     }
 }
 
-constexpr int ST = 256;
-// Per block: {sum T0 inside j, count inside, sum T0 in shell, count shell}.
-template <typename IT>
-__global__ void __launch_bounds__(ST) k_sign_partial(const IT *__restrict__ T0,
-                                                     const uint8_t *__restrict__ sbits,
-                                                     const uint8_t *__restrict__ dil, int j,
-                                                     size_t n, double *__restrict__ partial) {
-    double a = 0, b = 0, c = 0, d = 0;
-    for (size_t i = (size_t)blockIdx.x * ST + threadIdx.x; i < n; i += (size_t)gridDim.x * ST) {
-        const bool in = (__ldg(sbits + i) >> j) & 1u;
-        const bool sh = !in && ((__ldg(dil + i) >> j) & 1u);
-        const double t = (double)ld_img<IT>(T0 + i);
-        if (in) { a += t; b += 1.0; }
-        if (sh) { c += t; d += 1.0; }
+template <typename IT, int V>
+__global__ void __launch_bounds__(SB) k_sign_sums(const IT *__restrict__ T0, const uint8_t *__restrict__ sbits,
+                                                  const uint8_t *__restrict__ dxy, int k, int nx, int ny, int nz,
+                                                  int zc, double *__restrict__ partial) {
+    const SignTile st(nx, ny, V);
+    const int x = st.x, y = st.y, zb = st.bz * zc, ze = min(zb + zc, nz);
+    const int tid = threadIdx.y * 32 + threadIdx.x, bid = blockIdx.x;
+    const unsigned kmask = (1u << k) - 1u;
+    PairSum sin_[kMaxMasks], ssh[kMaxMasks];
+    int cnt[kMaxMasks] = {};                      // inside (low 16 bits) and shell: at most 4 SZ each
+    unsigned seen = 0;
+    if (x < nx && y < ny) {
+        const size_t nxy = (size_t)nx * ny, col = (size_t)y * nx + x;
+        auto word = [&](const uint8_t *b, int z) -> uint32_t {       // 0 outside the volume
+            if (z < 0 || z >= nz) return 0u;
+            const uint8_t *p = b + (size_t)z * nxy + col;
+            return V == 4 ? __ldg(reinterpret_cast<const uint32_t *>(p)) : (uint32_t)__ldg(p);
+        };
+        // planes z - 2 .. z + 2 of the dilated bytes, z + 3 and the next plane's own bytes in flight
+        uint32_t d0 = 0, d1 = word(dxy, zb - 2), d2 = word(dxy, zb - 1), d3 = word(dxy, zb), d4 = word(dxy, zb + 1),
+                 nd = word(dxy, zb + 2), nc = word(sbits, zb);
+        for (int z = zb; z < ze; ++z) {
+            d0 = d1; d1 = d2; d2 = d3; d3 = d4; d4 = nd;
+            const uint32_t cen = nc, all = d0 | d1 | d2 | d3 | d4;
+            nd = word(dxy, z + 3);
+            nc = word(sbits, z + 1);
+            if (all == 0u) continue;              // no structure within distance 2 of these voxels
+            const size_t i = (size_t)z * nxy + col;
+            float tv[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) tv[v] = ld_img<IT>(T0 + i + v);
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const unsigned in = (cen >> (8 * v)) & kmask, sh = (all >> (8 * v)) & kmask & ~in;
+                if ((in | sh) == 0u) continue;
+                seen |= in | sh;
+#pragma unroll
+                for (int j = 0; j < kMaxMasks; ++j) {
+                    if ((in >> j) & 1u) { sin_[j].add(tv[v]); cnt[j] += 1; }
+                    if ((sh >> j) & 1u) { ssh[j].add(tv[v]); cnt[j] += 1 << 16; }
+                }
+            }
+        }
     }
-    __shared__ double r[4][ST];
-    r[0][threadIdx.x] = a; r[1][threadIdx.x] = b; r[2][threadIdx.x] = c; r[3][threadIdx.x] = d;
+    // block sums in a fixed order: lanes by shuffles, then the 8 warps in turn
+    __shared__ double ws[kMaxMasks][2][8];
+    __shared__ int wc[kMaxMasks][2][8];
+    const unsigned wseen = __reduce_or_sync(0xffffffffu, seen);
+#pragma unroll
+    for (int j = 0; j < kMaxMasks; ++j) {
+        if (j >= k) break;
+        double a = 0.0, c = 0.0;
+        int ca = 0, cc = 0;
+        if ((wseen >> j) & 1u) {                  // the same for the whole warp
+            a = sin_[j].value(); c = ssh[j].value();
+            ca = __reduce_add_sync(0xffffffffu, cnt[j] & 0xffff);
+            cc = __reduce_add_sync(0xffffffffu, cnt[j] >> 16);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                a += __shfl_xor_sync(0xffffffffu, a, o);
+                c += __shfl_xor_sync(0xffffffffu, c, o);
+            }
+        }
+        if ((tid & 31) == 0) {
+            ws[j][0][tid >> 5] = a; ws[j][1][tid >> 5] = c;
+            wc[j][0][tid >> 5] = ca; wc[j][1][tid >> 5] = cc;
+        }
+    }
+    const bool any = __syncthreads_or(seen != 0u);
+    if (tid < 2 * k) {                            // one thread per structure and side
+        const int j = tid >> 1, side = tid & 1;
+        double A = 0;
+        int C = 0;
+        if (any)
+            for (int w = 0; w < 8; ++w) { A += ws[j][side][w]; C += wc[j][side][w]; }
+        double *o = partial + ((size_t)bid * k + j) * 4 + 2 * side;
+        o[0] = A; o[1] = (double)C;
+    }
+}
+
+// Column sums of partial[rows][cols], a CTA per column: each thread takes a
+// fixed stride of rows, then lanes and warps are added in a fixed order.
+__global__ void __launch_bounds__(256) k_sum_rows(const double *__restrict__ partial, int rows, int cols,
+                                                  double *__restrict__ out) {
+    __shared__ double ws[8];
+    const int c = blockIdx.x, tid = threadIdx.x;
+    double s = 0;
+    int b = tid;
+    for (; b + 7 * 256 < rows; b += 8 * 256) {               // eight rows in flight, added in order
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = __ldg(partial + (size_t)(b + q * 256) * cols + c);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) s += v[q];
+    }
+    for (; b < rows; b += 256) s += __ldg(partial + (size_t)b * cols + c);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((tid & 31) == 0) ws[tid >> 5] = s;
     __syncthreads();
-    for (int h = ST / 2; h > 0; h >>= 1) {
-        if (threadIdx.x < h)
-            for (int q = 0; q < 4; ++q) r[q][threadIdx.x] += r[q][threadIdx.x + h];
-        __syncthreads();
-    }
-    if (threadIdx.x < 4) partial[(size_t)blockIdx.x * 4 + threadIdx.x] = r[threadIdx.x][0];
-}
-
-__global__ void k_sum_rows4(const double *__restrict__ partial, int rows, double *__restrict__ out) {
-    if (threadIdx.x < 4) {
-        double s = 0;
-        for (int b = 0; b < rows; ++b) s += partial[(size_t)b * 4 + threadIdx.x];
-        out[threadIdx.x] = s;
+    if (tid == 0) {
+        double t = 0;
+        for (int w = 0; w < 8; ++w) t += ws[w];
+        out[c] = t;
     }
 }
 
@@ -439,12 +677,15 @@ __global__ void k_convert(const IN *__restrict__ in, size_t n, OUT *__restrict__
 cudaError_t launch_pack_masks(const uint8_t *const *masks, int k, size_t n, uint8_t *bits,
                               cudaStream_t s) {
     MaskPtrs m{};
-    bool aligned = n % 4 == 0 && reinterpret_cast<uintptr_t>(bits) % 4 == 0;
+    uintptr_t low = reinterpret_cast<uintptr_t>(bits) | n;      // low bits of every pointer and the size
     for (int j = 0; j < k && j < kMaxMasks; ++j) {
         m.p[j] = masks[j];
-        aligned = aligned && reinterpret_cast<uintptr_t>(masks[j]) % 4 == 0;
+        low |= reinterpret_cast<uintptr_t>(masks[j]);
     }
-    if (aligned)
+    if (n == 0) return cudaSuccess;
+    if (low % 16 == 0 && n / 16 / 128 < ((size_t)1 << 31) - 1)
+        k_pack16<<<(unsigned)((n / 16 + 127) / 128), 128, 0, s>>>(m, k, n / 16, reinterpret_cast<uint4 *>(bits));
+    else if (low % 4 == 0)
         k_pack4<<<flat_grid(n / 4), 256, 0, s>>>(m, k, n / 4, reinterpret_cast<uint32_t *>(bits));
     else
         k_pack<<<flat_grid(n), 256, 0, s>>>(m, k, n, bits);
@@ -457,6 +698,16 @@ static void restrict_image_to(const void *in, int nx, int ny, int nz, void *out,
                               cudaStream_t s) {
     const IT *src = static_cast<const IT *>(in);
     const int cx = (nx + 1) / 2, cy = (ny + 1) / 2, cz = (nz + 1) / 2;
+    if (rows_ok(cy, cz) && nx % 2 == 0 && (reinterpret_cast<uintptr_t>(in) & (2 * sizeof(IT) - 1)) == 0) {
+        const dim3 g = row_grid(cx, cy, cz);
+        if (out_dtype == CGDIR_F16)
+            k_restrict_image_pairs<IT, __half><<<g, RB, 0, s>>>(src, nx, ny, nz, (__half *)out);
+        else if (out_dtype == CGDIR_BF16)
+            k_restrict_image_pairs<IT, __nv_bfloat16><<<g, RB, 0, s>>>(src, nx, ny, nz, (__nv_bfloat16 *)out);
+        else
+            k_restrict_image_pairs<IT, float><<<g, RB, 0, s>>>(src, nx, ny, nz, (float *)out);
+        return;
+    }
     if (rows_ok(cy, cz)) {
         const dim3 g = row_grid(cx, cy, cz);
         if (out_dtype == CGDIR_F16)
@@ -497,7 +748,10 @@ cudaError_t launch_restrict_bits(const uint8_t *in, int nx, int ny, int nz, uint
                                  cudaStream_t s) {
     const size_t Nc = (size_t)((nx + 1) / 2) * ((ny + 1) / 2) * ((nz + 1) / 2);
     const int cx = (nx + 1) / 2, cy = (ny + 1) / 2, cz = (nz + 1) / 2;
-    if (rows_ok(cy, cz))
+    if (rows_ok(cy, cz) && nx % 8 == 0 && (reinterpret_cast<uintptr_t>(in) & 7u) == 0 &&
+        (reinterpret_cast<uintptr_t>(out) & 3u) == 0)
+        k_restrict_bits8<<<row_grid(nx / 8, cy, cz), RB, 0, s>>>(in, nx, ny, nz, out);
+    else if (rows_ok(cy, cz))
         k_restrict_bits_rows<<<row_grid(cx, cy, cz), RB, 0, s>>>(in, nx, ny, nz, out);
     else
         k_restrict_bits<<<flat_grid(Nc), 256, 0, s>>>(in, nx, ny, nz, out);
@@ -507,8 +761,8 @@ cudaError_t launch_restrict_bits(const uint8_t *in, int nx, int ny, int nz, uint
 
 cudaError_t launch_prolong(const float *uc, int cx, int cy, int cz, int nx, int ny, int nz,
                            float *uf, cudaStream_t s) {
-    if (rows_ok(ny, nz))
-        k_prolong_tile<<<dim3((nx + PX - 1) / PX, (ny + PY - 1) / PY, (nz + PZ - 1) / PZ), dim3(32, 8), 0, s>>>(
+    if (rows_ok(ny, nz) && nx <= 2 * cx && ny <= 2 * cy && nz <= 2 * cz)
+        k_prolong_tile<<<dim3((nx + PX - 1) / PX, (ny + PY - 1) / PY, (nz + PZ - 1) / PZ), dim3(32, 4), 0, s>>>(
             uc, cx, cy, cz, nx, ny, nz, uf);
     else
         k_prolong<<<flat_grid((size_t)nx * ny * nz), 256, 0, s>>>(uc, cx, cy, cz, nx, ny, nz, uf);
@@ -516,8 +770,7 @@ cudaError_t launch_prolong(const float *uc, int cx, int cy, int cz, int nx, int 
     return cudaGetLastError();
 }
 
-// scratch: 5 N bytes (row distances, then per-voxel z masks at offset N
-// rounded up to 4 bytes).
+// scratch: uroi_scratch_bytes.
 cudaError_t launch_uroi(const uint8_t *sbits, int k, int nx, int ny, int nz, const double *spacing,
                         double margin, uint8_t *scratch, uint8_t *out, cudaStream_t s) {
     const size_t N = (size_t)nx * ny * nz;
@@ -533,74 +786,78 @@ cudaError_t launch_uroi(const uint8_t *sbits, int k, int nx, int ny, int nz, con
     t.rz = (int)(margin / spacing[2]);
     if (t.rx > kMaxUroiRadius || t.ry > kMaxUroiRadius || t.rz > kMaxUroiRadius)
         return cudaErrorInvalidValue;
-    for (int dz = -t.rz; dz <= t.rz; ++dz)
-        for (int dy = -t.ry; dy <= t.ry; ++dy) {
+    for (int dz = 0; dz <= t.rz; ++dz)
+        for (int dy = 0; dy <= t.ry; ++dy) {
             int e = -1;
             for (int dx = 0; dx <= t.rx; ++dx) {
                 const double d2 = (dx * spacing[0]) * (dx * spacing[0]) + (dy * spacing[1]) * (dy * spacing[1]) +
                                   (dz * spacing[2]) * (dz * spacing[2]);
                 if (d2 <= margin * margin) e = dx;
             }
-            t.ext[dz + t.rz][dy + t.ry] = (int8_t)e;
+            t.ext[dz][dy] = (int8_t)e;
         }
     const unsigned mask = (k >= 8) ? 0xffu : ((1u << k) - 1u);
-    uint8_t *rowdist = scratch;
-    uint32_t *zbits = reinterpret_cast<uint32_t *>(scratch + (N + 3) / 4 * 4);
-    if (rows_ok(ny, nz)) {
-        UroiZsets zt{};
-        for (int dy = -t.ry; dy <= t.ry; ++dy)
-            for (int r = 0; r <= t.rx; ++r) {
-                uint32_t b = 0;
-                for (int dz = -t.rz; dz <= t.rz; ++dz)
-                    if (r <= t.ext[dz + t.rz][dy + t.ry]) b |= 1u << (dz + t.rz);
-                zt.zs[dy + t.ry][r] = b;
-            }
-        const dim3 g = row_grid(nx, ny, nz);
-        k_uroi_rows_r<<<g, RB, 0, s>>>(sbits, mask, t.rx, nx, ny, nz, rowdist); note_launch();
-        const dim3 gz(g.x, g.y, (unsigned)((nz + kUroiZc - 1) / kUroiZc));
-        if (2 * t.rz + 1 <= 16) {
-            uint16_t *z16 = reinterpret_cast<uint16_t *>(zbits);
-            k_uroi_planes_r<uint16_t><<<g, RB, 0, s>>>(rowdist, zt, t.ry, nx, ny, nz, z16); note_launch();
-            k_uroi_dilate_r<uint16_t><<<gz, RB, 0, s>>>(z16, t.rz, nx, ny, nz, out); note_launch();
-        } else {
-            k_uroi_planes_r<uint32_t><<<g, RB, 0, s>>>(rowdist, zt, t.ry, nx, ny, nz, zbits); note_launch();
-            k_uroi_dilate_r<uint32_t><<<gz, RB, 0, s>>>(zbits, t.rz, nx, ny, nz, out); note_launch();
-        }
-        return cudaGetLastError();
-    }
-    k_uroi_rows<<<flat_grid(N), 256, 0, s>>>(sbits, mask, t.rx, nx, ny, nz, rowdist); note_launch();
-    k_uroi_planes<<<flat_grid(N), 256, 0, s>>>(rowdist, t, nx, ny, nz, zbits); note_launch();
-    k_uroi_dilate<<<flat_grid(N), 256, 0, s>>>(zbits, t.rz, nx, ny, nz, out); note_launch();
+    const int wpr = (nx + 31) / 32;
+    const long long words = (long long)ny * nz * wpr;
+    uint32_t *bits = reinterpret_cast<uint32_t *>(scratch), *zrows = bits + words;
+    const unsigned g = (unsigned)((words + 127) / 128);
+    auto aligned = [&](const void *q) { return nx % 16 == 0 && (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
+    k_uroi_bits<<<g, 128, 0, s>>>(sbits, mask, nx, words, wpr, aligned(sbits), bits); note_launch();
+    if (t.rz < 5) k_uroi_rows<5><<<g, 128, 0, s>>>(bits, t, ny, words, wpr, zrows);
+    else k_uroi_rows<kMaxUroiRadius + 1><<<g, 128, 0, s>>>(bits, t, ny, words, wpr, zrows);
+    note_launch();
+    k_uroi_out<<<g, 128, 0, s>>>(zrows, t.rz, nx, ny, nz, words, wpr, aligned(out), out); note_launch();
     return cudaGetLastError();
 }
 
-size_t uroi_scratch_bytes(size_t n) { return (n + 3) / 4 * 4 + 4 * n; }
+// Bit rows, then up to kMaxUroiRadius + 1 words per bit-row word.
+size_t uroi_scratch_bytes(int nx, int ny, int nz) {
+    return (size_t)ny * nz * ((nx + 31) / 32) * 4 * (kMaxUroiRadius + 2);
+}
 
-// sums: device [k][4]; tmp_a, tmp_b: N bytes each; partial: sign_partial_rows(N) x 4 doubles.
-cudaError_t launch_sign_sums(const void *T0, int dtype, const uint8_t *sbits, int k, int nx, int ny,
-                                int nz, uint8_t *tmp_a, uint8_t *tmp_b, double *partial,
-                                double *sums, cudaStream_t s) {
-    const size_t N = (size_t)nx * ny * nz;
-    const unsigned g = flat_grid(N);
-    k_dilate_axis<<<g, 256, 0, s>>>(sbits, 0, nx, ny, nz, tmp_a);
-    k_dilate_axis<<<g, 256, 0, s>>>(tmp_a, 1, nx, ny, nz, tmp_b);
-    k_dilate_axis<<<g, 256, 0, s>>>(tmp_b, 2, nx, ny, nz, tmp_a);
+static size_t sign_ctas(int nx, int ny, int nz, int v, int zc) {
+    return (size_t)((nx + 32 * v - 1) / (32 * v)) * ((ny + 7) / 8) * ((nz + zc - 1) / zc);
+}
+// Planes per CTA: 16 where that gives 8 CTAs per SM (the march is bound by
+// latency), else 8 or 4 (each chunk reads 4 more planes of dilated bytes).
+static int sign_zchunk(int nx, int ny, int nz, int v) {
+    int zc = SZ;
+    while (zc > 4 && sign_ctas(nx, ny, nz, v, zc) < (size_t)8 * sm_count()) zc /= 2;
+    return zc;
+}
+size_t sign_partial_rows(int nx, int ny, int nz) {
+    return std::max(sign_ctas(nx, ny, nz, 1, sign_zchunk(nx, ny, nz, 1)),
+                    sign_ctas(nx, ny, nz, 4, sign_zchunk(nx, ny, nz, 4)));
+}
+
+template <typename IT>
+static void sign_sums_t(const void *T0, const uint8_t *sbits, int k, int nx, int ny, int nz, uint8_t *dxy,
+                        double *partial, double *sums, cudaStream_t s) {
+    // four voxels per thread: mask bytes as 32-bit words
+    const bool quad = nx % 4 == 0 && (reinterpret_cast<uintptr_t>(sbits) & 3u) == 0;
+    const int v = quad ? 4 : 1, zc = sign_zchunk(nx, ny, nz, v);
+    const unsigned g = (unsigned)sign_ctas(nx, ny, nz, v, zc);
+    const dim3 block(32, 8);
+    const IT *t0 = static_cast<const IT *>(T0);
+    if (quad) {
+        k_dilate_xy<4><<<(unsigned)sign_ctas(nx, ny, nz, 4, 1), block, 0, s>>>(sbits, nx, ny, dxy);
+        k_sign_sums<IT, 4><<<g, block, 0, s>>>(t0, sbits, dxy, k, nx, ny, nz, zc, partial);
+    } else {
+        k_dilate_xy<1><<<(unsigned)sign_ctas(nx, ny, nz, 1, 1), block, 0, s>>>(sbits, nx, ny, dxy);
+        k_sign_sums<IT, 1><<<g, block, 0, s>>>(t0, sbits, dxy, k, nx, ny, nz, zc, partial);
+    }
+    k_sum_rows<<<4 * k, 256, 0, s>>>(partial, (int)g, 4 * k, sums);
     note_launch(3);
-    const unsigned gp = flat_grid(N, 152 * 4);
-    for (int j = 0; j < k; ++j) {
-        if (dtype == CGDIR_F16)
-            k_sign_partial<__half><<<gp, ST, 0, s>>>((const __half *)T0, sbits, tmp_a, j, N, partial);
-        else if (dtype == CGDIR_BF16)
-            k_sign_partial<__nv_bfloat16><<<gp, ST, 0, s>>>((const __nv_bfloat16 *)T0, sbits, tmp_a, j, N, partial);
-        else
-            k_sign_partial<float><<<gp, ST, 0, s>>>((const float *)T0, sbits, tmp_a, j, N, partial);
-        note_launch();
-        k_sum_rows4<<<1, 32, 0, s>>>(partial, (int)gp, sums + 4 * j); note_launch();
-    }
-    return cudaGetLastError();
 }
 
-size_t sign_partial_rows(size_t n) { return flat_grid(n, 152 * 4); }
+// sums: device [k][4]; dxy: N bytes, 4-byte aligned; partial: sign_partial_rows x k x 4 doubles.
+cudaError_t launch_sign_sums(const void *T0, int dtype, const uint8_t *sbits, int k, int nx, int ny, int nz,
+                             uint8_t *dxy, double *partial, double *sums, cudaStream_t s) {
+    if (dtype == CGDIR_F16) sign_sums_t<__half>(T0, sbits, k, nx, ny, nz, dxy, partial, sums, s);
+    else if (dtype == CGDIR_BF16) sign_sums_t<__nv_bfloat16>(T0, sbits, k, nx, ny, nz, dxy, partial, sums, s);
+    else sign_sums_t<float>(T0, sbits, k, nx, ny, nz, dxy, partial, sums, s);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_make_texels(const void *I0, int dtype, const uint8_t *bits, size_t n, void *tex,
                                cudaStream_t s) {

@@ -188,7 +188,7 @@ int plan_make(cgdir_ctx *ctx, const cgdir_volume *S, const cgdir_volume *M, cons
     pl.need[RegPlan::B_FIELDS] = 4 * 3 * Nf * sizeof(float);
     pl.need[RegPlan::B_PARTIAL] = std::max<size_t>(np * kPartialStride * sizeof(double), 256);
     pl.need[RegPlan::B_STATE] = pl.state_bytes;
-    pl.need[RegPlan::B_ROWDIST] = std::max<size_t>(uroi_scratch_bytes(Nf), 256);
+    pl.need[RegPlan::B_ROWDIST] = std::max<size_t>(uroi_scratch_bytes(nx, ny, nz), 256);
     const bool need_stage = (S->where == CGDIR_HOST && S->dtype != pl.sdt) ||
                             (M->where == CGDIR_HOST && M->dtype != pl.sdt) ||
                             (k > 0 && (SM->where == CGDIR_HOST || MM->where == CGDIR_HOST));
@@ -277,7 +277,7 @@ int plan_prepare(cgdir_ctx *ctx, Slot &sl, RegPlan &pl, cudaStream_t s) {
     for (int j = 0; j < k; ++j) need_auto |= pl.sign[j] == 0;
     if (need_auto) {
         int8_t autos[kMaxMasks];
-        CK(cudaStreamSynchronize(s));
+        if (s != ctx->stream) CK(cudaStreamSynchronize(s));     // the sums run on the context's stream
         TRY(auto_sign_impl(ctx, pl.T[L - 1], pl.sdt, pl.SB[L - 1], k, pl.nx, pl.ny, pl.nz, autos));
         for (int j = 0; j < k; ++j)
             if (pl.sign[j] == 0) pl.sign[j] = autos[j];

@@ -583,7 +583,7 @@ int cgdir_uroi(cgdir_ctx *ctx, const uint8_t *sbits, int k, int nx, int ny, int 
         return fail(ctx, CGDIR_EINVAL, "uroi: bad arguments");
     DeviceGuard g(ctx->device);
     void *rd = nullptr;
-    TRY(ws_get(ctx, "rowdist", uroi_scratch_bytes((size_t)nx * ny * nz), &rd));
+    TRY(ws_get(ctx, "rowdist", uroi_scratch_bytes(nx, ny, nz), &rd));
     const double sp1[3] = {1, 1, 1};
     cudaError_t e = launch_uroi(sbits, k, nx, ny, nz, spacing ? spacing : sp1, margin, (uint8_t *)rd, out,
                                 ctx->stream);
@@ -602,14 +602,12 @@ int cgdir::rt::auto_sign_impl(cgdir_ctx *ctx, const void *T0, int dtype, const u
         return fail(ctx, CGDIR_EINVAL, "auto_sign: bad arguments");
     if (k == 0) return CGDIR_OK;
     DeviceGuard g(ctx->device);
-    const size_t N = (size_t)nx * ny * nz;
-    void *ta = nullptr, *tb = nullptr, *part = nullptr, *sums = nullptr;
-    TRY(ws_get(ctx, "sign_a", N, &ta));
-    TRY(ws_get(ctx, "sign_b", N, &tb));
-    TRY(ws_get(ctx, "sign_part", sign_partial_rows(N) * 4 * sizeof(double), &part));
+    void *dxy = nullptr, *part = nullptr, *sums = nullptr;
+    TRY(ws_get(ctx, "sign_dxy", (size_t)nx * ny * nz, &dxy));
+    TRY(ws_get(ctx, "sign_part", sign_partial_rows(nx, ny, nz) * k * 4 * sizeof(double), &part));
     TRY(ws_get(ctx, "sign_sums", kMaxMasks * 4 * sizeof(double), &sums));
-    CK(launch_sign_sums(T0, dtype, sbits, k, nx, ny, nz, (uint8_t *)ta, (uint8_t *)tb, (double *)part,
-                        (double *)sums, ctx->stream));
+    CK(launch_sign_sums(T0, dtype, sbits, k, nx, ny, nz, (uint8_t *)dxy, (double *)part, (double *)sums,
+                        ctx->stream));
     double h[kMaxMasks * 4];
     CK(cudaMemcpyAsync(h, sums, k * 4 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
