@@ -8,7 +8,8 @@
 //              update kernel), the 3-D shared-memory tile kernel (idem), and
 //              the split xy + z kernels with the update fused into the z pass;
 //   force:     the stencil pass with the default z chunk, half, a quarter
-//              and double;
+//              and double, at four, two and (structure terms) one voxels per
+//              thread;
 // then the fused schedule (force stencil pass alone, 3-D tiles of G(du)
 // with the update, 3-D tiles of G(u') with the next iteration's warp)
 // against the best of those two, summed.
@@ -75,7 +76,9 @@ static const TunedLevel *find_tuned(const cgdir_ctx *ctx, int nx, int ny, int nz
     return it == ctx->tuned.end() ? nullptr : &it->second;
 }
 
-SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt, bool allow_fused) {
+// sigma: the larger Gaussian width of the level.
+SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt, bool allow_fused,
+                           float sigma) {
     SmoothChoice ch;
     // registrations that share the GPU (batched, served) cap the z-march's
     // CTAs per SM: uncapped they fill an SM's registers and starve the other
@@ -89,6 +92,12 @@ SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int con
     if (const TunedLevel *t = find_tuned(ctx, nx, ny, nz, contour, sdt)) {
         ch.variant = t->fused && allow_fused ? SMOOTH_FUSED : t->smooth_variant;
         ch.zchunk = t->fused && allow_fused ? 0 : t->smooth_zchunk;
+    } else if (allow_fused && nx % 4 == 0 && gauss_radius(sigma) <= 3 && (size_t)nx * ny * nz <= 350000) {
+        // untuned small levels: three kernels per iteration instead of five
+        // (per iteration: 32x32x16 19.8 against 23.9 us, 64x64x32 23.8 against
+        // 27.6, 120x80x35 33.6 against 35.3; 96x96x48 is past the line, 37.5
+        // against 35.7; without TMA, nx % 4 != 0, 58.8 against 48.3)
+        ch.variant = SMOOTH_FUSED;
     }
     return ch;
 }
@@ -103,7 +112,8 @@ bool use_level_coop(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, i
 int force_width_for(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt) {
     if (ctx->force_width > 0) return ctx->force_width;
     if (const TunedLevel *t = find_tuned(ctx, nx, ny, nz, contour, sdt)) return t->force_width;
-    return 0;
+    if (ctx->force_zchunk > 0) return 0;
+    return force_default_shape(nx, ny, nz, contour != 0).width;
 }
 
 // Never below force_zchunk_min: the registration's partial-sum buffer is
@@ -113,7 +123,20 @@ int force_zchunk_for(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, 
     if (ctx->force_zchunk > 0) return std::max(lo, std::min(ctx->force_zchunk, nz));
     if (const TunedLevel *t = find_tuned(ctx, nx, ny, nz, contour, sdt))
         if (t->force_zchunk > 0) return std::max(lo, std::min(t->force_zchunk, nz));
-    return force_default_zchunk(nx, ny, nz);
+    if (ctx->force_width > 0) return force_default_zchunk(nx, ny, nz);
+    return std::max(lo, force_default_shape(nx, ny, nz, contour != 0).zchunk);
+}
+
+// Pass 2's z chunk (returned) and its width and chains (in a) for a level.
+int force_schedule(const cgdir_ctx *ctx, ForceArgs &a, int sdt) {
+    const int contour = a.contour && a.k > 0;
+    const bool dflt = ctx->force_width == 0 && ctx->force_zchunk == 0 &&
+                      find_tuned(ctx, a.nx, a.ny, a.nz, contour, sdt) == nullptr;
+    const ForceShape f = force_default_shape(a.nx, a.ny, a.nz, contour != 0);
+    a.pass2_width = force_width_for(ctx, a.nx, a.ny, a.nz, contour, sdt);
+    a.chain_w = dflt ? f.chain_w : 0;
+    a.chain_z = dflt ? f.chain_z : 0;
+    return force_zchunk_for(ctx, a.nx, a.ny, a.nz, contour, sdt);
 }
 
 // Average time of `reps` launches of `body` after two untimed ones (ms).
@@ -193,11 +216,20 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
     {
         const int d = force_default_zchunk(nx, ny, nz);
         const int cand[4] = {d, std::max(1, d / 2), std::max(1, d / 4), std::min(nz, 2 * d)};
-        // the stencil pass's width: four voxels per thread (the default where
-        // nx % 4 == 0) or two (twice the CTAs, for small levels)
-        const int widths[2] = {0, 2};
-        const int nw = (nx % 4 == 0 && ctx->force_width == 0) ? 2 : 1;
+        // the stencil pass's width: four voxels per thread (the widest where
+        // nx % 4 == 0), two or, with structure terms, one (more threads, for
+        // small levels)
+        const int widths[3] = {0, 2, 1};
+        const int nw = nx % 4 == 0 && ctx->force_width == 0 ? (contour ? 3 : 2) : 1;
         float bt = 1e30f;
+        // the untuned choice
+        rc = time_ms(ctx, e0, e1, reps, &bt, [&](cudaStream_t st) {
+            ForceArgs b = a;
+            const int zc = force_schedule(ctx, b, -1);
+            return launch_force(b, zc, nullptr, st, kerr(ctx));
+        });
+        best.default_force_ms = bt;
+        bt = 1e30f;
         for (int wi = 0; wi < nw && rc == CGDIR_OK; ++wi) {
             a.pass2_width = ctx->force_width > 0 ? ctx->force_width : widths[wi];
             for (int ci = 0; ci < 4 && rc == CGDIR_OK; ++ci) {
@@ -207,14 +239,22 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 float ms = 0.f;
                 rc = time_ms(ctx, e0, e1, reps, &ms,
                              [&](cudaStream_t st) { return launch_force(a, cand[ci], nullptr, st, kerr(ctx)); });
-                if (wi == 0 && ci == 0) best.default_force_ms = ms;
-                if (rc == CGDIR_OK && ms < bt) {
+                // within the noise of these timings the wider thread and the
+                // longer chunk (fewer CTAs and halo planes) stand
+                const float slack = wi > 0 && best.force_width != widths[wi] ? 0.97f
+                                    : cand[ci] > best.force_zchunk ? 1.03f : 0.97f;
+                if (rc == CGDIR_OK && ms < slack * bt) {
                     bt = ms;
                     best.force_zchunk = cand[ci];
                     best.force_width = widths[wi];
                     best.force_ms = ms;
                 }
             }
+        }
+        if (rc == CGDIR_OK && best.default_force_ms <= best.force_ms) {       // nothing beat the untuned choice
+            best.force_zchunk = force_zchunk_for(ctx, nx, ny, nz, contour, -1);
+            best.force_width = ctx->force_width > 0 ? 0 : force_width_for(ctx, nx, ny, nz, contour, -1);
+            best.force_ms = best.default_force_ms;
         }
         a.pass2_width = ctx->force_width > 0 ? ctx->force_width : best.force_width;
     }
@@ -280,6 +320,10 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 return launch_fused_smooth_warp(out, sigma, u, a2, kerr(ctx), st);
             });
         fs = std::max(fs - f2, 0.f);
+        if (rc == CGDIR_OK && smooth_choice(ctx, nx, ny, nz, contour, -1, true, sigma).variant == SMOOTH_FUSED) {
+            best.default_smooth_ms = fs;                   // the untuned choice is the fused schedule
+            best.default_force_ms = f2;
+        }
         if (rc == CGDIR_OK && f2 + fs < best.force_ms + best.smooth_ms) {
             best.fused = 1;
             best.fused_smooth_ms = fs;

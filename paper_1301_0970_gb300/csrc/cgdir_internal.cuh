@@ -53,8 +53,9 @@ struct Taps {
 int gauss_radius(float sigma);
 Taps gauss_taps(float sigma);
 
-// Per-block partial sums of the stopping metric: {sum (I0~ - T0)^2 over the
-// UROI, UROI count, max |du|}, FP64, written by the force / metric kernels.
+// Per-block partial sums of the stopping metric (sum (I0~ - T0)^2 over the
+// UROI, UROI count, max |du|), written by the force / metric kernels: rows of
+// this many doubles (Partial in kernels_force.cu).
 constexpr int kPartialStride = 4;
 
 // Device-side state of one level's stopping logic, updated by the reduction.
@@ -105,6 +106,11 @@ struct ForceArgs {
     float *pfield;
     int pass2_width;              // voxels per thread in pass 2: 1 or 2 (at most), 0 = the
                                   // widest the shape and the fields' alignment allow
+    // The FP32 chains of the RMS-ID sums, where they are not a thread's own
+    // columns over its z chunk (0): chain_w = 4: one chain per quad of
+    // x-adjacent voxels (nx % 4 == 0) and chain_z planes; chain_w = 0, chain_z >
+    // 0: a thread's own columns over chain_z planes each
+    int chain_w, chain_z;
     int skip_warp;                // 1: pass 1's outputs are already current for u (the fused
                                   // smoothing + warp kernel wrote them): launch pass 2 only
 };
@@ -149,6 +155,12 @@ inline void force_scratch_assign(ForceArgs &a, void *scratch, size_t n) {
     a.pfield = reinterpret_cast<float *>(p + ((n * 4 + 255) / 256) * 256 + ((n * 2 + 255) / 256) * 256);
 }
 
+// The stop flag of a level (false without one).  Where registers allow, a
+// kernel of an iteration reads it first and acts on it only after its first
+// loads have been issued: the flag's own latency (0.4 us from L2, on every
+// launch) overlaps theirs.
+__device__ __forceinline__ bool stopped(const int *flag) { return flag != nullptr && *flag != 0; }
+
 // Process-wide count of kernels launched by this library (instrumentation).
 void note_launch(unsigned n = 1);
 
@@ -167,6 +179,11 @@ cudaError_t launch_force(const ForceArgs &a, int zchunk, int *nblocks_out, cudaS
                          int *err = nullptr);
 size_t force_partial_count(int nx, int ny, int nz, int zchunk);
 int force_default_zchunk(int nx, int ny, int nz);
+// The untuned schedule of pass 2 and the chains of its sums.
+struct ForceShape {
+    int zchunk, width, chain_w, chain_z;
+};
+ForceShape force_default_shape(int nx, int ny, int nz, bool contour);
 cudaError_t launch_metric(const void *I0, const void *T0, int img_dtype, const float *u,
                           const uint8_t *uroi, int nx, int ny, int nz, double *partial,
                           const int *stop_flag, int *nblocks_out, cudaStream_t s,

@@ -50,47 +50,73 @@ __device__ __forceinline__ float warp_max(float v) {
     return v;
 }
 
-// Block reduction of (ssd, count, max) into partial[bid].  Each thread's
-// SSD covers only its own column of a z-chunk (a few dozen non-negative
-// terms) and is kept in FP32; it enters the block sum as an exact
-// fixed-point integer (units of 2^-12 HU^2), so the in-block sum is exact
-// and independent of order and needs no FP64 arithmetic (slow on this
-// GPU).  The block total is exactly representable in FP64 and the
-// cross-block sum (finalize_block) is FP64.
+// Block reduction of (ssd, count, max) into partial[bid].  A chain of the SSD
+// (one thread's column of a z chunk: a few dozen non-negative terms) is kept
+// in FP32; it enters the block sum as an exact fixed-point integer (units of
+// 2^-12 HU^2), so the in-block sum is exact and independent of order and
+// needs no FP64 arithmetic (slow on this GPU).  The cross-block sum
+// (finalize_block) is exact too.
 constexpr float kSsdScale = 4096.f;
 
+// One thread's finished chains.  Beyond 2^40 HU^2 a chain could overflow the
+// fixed-point block sum (256 threads of at most 8 chains): such a chain (never
+// met by CT-range images) is summed in FP64 instead.
+struct ChainSum {
+    unsigned long long q = 0;
+    double wide = 0.0;
+    __device__ __forceinline__ void add(float ssd) {
+        if (ssd <= 1.0995e12f) q += __float2ull_rn(ssd * kSsdScale);
+        else wide += (double)ssd;                  // NaN as well
+    }
+};
+
+// One CTA's partial sums (a row of kPartialStride doubles).
+struct alignas(16) Partial {
+    unsigned long long q;
+    double wide;
+    unsigned cnt, is_wide;
+    float mx, pad;
+};
+static_assert(sizeof(Partial) == kPartialStride * sizeof(double), "row of the partial buffer");
+
 template <int NTHREADS>
-__device__ void block_partial(float ssd_f, int cnt_i, float mx, double *partial, int bid) {
+__device__ void block_partial(const ChainSum &c, int cnt_i, float mx, double *partial, int bid) {
     __shared__ unsigned long long rs[NTHREADS / 32];
     __shared__ double rd[NTHREADS / 32];
     __shared__ int rc[NTHREADS / 32];
     __shared__ float rm[NTHREADS / 32];
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-    // beyond 2^40 HU^2 per thread the fixed-point block sum could overflow:
-    // such a block (never met by CT-range images) sums in FP64 instead
-    const bool wide = __syncthreads_or(!(ssd_f <= 1.0995e12f));
-    unsigned long long q = wide ? 0ull : __float2ull_rn(ssd_f * kSsdScale);
-    double d = wide ? (double)ssd_f : 0.0;
+    const bool wide = __syncthreads_or(!(c.wide == 0.0));
+    unsigned long long q = c.q;
+    double d = c.wide;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
+        q += __shfl_xor_sync(0xffffffffu, q, o);
         if (wide) d += __shfl_xor_sync(0xffffffffu, d, o);
-        else q += __shfl_xor_sync(0xffffffffu, q, o);
-        cnt_i += __shfl_xor_sync(0xffffffffu, cnt_i, o);
     }
+    cnt_i = __reduce_add_sync(0xffffffffu, cnt_i);
     mx = warp_max(mx);
     if ((tid & 31) == 0) { rs[tid >> 5] = q; rd[tid >> 5] = d; rc[tid >> 5] = cnt_i; rm[tid >> 5] = mx; }
     __syncthreads();
     if (tid == 0) {
-        unsigned long long s = 0;
-        double sd = 0.0;
-        long long c = 0;
-        float m = 0.f;
-        for (int w = 0; w < NTHREADS / 32; ++w) { s += rs[w]; sd += rd[w]; c += rc[w]; m = fmaxf(m, rm[w]); }
-        partial[(size_t)bid * kPartialStride + 0] = wide ? sd : (double)s * (1.0 / (double)kSsdScale);
-        partial[(size_t)bid * kPartialStride + 1] = (double)c;
-        partial[(size_t)bid * kPartialStride + 2] = (double)m;
-        partial[(size_t)bid * kPartialStride + 3] = 0.0;
+        Partial p{};
+        for (int w = 0; w < NTHREADS / 32; ++w) {
+            p.q += rs[w];
+            p.cnt += (unsigned)rc[w];
+            p.mx = fmaxf(p.mx, rm[w]);
+        }
+        if (wide) {
+            p.is_wide = 1u;
+            for (int w = 0; w < NTHREADS / 32; ++w) p.wide += rd[w];
+        }
+        reinterpret_cast<Partial *>(partial)[bid] = p;
     }
+}
+template <int NTHREADS>
+__device__ __forceinline__ void block_partial(float ssd, int cnt_i, float mx, double *partial, int bid) {
+    ChainSum c;
+    c.add(ssd);
+    block_partial<NTHREADS>(c, cnt_i, mx, partial, bid);
 }
 
 // Stopping test of Sec. 2.2 on delta^n = dn and the earlier deltas it needs
@@ -115,48 +141,74 @@ __device__ int stop_test(double dn, const PastDeltas &p, int n, int mode, double
     return 0;
 }
 
-// Fixed-order sum of the per-CTA partials, RMS-ID into the level history and
-// the stop decision (kernel 5).  Run by one whole CTA (any shape, blockDim a
-// multiple of 32, at most 1024 threads): each thread sums a fixed stride of
-// partials, then warp shuffles and warp 0 combine them in a fixed order.
-__device__ void finalize_block(const double *__restrict__ partial, int nblocks, const FinishArgs &f) {
-    __shared__ double ws[32], wc[32], wm[32];
+// Sum of the per-CTA partials, RMS-ID into the level history and the stop
+// decision (kernel 5).  Run by one whole CTA (any shape, blockDim a multiple
+// of 32, at most 1024 threads).  The fixed-point sums are added as integers
+// (32-bit halves apart, so no total overflows), exactly and in any order; FP64
+// adds, which take a warp 14 cycles of the SM here and would sit on the
+// iteration's critical path, are left to wide blocks (fixed order: a fixed
+// stride per thread, then lanes, then warps) and to the final quotient.
+__device__ __forceinline__ void finalize_block(const double *__restrict__ partial, int nblocks, const FinishArgs &f) {
+    __shared__ unsigned long long wl[32], wh[32], wc[32];
+    __shared__ double ww[32];
+    __shared__ float wm[32];
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     const int nt = blockDim.x * blockDim.y;
-    double s = 0.0, c = 0.0, m = 0.0;
+    unsigned long long lo = 0, hi = 0, c = 0;
+    double w = 0.0;
+    float m = 0.f;
+    unsigned any_wide = 0;
     // the earlier deltas of the stop test, read now so their latency overlaps the sums
     PastDeltas past{0.0, 0.0, 0.0};
     if (tid == 0 && f.st.hist) past = past_deltas(f.st.hist, f.n, f.stop_mode);
-    // four partials in flight per thread, summed in the same (ascending) order
+    const int4 *rows = reinterpret_cast<const int4 *>(partial);
+    auto add = [&](const int4 &x, const int4 &y) {
+        lo += (unsigned)x.x;
+        hi += (unsigned)x.y;
+        c += (unsigned)y.x;
+        if (y.y) { any_wide = 1u; w += __hiloint2double(x.w, x.z); }
+        m = fmaxf(m, __int_as_float(y.z));
+    };
+    // four partials in flight per thread
     constexpr int U = 4;
     int b = tid;
     for (; b + (U - 1) * nt < nblocks; b += U * nt) {
-        double3 v[U];
+        int4 x[U], y[U];
 #pragma unroll
         for (int q = 0; q < U; ++q) {
-            const double *p = partial + (size_t)(b + q * nt) * kPartialStride;
-            v[q] = make_double3(__ldcg(p), __ldcg(p + 1), __ldcg(p + 2));
+            x[q] = __ldcg(rows + 2 * (size_t)(b + q * nt));
+            y[q] = __ldcg(rows + 2 * (size_t)(b + q * nt) + 1);
         }
 #pragma unroll
-        for (int q = 0; q < U; ++q) { s += v[q].x; c += v[q].y; m = fmax(m, v[q].z); }
+        for (int q = 0; q < U; ++q) add(x[q], y[q]);
     }
-    for (; b < nblocks; b += nt) {
-        s += __ldcg(partial + (size_t)b * kPartialStride + 0);
-        c += __ldcg(partial + (size_t)b * kPartialStride + 1);
-        m = fmax(m, __ldcg(partial + (size_t)b * kPartialStride + 2));
-    }
+    for (; b < nblocks; b += nt) add(__ldcg(rows + 2 * (size_t)b), __ldcg(rows + 2 * (size_t)b + 1));
+    any_wide = __syncthreads_or(any_wide);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
+        lo += __shfl_xor_sync(0xffffffffu, lo, o);
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
         c += __shfl_xor_sync(0xffffffffu, c, o);
-        m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (any_wide) w += __shfl_xor_sync(0xffffffffu, w, o);
     }
-    if ((tid & 31) == 0) { ws[tid >> 5] = s; wc[tid >> 5] = c; wm[tid >> 5] = m; }
+    m = warp_max(m);
+    if ((tid & 31) == 0) { wl[tid >> 5] = lo; wh[tid >> 5] = hi; wc[tid >> 5] = c; ww[tid >> 5] = w; wm[tid >> 5] = m; }
     __syncthreads();
     if (tid == 0) {
-        double S = 0.0, C = 0.0, M = 0.0;
-        for (int w = 0; w < nt / 32; ++w) { S += ws[w]; C += wc[w]; M = fmax(M, wm[w]); }
-        if (f.stats_out) { f.stats_out[0] = S; f.stats_out[1] = C; f.stats_out[2] = M; }
+        lo = hi = c = 0;
+        w = 0.0;
+        m = 0.f;
+        for (int q = 0; q < nt / 32; ++q) {
+            lo += wl[q];
+            hi += wh[q];
+            c += wc[q];
+            if (any_wide) w += ww[q];
+            m = fmaxf(m, wm[q]);
+        }
+        hi += lo >> 32;                                    // units of 2^32 steps of 1 / kSsdScale
+        const double S = ((double)hi * 4294967296.0 + (double)(lo & 0xffffffffull)) * (1.0 / (double)kSsdScale) + w;
+        const double C = (double)c;
+        if (f.stats_out) { f.stats_out[0] = S; f.stats_out[1] = C; f.stats_out[2] = (double)m; }
         const LevelState &st = f.st;
         if (st.hist) {
             const double d = C > 0 ? sqrt(S / C) : 0.0;
@@ -171,8 +223,14 @@ __device__ void finalize_block(const double *__restrict__ partial, int nblocks, 
     }
 }
 
+// The same as a call, for kernels whose registers it would overflow.
+__device__ __noinline__ void finalize_call(const double *__restrict__ partial, int nblocks, const FinishArgs &f) {
+    finalize_block(partial, nblocks, f);
+}
+
 // Called by every CTA after its partial is written: the CTA that completes
 // the grid runs finalize_block and resets the counter for the next launch.
+template <bool CALL = false>
 __device__ void finish_if_last(const double *partial, int nblocks, const FinishArgs &f) {
     __shared__ int last;
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
@@ -183,7 +241,8 @@ __device__ void finish_if_last(const double *partial, int nblocks, const FinishA
     __syncthreads();
     if (last) {
         __threadfence();
-        finalize_block(partial, nblocks, f);
+        if (CALL) finalize_call(partial, nblocks, f);
+        else finalize_block(partial, nblocks, f);
         if (tid == 0) *f.done = 0u;
     }
 }
@@ -343,7 +402,7 @@ __global__ void __launch_bounds__(NT) k_force(ForceArgs a, int zchunk) {
 // texels and image + bits at each plane cost all of that gain.
 template <bool CONTOUR, typename IT>
 __global__ void __launch_bounds__(NT, 5) k_warp_pass(ForceArgs a, int zw) {
-    if (a.stop_flag && *a.stop_flag) return;
+    const bool stop = stopped(a.stop_flag);
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int x = blockIdx.x * TX + threadIdx.x, y = blockIdx.y * TY + threadIdx.y;
     if (x >= nx || y >= ny) return;
@@ -359,6 +418,7 @@ __global__ void __launch_bounds__(NT, 5) k_warp_pass(ForceArgs a, int zw) {
     float ax = 0.f, ay = 0.f, az = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
     if (zb < ze) disp(zb, ax, ay, az);
     if (zb + 1 < ze) disp(zb + 1, bx, by, bz);
+    if (stop) return;
     CornerQuad<IT> A = {}, B = {};
     int held = -1, z = zb;             // low corner of the plane whose corners `lo` holds (-1: none)
     auto step = [&](CornerQuad<IT> &lo, CornerQuad<IT> &hi, float &ux, float &uy, float &uz) {
@@ -548,9 +608,45 @@ __device__ __forceinline__ void plane_load(const ForceArgs &a, int ic, int ip, i
     }
 }
 
+// The chain of the RMS-ID sums over the quad x .. x + 3 and the planes from z
+// on (chain_z of them at most), as the four-voxel pass runs it.  Every load is
+// issued at once.
+template <typename IT>
+__device__ __forceinline__ float chain_quad(const ForceArgs &a, int x, int y, int z) {
+    constexpr int U = 4;
+    const int nxy = a.nx * a.ny, i0 = z * nxy + y * a.nx + x, n = min(a.chain_z, a.nz - z);
+    float ssd = 0.f;
+    for (int p0 = 0; p0 < n; p0 += U) {
+        float4 w[U], t[U];
+        uint2 t16[U];
+        unsigned ur[U];
+#pragma unroll
+        for (int p = 0; p < U; ++p) {
+            if (p0 + p >= n) continue;
+            const int i = i0 + (p0 + p) * nxy;
+            w[p] = __ldg(reinterpret_cast<const float4 *>(a.wfield + i));
+            if (sizeof(IT) == 2) t16[p] = __ldg(reinterpret_cast<const uint2 *>(static_cast<const IT *>(a.T0) + i));
+            else t[p] = __ldg(reinterpret_cast<const float4 *>(static_cast<const float *>(a.T0) + i));
+            ur[p] = a.uroi ? __ldg(reinterpret_cast<const unsigned *>(a.uroi + i)) : 0x01010101u;
+        }
+#pragma unroll
+        for (int p = 0; p < U; ++p) {
+            if (p0 + p >= n) continue;
+            if (sizeof(IT) == 2)
+                t[p] = make_float4(t_of<IT>(t16[p].x & 0xffffu), t_of<IT>(t16[p].x >> 16),
+                                   t_of<IT>(t16[p].y & 0xffffu), t_of<IT>(t16[p].y >> 16));
+            const float r[4] = {t[p].x - w[p].x, t[p].y - w[p].y, t[p].z - w[p].z, t[p].w - w[p].w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if ((ur[p] >> (8 * q)) & 0xffu) ssd = fmaf(r[q], r[q], ssd);
+        }
+    }
+    return ssd;
+}
+
 template <bool CONTOUR, typename IT, bool MAXDU>
 __global__ void __launch_bounds__(NT, 3) k_force_pass(ForceArgs a, int zchunk) {
-    if (a.stop_flag && *a.stop_flag) return;
+    if (stopped(a.stop_flag)) return;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int x = blockIdx.x * TX + threadIdx.x, y = blockIdx.y * TY + threadIdx.y;
     const int nxy = nx * ny, N = nxy * nz;
@@ -562,6 +658,7 @@ __global__ void __launch_bounds__(NT, 3) k_force_pass(ForceArgs a, int zchunk) {
         build_tables(a, tab, threadIdx.y * TX + threadIdx.x);
         __syncthreads();
     }
+    ChainSum sum;
     if (x < nx && y < ny) {
         float *__restrict__ du = a.du;
         const int col = y * nx + x;
@@ -574,6 +671,9 @@ __global__ void __launch_bounds__(NT, 3) k_force_pass(ForceArgs a, int zchunk) {
         if (CONTOUR) { Sm = __ldg(a.wstate + im); Sc = __ldg(a.wstate + ic); }
         PlaneLoads<CONTOUR, IT> bufA, bufB;
         plane_load<CONTOUR, IT>(a, ic, zb < nz - 1 ? ic + nxy : ic, oxm, oxp, oym, oyp, bufA);
+        if (a.partial && a.chain_w == 4 && (x & 3) == 0)      // the chains that start here
+            for (int zc = (zb + a.chain_z - 1) / a.chain_z * a.chain_z; zc < ze; zc += a.chain_z)
+                sum.add(chain_quad<IT>(a, x, y, zc));
         int z = zb;
         // one plane: consumes `cur`, prefetches the next plane into `nxt`
         auto step = [&](const PlaneLoads<CONTOUR, IT> &cur, PlaneLoads<CONTOUR, IT> &nxt) {
@@ -591,10 +691,9 @@ __global__ void __launch_bounds__(NT, 3) k_force_pass(ForceArgs a, int zchunk) {
             du[ic] = dux;
             du[N + ic] = duy;
             du[N + N + ic] = duz;
-            if (cur.ur) {
-                ssd = fmaf(r0, r0, ssd);
-                cnt += 1;
-            }
+            cnt += cur.ur ? 1 : 0;
+            if (cur.ur) ssd = fmaf(r0, r0, ssd);
+            if (a.chain_w == 0 && a.chain_z > 0 && (z + 1) % a.chain_z == 0) { sum.add(ssd); ssd = 0.f; }
             if (MAXDU) mx = fmaxf(mx, dux * dux + duy * duy + duz * duz);
             Wm = Wc; Wc = Wp; im = ic;
             if (CONTOUR) { Sm = Sc; Sc = Sp; }
@@ -607,11 +706,12 @@ __global__ void __launch_bounds__(NT, 3) k_force_pass(ForceArgs a, int zchunk) {
             step(bufB, bufA);
         }
         if (z < ze) step(bufA, bufB);
+        if (a.chain_w == 0) sum.add(ssd);
     }
     if (a.partial) {
-        block_partial<NT>(ssd, cnt, sqrtf(mx), a.partial,
+        block_partial<NT>(sum, cnt, sqrtf(mx), a.partial,
                           (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
-        if (a.fin.done) finish_if_last(a.partial, gridDim.x * gridDim.y * gridDim.z, a.fin);
+        if (a.fin.done) finish_if_last<true>(a.partial, gridDim.x * gridDim.y * gridDim.z, a.fin);
     }
 }
 
@@ -675,7 +775,7 @@ __device__ __forceinline__ void plane_load2(const ForceArgs &a, int ic, int ip, 
 
 template <bool CONTOUR, typename IT, bool MAXDU>
 __global__ void __launch_bounds__(NT, 2) k_force_pass2(ForceArgs a, int zchunk) {
-    if (a.stop_flag && *a.stop_flag) return;
+    const bool stop = stopped(a.stop_flag);
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int x = 2 * (blockIdx.x * TX + threadIdx.x), y = blockIdx.y * TY + threadIdx.y;
     const int nxy = nx * ny, N = nxy * nz;
@@ -683,10 +783,10 @@ __global__ void __launch_bounds__(NT, 2) k_force_pass2(ForceArgs a, int zchunk) 
     float ssd = 0.f, mx = 0.f;
     int cnt = 0;
     __shared__ ContourTables tab;
-    if (CONTOUR) {
-        build_tables(a, tab, threadIdx.y * TX + threadIdx.x);
-        __syncthreads();
-    }
+    if (CONTOUR) build_tables(a, tab, threadIdx.y * TX + threadIdx.x);
+    if (stop) return;
+    if (CONTOUR) __syncthreads();
+    ChainSum sum;
     if (x < nx && y < ny) {
         float *__restrict__ du = a.du;
         const int col = y * nx + x;
@@ -703,6 +803,9 @@ __global__ void __launch_bounds__(NT, 2) k_force_pass2(ForceArgs a, int zchunk) 
         }
         PlaneLoads2 bufA, bufB;
         plane_load2<CONTOUR, IT>(a, ic, zb < nz - 1 ? ic + nxy : ic, oxm, oxp, oym, oyp, bufA);
+        if (a.partial && a.chain_w == 4 && (x & 3) == 0)      // the chains that start here
+            for (int zc = (zb + a.chain_z - 1) / a.chain_z * a.chain_z; zc < ze; zc += a.chain_z)
+                sum.add(chain_quad<IT>(a, x, y, zc));
         int z = zb;
         auto step = [&](const PlaneLoads2 &cur, PlaneLoads2 &nxt) {
             const int ip = z < nz - 1 ? ic + nxy : ic;
@@ -725,6 +828,7 @@ __global__ void __launch_bounds__(NT, 2) k_force_pass2(ForceArgs a, int zchunk) 
             *reinterpret_cast<float2 *>(du + N + N + ic) = make_float2(d0z, d1z);
             if (cur.ur & 0xffu) { ssd = fmaf(r00, r00, ssd); cnt += 1; }
             if (cur.ur >> 8) { ssd = fmaf(r01, r01, ssd); cnt += 1; }
+            if (a.chain_w == 0 && a.chain_z > 0 && (z + 1) % a.chain_z == 0) { sum.add(ssd); ssd = 0.f; }
             if (MAXDU) mx = fmaxf(mx, fmaxf(d0x * d0x + d0y * d0y + d0z * d0z, d1x * d1x + d1y * d1y + d1z * d1z));
             Wm = Wc; Wc = cur.wp; im = ic;
             Sm = Sc; Sc = cur.sp;
@@ -736,9 +840,10 @@ __global__ void __launch_bounds__(NT, 2) k_force_pass2(ForceArgs a, int zchunk) 
             step(bufB, bufA);
         }
         if (z < ze) step(bufA, bufB);
+        if (a.chain_w == 0) sum.add(ssd);
     }
     if (a.partial) {
-        block_partial<NT>(ssd, cnt, sqrtf(mx), a.partial,
+        block_partial<NT>(sum, cnt, sqrtf(mx), a.partial,
                           (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
         if (a.fin.done) finish_if_last(a.partial, gridDim.x * gridDim.y * gridDim.z, a.fin);
     }
@@ -816,7 +921,7 @@ __device__ __forceinline__ void pair_ao(unsigned c, unsigned l, unsigned r, unsi
 
 template <bool CONTOUR, typename IT, bool MAXDU>
 __global__ void __launch_bounds__(NT, 2) k_force_pass4(ForceArgs a, int zchunk) {
-    if (a.stop_flag && *a.stop_flag) return;
+    const bool stop = stopped(a.stop_flag);
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int x = 4 * (blockIdx.x * TX + threadIdx.x), y = blockIdx.y * TY + threadIdx.y;
     const int nxy = nx * ny, N = nxy * nz;
@@ -824,10 +929,9 @@ __global__ void __launch_bounds__(NT, 2) k_force_pass4(ForceArgs a, int zchunk) 
     float ssd = 0.f, mx = 0.f;
     int cnt = 0;
     __shared__ ContourTables tab;
-    if (CONTOUR) {
-        build_tables(a, tab, threadIdx.y * TX + threadIdx.x);
-        __syncthreads();
-    }
+    if (CONTOUR) build_tables(a, tab, threadIdx.y * TX + threadIdx.x);
+    if (stop) return;
+    if (CONTOUR) __syncthreads();
     if (x < nx && y < ny) {
         float *__restrict__ du = a.du;
         const int col = y * nx + x;
@@ -1403,7 +1507,7 @@ __device__ __forceinline__ void coords(size_t i, size_t N, int nx, int ny, int &
 // UROI's voxels, a few compact regions, spread evenly over the threads.
 constexpr int MT = 256;
 template <typename IT>
-__global__ void __launch_bounds__(MT) k_metric(const IT *__restrict__ I0,
+__global__ void __launch_bounds__(MT, 5) k_metric(const IT *__restrict__ I0,
                                                const IT *__restrict__ T0,
                                                const float *__restrict__ u,
                                                const uint8_t *__restrict__ uroi, int nx, int ny,
@@ -1480,6 +1584,38 @@ int force_default_zchunk(int nx, int ny, int nz) {
     return pick_zchunk(nz, (long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY), 4, 2);
 }
 
+// What pass 2 does that no tuning table or setting names.  The chains of the
+// RMS-ID sums are always those of the widest thread and the chunk above, so
+// the histories do not depend on the schedule, which differs from them on
+// small levels:
+//  * with structure terms a voxel at a structure border loads its P_j after
+//    its bits are known, once per voxel of the thread: one or two voxels per
+//    thread instead of four, and one plane on the smallest levels (per
+//    iteration, 3 structures: 64x64x24 26.7 against 33.5 us, 120x80x35 38.9
+//    against 43.8, 96x96x48 39.6 against 44.2, 128x128x64 63.0 against 63.8,
+//    160x160x48 71.6 against 74.1; 240x160x70 is past the line: 61.8 against
+//    53.6);
+//  * where nx % 4 != 0, several chains of fewer than 4 planes per thread
+//    (each CTA pays for its halo planes and partial sums: 95x71x34 43 against
+//    48 us per iteration).
+ForceShape force_default_shape(int nx, int ny, int nz, bool contour) {
+    const size_t N = (size_t)nx * ny * nz;
+    const int zc = force_default_zchunk(nx, ny, nz);
+    ForceShape f{zc, 0, 0, 0};
+    if (nx % 4 == 0) {
+        if (contour && N <= 1600000) {
+            f.width = N > 200000 && N <= 600000 ? 1 : 2;
+            f.zchunk = N <= 200000 ? 1 : std::min(4, nz);
+            f.chain_w = 4;
+            f.chain_z = zc;
+        }
+    } else if (zc < 4) {
+        f.zchunk = std::min((4 + zc - 1) / zc * zc, nz);      // 4 chains at most
+        f.chain_z = zc;
+    }
+    return f;
+}
+
 // z chunks of pass 1 of the two-pass force: short, so the grid is several
 // waves deep.
 static int two_pass_zchunk(int nx, int ny, int nz) {
@@ -1495,12 +1631,13 @@ size_t force_partial_count(int nx, int ny, int nz, int zchunk) {
 // (512x512x160, contour terms on: 525 against 548 us per force step with
 // FP32 images, 482 against 507 with FP16, from twice the bytes in flight per
 // thread at the same 2 CTAs per SM.)
-static bool pass2_quad(const ForceArgs &a) {
+static bool quad_aligned(const ForceArgs &a) {
     auto al = [](const void *p, unsigned b) { return p == nullptr || ((uintptr_t)p & (b - 1)) == 0; };
     const unsigned tb = a.img_dtype == CGDIR_F32 ? 16u : 8u;
-    return a.nx % 4 == 0 && a.pass2_width == 0 && al(a.wfield, 16) && al(a.wstate, 8) && al(a.T0, tb) &&
+    return a.nx % 4 == 0 && al(a.wfield, 16) && al(a.wstate, 8) && al(a.T0, tb) &&
            al(a.du, 16) && al(a.warped, 16) && al(a.uroi, 4) && al(a.sbits, 4);
 }
+static bool pass2_quad(const ForceArgs &a) { return a.pass2_width == 0 && quad_aligned(a); }
 
 template <typename IT>
 static cudaError_t launch_force_t(const ForceArgs &a, int zchunk, dim3 grid, dim3 block, cudaStream_t s,
@@ -1514,6 +1651,8 @@ static cudaError_t launch_force_t(const ForceArgs &a, int zchunk, dim3 grid, dim
         // end-of-block fences before the fused reduction
         const bool quad = pass2_quad(a);
         const bool paired = a.nx % 2 == 0 && a.pass2_width != 1;
+        ForceArgs b = a;
+        if (a.chain_w == 4 && (quad || !quad_aligned(a))) b.chain_w = b.chain_z = 0;      // the threads' own
         dim3 g2 = quad ? dim3((a.nx / 4 + TX - 1) / TX, grid.y, grid.z)
                        : paired ? dim3((a.nx / 2 + TX - 1) / TX, grid.y, grid.z) : grid;
         const bool warp = !a.skip_warp;
@@ -1522,9 +1661,9 @@ static cudaError_t launch_force_t(const ForceArgs &a, int zchunk, dim3 grid, dim
         const bool maxdu = a.partial != nullptr && (a.fin.done == nullptr || a.fin.stats_out != nullptr);
 #define CGDIR_PASS2(C, M)                                                        \
     do {                                                                         \
-        if (quad) k_force_pass4<C, IT, M><<<g2, block, 0, s>>>(a, zchunk);       \
-        else if (paired) k_force_pass2<C, IT, M><<<g2, block, 0, s>>>(a, zchunk);\
-        else k_force_pass<C, IT, M><<<grid, block, 0, s>>>(a, zchunk);           \
+        if (quad) k_force_pass4<C, IT, M><<<g2, block, 0, s>>>(b, zchunk);       \
+        else if (paired) k_force_pass2<C, IT, M><<<g2, block, 0, s>>>(b, zchunk);\
+        else k_force_pass<C, IT, M><<<grid, block, 0, s>>>(b, zchunk);           \
     } while (0)
         if (contour) {
             if (warp) k_warp_pass<true, IT><<<g, block, 0, s>>>(a, zc);

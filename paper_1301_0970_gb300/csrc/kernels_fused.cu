@@ -74,13 +74,14 @@ struct FusedTile {
 };
 
 // G(in) over the CTA's tile into Z (smem), all three components.  Returns
-// false (every thread) if the TMA wait ran out; the error word is then set.
+// false (every thread) if the level has stopped or the TMA wait ran out; the
+// error word is set in the second case.
 // With umap, the u tile's TMA copy (completing on bar[1]) is issued as soon
 // as the input box has been read.
 template <int R>
 __device__ __forceinline__ bool tile_smooth(const CUtensorMap *tin, bool use_tma, const float *__restrict__ in,
                                             const Taps &t, int nx, int ny, int nz, int x0, int y0, int z0,
-                                            float *S, float *X, uint64_t *bar, int *err, int tid,
+                                            float *S, float *X, uint64_t *bar, int *err, int tid, bool stop,
                                             const CUtensorMap *umap = nullptr) {
     using G = FusedTile<R>;
     constexpr int K = 2 * R + 1, A = G::A, ML = G::ML, W = G::W, XS = G::XS, XP = G::XP, YP = G::YP;
@@ -97,6 +98,7 @@ __device__ __forceinline__ bool tile_smooth(const CUtensorMap *tin, bool use_tma
         }
         __syncthreads();
         const bool ok = mbar_wait_bounded(bar, 0);
+        if (stop) return false;                         // the box has landed; nothing else is in flight
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {
                 atomicExch(err, 1);
@@ -106,6 +108,7 @@ __device__ __forceinline__ bool tile_smooth(const CUtensorMap *tin, bool use_tma
             return false;
         }
     } else {
+        if (stop) return false;
         const int nxy = nx * ny, N = nxy * nz;
         constexpr int kBatch = 16;
         for (int p0 = 0; p0 < G::SN; p0 += kBatch * FT) {
@@ -251,13 +254,13 @@ __global__ void __launch_bounds__(FT, 3) k_fused_smooth_compose(const __grid_con
                                                               const float *__restrict__ u, int mode, Taps t,
                                                               int nx, int ny, int nz, float *__restrict__ out,
                                                               const int *stop_flag, int *err) {
-    if (stop_flag && *stop_flag) return;
+    const bool stop = stopped(stop_flag);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     TileSmem<R> sm(smem_raw);
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * FQ, y0 = blockIdx.y * FQ, z0 = blockIdx.z * FQ;
     const bool utile = use_tma != 0 && mode != CGDIR_ADDITIVE;
-    if (!tile_smooth<R>(&tin, use_tma != 0, du, t, nx, ny, nz, x0, y0, z0, sm.S, sm.X, sm.bar, err, tid,
+    if (!tile_smooth<R>(&tin, use_tma != 0, du, t, nx, ny, nz, x0, y0, z0, sm.S, sm.X, sm.bar, err, tid, stop,
                         utile ? &umap : nullptr))
         return;
     const float *Z = sm.X;
@@ -359,13 +362,13 @@ template <int R, bool CONTOUR, typename IT>
 __global__ void __launch_bounds__(FT) k_fused_smooth_warp(const __grid_constant__ CUtensorMap tin, int use_tma,
                                                            const float *__restrict__ in, Taps t,
                                                            float *__restrict__ u, ForceArgs a, int *err) {
-    if (a.stop_flag && *a.stop_flag) return;
+    const bool stop = stopped(a.stop_flag);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     TileSmem<R> sm(smem_raw);
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * FQ, y0 = blockIdx.y * FQ, z0 = blockIdx.z * FQ;
-    if (!tile_smooth<R>(&tin, use_tma != 0, in, t, nx, ny, nz, x0, y0, z0, sm.S, sm.X, sm.bar, err, tid)) return;
+    if (!tile_smooth<R>(&tin, use_tma != 0, in, t, nx, ny, nz, x0, y0, z0, sm.S, sm.X, sm.bar, err, tid, stop)) return;
     const float *Z = sm.X;
     const int nxy = nx * ny, N = nxy * nz;
     Cell cell[kVoxPerThread];

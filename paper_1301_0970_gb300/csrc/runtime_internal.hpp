@@ -50,7 +50,7 @@ struct WsSet {
 
 // Kernel choices for one pyramid level shape, picked by timing (autotune.cu).
 struct TunedLevel {
-    int smooth_variant = 0;    // best per-step smoothing: SMOOTH_MARCH / TILE / SPLIT (0 = by size)
+    int smooth_variant = 0;    // best per-step smoothing: SMOOTH_MARCH / TILE / SPLIT (0 = the z-march)
     int smooth_zchunk = 0;     // z chunk of the z-march smoothing (0 = default)
     int force_zchunk = 0;      // z chunk of the force stencil pass (0 = default)
     int force_width = 0;       // voxels per thread of the stencil pass: 0 = the widest, 2, 1
@@ -191,8 +191,10 @@ void launches_sub(unsigned long long n);
 // Tuned (else default) kernel choices for a level shape.
 // allow_fused: false for registrations that share the GPU (batches, served
 // requests), which take the best per-step schedule.
-SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt, bool allow_fused);
+SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt, bool allow_fused,
+                           float sigma);
 int force_zchunk_for(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt);
+int force_schedule(const cgdir_ctx *ctx, ForceArgs &a, int sdt);
 bool use_level_coop(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt);
 // Smallest force z chunk any tuning may choose (sizes the partial buffers).
 int force_zchunk_min(int nx, int ny, int nz);

@@ -95,3 +95,41 @@ def test_smooth_march_equals_tile_kernel(shape, sigma):
 
 def hash_of(shape):
     return shape[0] * 10007 + shape[1] * 101 + shape[2]
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float16])
+@pytest.mark.parametrize("shape", [(1, 3, 4), (9, 21, 44), (30, 40, 64), (33, 50, 200), (70, 90, 128), (13, 22, 45), (21, 30, 70)])
+def test_small_level_schedule_keeps_histories(shape, dtype, monkeypatch):
+    """The untuned schedule of small levels (narrow threads, short chunks, the
+    sums' chains taken up by other threads, the fused tile kernels) against the
+    four-voxel / per-step one: DVF and RMS-ID histories bit for bit, structure
+    terms on, over the schedule's size classes and a width that is no multiple
+    of four."""
+    rng = np.random.default_rng(hash_of(shape))
+    img = rng.normal(0, 300, shape).astype(np.float32)
+    mov = torch.from_numpy(img + rng.normal(0, 40, shape).astype(np.float32)).to(DEV, dtype)
+    img = torch.from_numpy(img).to(DEV, dtype)
+    masks = [torch.from_numpy((rng.random(shape) < p).astype(np.uint8)).to(DEV) for p in (0.02, 0.5)]
+    kw = dict(levels=1, iters=[4], lam=[1e-3, 0.5], sign=[1, -1], stop_mode=cg.CGDIR_STOP_FIXED)
+    out = []
+    for env in ({}, {"CGDIR_SMOOTH": "march"}, {"CGDIR_SMOOTH": "tile", "CGDIR_FORCE_ZCHUNK": str(default_zchunk(shape))}):
+        for name, v in env.items():
+            monkeypatch.setenv(name, v)
+        with cg.Context(0) as c:
+            out.append(c.register(img, mov, masks, masks, **kw))
+        for name in env:
+            monkeypatch.delenv(name)
+    for dvf, stats in out[1:]:
+        assert torch.equal(dvf, out[0][0])
+        assert stats[0]["rms_id"] == out[0][1][0]["rms_id"]
+
+
+def default_zchunk(shape):
+    """The chunk of the widest thread's pass: two CTAs per SM and four waves of
+    128-wide tiles (at least 4 planes), or four and two of 32-wide ones."""
+    nz, ny, nx = shape
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tiles = -(-(nx // 4 if nx % 4 == 0 else nx) // 32) * -(-ny // 8)
+    chunks = max(1, min(nz, -(-8 * sms // tiles)))
+    zc = -(-nz // chunks)
+    return max(min(4, nz), zc) if nx % 4 == 0 else zc
