@@ -128,15 +128,23 @@ int force_zchunk_for(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, 
 }
 
 // Pass 2's z chunk (returned) and its width and chains (in a) for a level.
+// A tuned level whose choice is the widest thread with the default chunk runs
+// the untuned schedule: the same sums, on more threads where the level is
+// small.
 int force_schedule(const cgdir_ctx *ctx, ForceArgs &a, int sdt) {
     const int contour = a.contour && a.k > 0;
-    const bool dflt = ctx->force_width == 0 && ctx->force_zchunk == 0 &&
-                      find_tuned(ctx, a.nx, a.ny, a.nz, contour, sdt) == nullptr;
-    const ForceShape f = force_default_shape(a.nx, a.ny, a.nz, contour != 0);
     a.pass2_width = force_width_for(ctx, a.nx, a.ny, a.nz, contour, sdt);
-    a.chain_w = dflt ? f.chain_w : 0;
-    a.chain_z = dflt ? f.chain_z : 0;
-    return force_zchunk_for(ctx, a.nx, a.ny, a.nz, contour, sdt);
+    a.chain_w = a.chain_z = 0;
+    const int zc = force_zchunk_for(ctx, a.nx, a.ny, a.nz, contour, sdt);
+    if (ctx->force_width > 0 || ctx->force_zchunk > 0) return zc;
+    if (find_tuned(ctx, a.nx, a.ny, a.nz, contour, sdt) &&
+        (a.pass2_width != 0 || zc != force_default_zchunk(a.nx, a.ny, a.nz)))
+        return zc;
+    const ForceShape f = force_default_shape(a.nx, a.ny, a.nz, contour != 0);
+    a.pass2_width = f.width;
+    a.chain_w = f.chain_w;
+    a.chain_z = f.chain_z;
+    return std::max(force_zchunk_min(a.nx, a.ny, a.nz), f.zchunk);
 }
 
 // Average time of `reps` launches of `body` after two untimed ones (ms).
@@ -211,25 +219,18 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     TunedLevel best;
+    int run_zc = 0;                 // the chosen stencil pass's chunk as a registration runs it
     const int reps = N > ((size_t)4 << 20) ? 5 : 20;
     int rc = CGDIR_OK;
     {
         const int d = force_default_zchunk(nx, ny, nz);
         const int cand[4] = {d, std::max(1, d / 2), std::max(1, d / 4), std::min(nz, 2 * d)};
         // the stencil pass's width: four voxels per thread (the widest where
-        // nx % 4 == 0), two or, with structure terms, one (more threads, for
-        // small levels)
-        const int widths[3] = {0, 2, 1};
-        const int nw = nx % 4 == 0 && ctx->force_width == 0 ? (contour ? 3 : 2) : 1;
+        // nx % 4 == 0) or two (twice the CTAs, for small levels)
+        const int widths[2] = {0, 2};
+        const int nw = nx % 4 == 0 && ctx->force_width == 0 ? 2 : 1;
+        const bool wave = N > 200000;
         float bt = 1e30f;
-        // the untuned choice
-        rc = time_ms(ctx, e0, e1, reps, &bt, [&](cudaStream_t st) {
-            ForceArgs b = a;
-            const int zc = force_schedule(ctx, b, -1);
-            return launch_force(b, zc, nullptr, st, kerr(ctx));
-        });
-        best.default_force_ms = bt;
-        bt = 1e30f;
         for (int wi = 0; wi < nw && rc == CGDIR_OK; ++wi) {
             a.pass2_width = ctx->force_width > 0 ? ctx->force_width : widths[wi];
             for (int ci = 0; ci < 4 && rc == CGDIR_OK; ++ci) {
@@ -239,11 +240,14 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 float ms = 0.f;
                 rc = time_ms(ctx, e0, e1, reps, &ms,
                              [&](cudaStream_t st) { return launch_force(a, cand[ci], nullptr, st, kerr(ctx)); });
-                // within the noise of these timings the wider thread and the
-                // longer chunk (fewer CTAs and halo planes) stand
-                const float slack = wi > 0 && best.force_width != widths[wi] ? 0.97f
-                                    : cand[ci] > best.force_zchunk ? 1.03f : 0.97f;
-                if (rc == CGDIR_OK && ms < slack * bt) {
+                // within the noise of these timings (2 %) the wider thread
+                // and the longer chunk (fewer CTAs and halo planes) stand; on
+                // a level of less than a wave (where the default shape, too,
+                // takes one plane per thread) the shorter and narrower ones
+                const bool preferred = wave ? cand[ci] > best.force_zchunk && widths[wi] == best.force_width
+                                            : cand[ci] < best.force_zchunk ||
+                                                  (cand[ci] == best.force_zchunk && widths[wi] > best.force_width);
+                if (rc == CGDIR_OK && ms < (preferred ? 1.02f : 0.98f) * bt) {
                     bt = ms;
                     best.force_zchunk = cand[ci];
                     best.force_width = widths[wi];
@@ -251,12 +255,19 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 }
             }
         }
-        if (rc == CGDIR_OK && best.default_force_ms <= best.force_ms) {       // nothing beat the untuned choice
-            best.force_zchunk = force_zchunk_for(ctx, nx, ny, nz, contour, -1);
-            best.force_width = ctx->force_width > 0 ? 0 : force_width_for(ctx, nx, ny, nz, contour, -1);
-            best.force_ms = best.default_force_ms;
-        }
+        // the untuned schedule
+        ForceArgs b = a;
+        const int zc = force_schedule(ctx, b, -1);
+        if (rc == CGDIR_OK)
+            rc = time_ms(ctx, e0, e1, reps, &best.default_force_ms,
+                         [&](cudaStream_t st) { return launch_force(b, zc, nullptr, st, kerr(ctx)); });
         a.pass2_width = ctx->force_width > 0 ? ctx->force_width : best.force_width;
+        run_zc = best.force_zchunk;
+        if (best.force_width == 0 && best.force_zchunk == d) {      // runs the untuned schedule
+            best.force_ms = best.default_force_ms;
+            a = b;
+            run_zc = zc;
+        }
     }
     if (rc == CGDIR_OK) {
         float bt = 1e30f;
@@ -270,31 +281,42 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
             cand[nc++].zchunk = zc;
         };
         // z chunks: the estimated best and the volume cut into 1 .. 16 chunks
-        // (longer chunks reload fewer halo planes; more chunks fill more SMs);
+        // (longer chunks reload fewer halo planes; more chunks fill more SMs;
+        // without TMA, where an iteration takes longer to time, 2 and 4);
         // the 32 x 16 z-march with 2, 4 and 8 chunks (more CTAs per chunk on
         // small levels)
         add(SMOOTH_MARCH, d);
-        const int nch[7] = {1, 2, 3, 4, 6, 8, 16};
-        for (int q = 0; q < 7; ++q) add(SMOOTH_MARCH, (nz + nch[q] - 1) / nch[q]);
-        for (int c = 2; c <= 8; c *= 2) add(SMOOTH_MARCH_NARROW, (nz + c - 1) / c);
+        const int nch[7] = {2, 4, 1, 3, 6, 8, 16};
+        for (int q = 0; q < (nx % 4 == 0 ? 7 : 2); ++q) add(SMOOTH_MARCH, (nz + nch[q] - 1) / nch[q]);
+        for (int c = 2; c <= 8 && nx % 4 == 0; c *= 2) add(SMOOTH_MARCH_NARROW, (nz + c - 1) / c);
         cand[nc].variant = SMOOTH_TILE; cand[nc++].zchunk = 0;
         cand[nc].variant = SMOOTH_SPLIT; cand[nc++].zchunk = 0;
+        const int dflt = smooth_auto_variant(nx, ny, nz);
         for (int ci = 0; ci < nc && rc == CGDIR_OK; ++ci) {
             float ms = 0.f;
+            const bool untuned = cand[ci].variant == dflt && (ci == 0 || dflt != SMOOTH_MARCH);
             // one iteration: the force step (so du and the caches are as in a
             // registration: timed alone on a level that fits in L2, the
             // smoothing favours other z chunks), G(du) with the composite
             // update, then G(u'); the force step's own time is taken off
-            rc = time_ms(ctx, e0, e1, reps, &ms, [&](cudaStream_t st) {
-                cudaError_t e = launch_force(a, best.force_zchunk, nullptr, st, kerr(ctx));
+            auto iteration = [&](cudaStream_t st) {
+                cudaError_t e = launch_force(a, run_zc, nullptr, st, kerr(ctx));
                 if (e != cudaSuccess) return e;
                 e = launch_smooth_compose(du, u, CGDIR_COMPOSE, sigma, nx, ny, nz, out, sscr, nullptr, st, kerr(ctx),
                                           false, cand[ci]);
                 if (e != cudaSuccess) return e;
                 return launch_smooth(out, 3, sigma, nx, ny, nz, du, nullptr, st, kerr(ctx), cand[ci], sscr);
-            });
+            };
+            // a candidate that three iterations show to be a tenth and 2 us
+            // (the resolution of so short a span) behind is dropped: timing
+            // all of them in full doubled the tuner's time on odd shapes
+            rc = time_ms(ctx, e0, e1, ci ? 3 : reps, &ms, iteration);
+            if (rc == CGDIR_OK && ci && ms - best.force_ms < 1.1f * bt + 2e-3f)
+                rc = time_ms(ctx, e0, e1, reps, &ms, iteration);
+            else if (ci && !untuned)
+                continue;
             ms = std::max(ms - best.force_ms, 0.f);
-            if (ci == 0) best.default_smooth_ms = ms;      // the untuned choice
+            if (untuned) best.default_smooth_ms = ms;
             if (rc == CGDIR_OK && ms < bt) {
                 bt = ms;
                 best.smooth_variant = cand[ci].variant;
@@ -310,10 +332,10 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
         a2.skip_warp = 1;
         float f2 = 0.f, fs = 0.f;
         rc = time_ms(ctx, e0, e1, reps, &f2,
-                     [&](cudaStream_t st) { return launch_force(a2, best.force_zchunk, nullptr, st, kerr(ctx)); });
+                     [&](cudaStream_t st) { return launch_force(a2, run_zc, nullptr, st, kerr(ctx)); });
         if (rc == CGDIR_OK)    // timed after the stencil pass, as in an iteration
             rc = time_ms(ctx, e0, e1, reps, &fs, [&](cudaStream_t st) {
-                cudaError_t e = launch_force(a2, best.force_zchunk, nullptr, st, kerr(ctx));
+                cudaError_t e = launch_force(a2, run_zc, nullptr, st, kerr(ctx));
                 if (e != cudaSuccess) return e;
                 e = launch_fused_smooth_compose(du, u, CGDIR_COMPOSE, sigma, nx, ny, nz, out, nullptr, kerr(ctx), st);
                 if (e != cudaSuccess) return e;

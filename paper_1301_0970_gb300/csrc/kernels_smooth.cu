@@ -1112,6 +1112,16 @@ static cudaError_t smooth_march(const float *in, float *out, int ncomp, const Ta
 #undef CGDIR_MARCH
 }
 
+// Small volumes without TMA take the one-pass tile: the z-march's planes there
+// wait for one asynchronous copy after another (smoothing du with the update
+// plus u, r = 2: 53x59x24 15.7 + 12.4 against 17.5 + 13.5 us, 95x71x34 22.8 +
+// 17.5 against 23.7 + 17.7; 83x157x24 is past the line, 26.8 + 20.0 against
+// 26.1 + 19.8).  With TMA the z-march is never behind (64x64x24 14.3 + 11.4
+// against 15.9 + 12.4 us).
+int smooth_auto_variant(int nx, int ny, int nz) {
+    return nx % 4 != 0 && (size_t)nx * ny * nz <= 250000 ? SMOOTH_TILE : SMOOTH_MARCH;
+}
+
 int smooth_default_zchunk(int nx, int ny, int nz, int ncomp, float sigma) {
     const int r = std::max(gauss_radius(sigma), 1), wy = r <= 4 ? 32 : 16;
     const int res = r <= 3 ? 5 : 4;          // MarchGeom::CTAS
@@ -1210,6 +1220,7 @@ cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int n
         return cudaGetLastError();
     }
     if (err != nullptr) {
+        if (variant == SMOOTH_AUTO && ch.zchunk == 0) variant = smooth_auto_variant(nx, ny, nz);
         if (variant == SMOOTH_FUSED) variant = SMOOTH_TILE;     // nothing to fuse with here
         if (variant == SMOOTH_TILE) return smooth_tile(in, ncomp, t, nx, ny, nz, out, stop_flag, s);
         if (variant == SMOOTH_SPLIT && scratch != nullptr && scratch != in && scratch != out)
