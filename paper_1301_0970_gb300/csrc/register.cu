@@ -560,10 +560,10 @@ int cgdir_register(cgdir_ctx *ctx, const cgdir_volume *S, const cgdir_volume *M,
     const ProfList *used = nullptr;
     TRY(plan_run(ctx, sl, pl, s, &used));
     TRY(plan_outputs(ctx, sl, pl, dvf_out, false, s));
-    CK(cudaStreamSynchronize(s));
+    const int words = read_words(ctx, sizeof(int), s);
     CK(cudaGetLastError());
     prof_collect(ctx, *used);
-    TRY(check_err_word(ctx));
+    TRY(words);
     plan_stats(sl, pl, stats_out);
     return CGDIR_OK;
 }
@@ -640,10 +640,10 @@ int cgdir_register_batch(cgdir_ctx *ctx, int count, const cgdir_volume *statics,
         used = &ctx->eager;
     }
     for (int i = 0; i < count; ++i) TRY(plan_outputs(ctx, *ctx->slots[i], pls[i], dvf_outs[i], false, s));
-    CK(cudaStreamSynchronize(s));
+    const int words = read_words(ctx, sizeof(int), s);
     CK(cudaGetLastError());
     prof_collect(ctx, *used);
-    TRY(check_err_word(ctx));
+    TRY(words);
     if (stats_out)
         for (int i = 0; i < count; ++i) plan_stats(*ctx->slots[i], pls[i], stats_out + (size_t)i * pls[i].L);
     return CGDIR_OK;

@@ -174,15 +174,25 @@ bool dims_ok(int nx, int ny, int nz) { return nx >= 1 && ny >= 1 && nz >= 1; }
 int *kerr(cgdir_ctx *ctx) { return ctx->plain_kernels ? nullptr : ctx->err_word; }
 
 // After the stream has drained: a kernel wait that ran out is a timeout.
-int check_err_word(cgdir_ctx *ctx) {
-    int h = 0;
-    cudaError_t e = cudaMemcpy(&h, ctx->err_word, sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return fail(ctx, CGDIR_ECUDA, std::string("error word: ") + cudaGetErrorString(e));
+static int judge_err_word(cgdir_ctx *ctx, int h) {
     if (h) {
         cudaMemset(ctx->err_word, 0, sizeof(int));
         return fail(ctx, CGDIR_ETIMEDOUT, "a bounded wait inside a kernel ran out (TMA load not completed)");
     }
     return CGDIR_OK;
+}
+
+int check_err_word(cgdir_ctx *ctx) {
+    int h = 0;
+    cudaError_t e = cudaMemcpy(&h, ctx->err_word, sizeof(int), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return fail(ctx, CGDIR_ECUDA, std::string("error word: ") + cudaGetErrorString(e));
+    return judge_err_word(ctx, h);
+}
+
+int read_words(cgdir_ctx *ctx, size_t bytes, cudaStream_t s) {
+    CK(cudaMemcpyAsync(ctx->h_words, ctx->words, bytes, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    return judge_err_word(ctx, ctx->h_words->err);
 }
 
 bool sigma_ok(float s) { return std::isfinite(s) && s >= 0.f && s <= CGDIR_MAX_SIGMA; }
@@ -346,13 +356,17 @@ int cgdir_create(cgdir_ctx **out, const cgdir_config *cfg) {
         c->use_graphs = false;
         c->cap_stream = nullptr;
     }
-    if (cudaMalloc(&c->err_word, sizeof(int)) != cudaSuccess ||
-        cudaMemsetAsync(c->err_word, 0, sizeof(int), c->stream) != cudaSuccess) {
+    if (cudaMalloc(&c->words, sizeof(CallWords)) != cudaSuccess ||
+        cudaMallocHost(&c->h_words, sizeof(CallWords)) != cudaSuccess ||
+        cudaMemsetAsync(c->words, 0, sizeof(CallWords), c->stream) != cudaSuccess) {
         cudaGetLastError();
+        if (c->words) cudaFree(c->words);
+        if (c->h_words) cudaFreeHost(c->h_words);
         if (c->own_stream) cudaStreamDestroy(c->stream);
         delete c;
         return CGDIR_ECUDA;
     }
+    c->err_word = &c->words->err;
     *out = c;
     return CGDIR_OK;
 }
@@ -376,7 +390,8 @@ void cgdir_destroy(cgdir_ctx *ctx) {
     ctx->eager.release();
     for (cudaStream_t b : ctx->branch_streams) cudaStreamDestroy(b);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
-    if (ctx->err_word) cudaFree(ctx->err_word);
+    if (ctx->words) cudaFree(ctx->words);
+    if (ctx->h_words) cudaFreeHost(ctx->h_words);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }
@@ -409,7 +424,7 @@ static SmoothChoice prim_smooth(const cgdir_ctx *ctx) {
 }
 
 static int force_impl(cgdir_ctx *ctx, const ForceArgs &a, double *stats_host) {
-    void *part = nullptr, *st = nullptr;
+    void *part = nullptr;
     ForceArgs b = a;
     const int zc = force_schedule(ctx, b, a.img_dtype);
     if (b.contour && b.k > 0 && !ctx->plain_kernels && b.mtex == nullptr) {
@@ -426,19 +441,26 @@ static int force_impl(cgdir_ctx *ctx, const ForceArgs &a, double *stats_host) {
         TRY(ws_get(ctx, "force_scr", force_scratch_bytes(N, b.contour ? b.k : 0), &scr));
         force_scratch_assign(b, scr, N);
     }
+    // the two-pass kernels' last CTA sums the partials itself; the others
+    // can give up a bounded wait and leave the counter behind
+    const bool fused_sum = b.wfield != nullptr && (size_t)a.nx * a.ny * a.nz < (size_t)1 << 31;
     if (stats_host) {
         TRY(ws_get(ctx, "partial", force_partial_count(a.nx, a.ny, a.nz, zc) * kPartialStride * sizeof(double), &part));
-        TRY(ws_get(ctx, "stats", 4 * sizeof(double), &st));
         b.partial = (double *)part;
+        if (fused_sum) {
+            b.fin.done = &ctx->words->done;
+            b.fin.stats_out = ctx->words->stats;
+        }
     }
     int nb = 0;
     CK(launch_force(b, zc, &nb, ctx->stream, kerr(ctx)));
     if (stats_host) {
         LevelState ls{};
-        CK(launch_finalize((double *)part, nb, ls, 0, 0, CGDIR_STOP_FIXED, 0.0, (double *)st, ctx->stream));
-        CK(cudaMemcpyAsync(stats_host, st, 3 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-        CK(cudaStreamSynchronize(ctx->stream));
-        TRY(check_err_word(ctx));
+        if (!fused_sum)
+            CK(launch_finalize((double *)part, nb, ls, 0, 0, CGDIR_STOP_FIXED, 0.0, ctx->words->stats, ctx->stream));
+        const int rc = read_words(ctx, offsetof(CallWords, sums), ctx->stream);
+        std::copy_n(ctx->h_words->stats, 3, stats_host);
+        TRY(rc);
     }
     return CGDIR_OK;
 }
@@ -601,14 +623,13 @@ int cgdir::rt::auto_sign_impl(cgdir_ctx *ctx, const void *T0, int dtype, const u
         return fail(ctx, CGDIR_EINVAL, "auto_sign: bad arguments");
     if (k == 0) return CGDIR_OK;
     DeviceGuard g(ctx->device);
-    void *dxy = nullptr, *part = nullptr, *sums = nullptr;
+    void *dxy = nullptr, *part = nullptr;
     TRY(ws_get(ctx, "sign_dxy", (size_t)nx * ny * nz, &dxy));
     TRY(ws_get(ctx, "sign_part", sign_partial_rows(nx, ny, nz) * k * 4 * sizeof(double), &part));
-    TRY(ws_get(ctx, "sign_sums", kMaxMasks * 4 * sizeof(double), &sums));
-    CK(launch_sign_sums(T0, dtype, sbits, k, nx, ny, nz, (uint8_t *)dxy, (double *)part, (double *)sums,
+    CK(launch_sign_sums(T0, dtype, sbits, k, nx, ny, nz, (uint8_t *)dxy, (double *)part, ctx->words->sums,
                         ctx->stream));
-    double h[kMaxMasks * 4];
-    CK(cudaMemcpyAsync(h, sums, k * 4 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    double *h = ctx->h_words->sums;
+    CK(cudaMemcpyAsync(h, ctx->words->sums, k * 4 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     for (int j = 0; j < k; ++j) {
         const double sin_ = h[4 * j], cin = h[4 * j + 1], ssh = h[4 * j + 2], csh = h[4 * j + 3];
@@ -631,15 +652,15 @@ int cgdir_rms_id(cgdir_ctx *ctx, const float *I0, const float *T0, const float *
     if (!I0 || !T0 || !u || !rms_host || !dims_ok(nx, ny, nz))
         return fail(ctx, CGDIR_EINVAL, "rms_id: bad arguments");
     DeviceGuard g(ctx->device);
-    void *part = nullptr, *st = nullptr;
+    void *part = nullptr;
     TRY(ws_get(ctx, "partial_m", metric_partial_count(nx, ny, nz) * kPartialStride * sizeof(double), &part));
-    TRY(ws_get(ctx, "stats", 4 * sizeof(double), &st));
     int nb = 0;
-    CK(launch_metric(I0, T0, CGDIR_F32, u, uroi, nx, ny, nz, (double *)part, nullptr, &nb, ctx->stream));
-    LevelState ls{};
-    CK(launch_finalize((double *)part, nb, ls, 0, 0, CGDIR_STOP_FIXED, 0.0, (double *)st, ctx->stream));
-    double h[3];
-    CK(cudaMemcpyAsync(h, st, 3 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    FinishArgs fin{};
+    fin.done = &ctx->words->done;
+    fin.stats_out = ctx->words->stats;
+    CK(launch_metric(I0, T0, CGDIR_F32, u, uroi, nx, ny, nz, (double *)part, nullptr, &nb, ctx->stream, &fin));
+    double *h = ctx->h_words->stats;
+    CK(cudaMemcpyAsync(h, ctx->words->stats, 3 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     *rms_host = h[1] > 0 ? std::sqrt(h[0] / h[1]) : 0.0;
     if (count_host) *count_host = (long long)h[1];
