@@ -199,8 +199,8 @@ cudaError_t launch_finalize(const double *partial, int nblocks, LevelState st, i
 // composite update fused into the du pass and the next warp into the u
 // pass; a standalone smoothing takes the tile kernel), or chosen by size.
 // SMOOTH_AUTO takes the z-march (its z chunks fill the SMs also on small
-// levels: 64x64x32 5 us against 11 for the tile kernel) except on small
-// volumes without TMA (smooth_auto_variant);
+// levels: 64x64x32 5 us against 11 for the tile kernel) except without TMA
+// (smooth_auto_variant);
 // SMOOTH_MARCH_NARROW is its 32 x 16 tile (same bits).
 enum { SMOOTH_AUTO = 0, SMOOTH_MARCH = 1, SMOOTH_TILE = 2, SMOOTH_SPLIT = 3, SMOOTH_FUSED = 4,
        SMOOTH_MARCH_NARROW = 5 };
@@ -215,7 +215,8 @@ struct SmoothChoice {
     int ctas_per_sm = 0;          // at most this many z-march CTAs per SM (0: no cap)
 };
 int smooth_default_zchunk(int nx, int ny, int nz, int ncomp, float sigma);
-int smooth_auto_variant(int nx, int ny, int nz);
+// scratch: the launch has a field of its own to hold a pass between kernels.
+int smooth_auto_variant(int nx, int ny, int nz, bool scratch);
 // err: device word set to 1 if a bounded wait inside the kernel ran out;
 // nullptr selects the plain-load kernel (no waits).
 cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int ny, int nz,

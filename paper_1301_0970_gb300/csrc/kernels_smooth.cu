@@ -1112,14 +1112,23 @@ static cudaError_t smooth_march(const float *in, float *out, int ncomp, const Ta
 #undef CGDIR_MARCH
 }
 
-// Small volumes without TMA take the one-pass tile: the z-march's planes there
-// wait for one asynchronous copy after another (smoothing du with the update
-// plus u, r = 2: 53x59x24 15.7 + 12.4 against 17.5 + 13.5 us, 95x71x34 22.8 +
-// 17.5 against 23.7 + 17.7; 83x157x24 is past the line, 26.8 + 20.0 against
-// 26.1 + 19.8).  With TMA the z-march is never behind (64x64x24 14.3 + 11.4
-// against 15.9 + 12.4 us).
-int smooth_auto_variant(int nx, int ny, int nz) {
-    return nx % 4 != 0 && (size_t)nx * ny * nz <= 250000 ? SMOOTH_TILE : SMOOTH_MARCH;
+// Without TMA the z-march's planes wait for one asynchronous copy after
+// another.  With a scratch field (an iteration has one) the split kernels are
+// ahead while the field between them stays in L2 (du smoothed with the update
+// plus u, per iteration: 107x91x40 24 + 20 against 33 + 25 us, 181x217x91 92 + 55
+// against 102 + 60, 301x213x113 168 + 112 against 202 + 121; 313x301x97, 9.1 M
+// voxels, is past the line, 208 + 132 against 197 + 100).
+// Without one, small volumes take the one-pass tile (53x59x24 12.3 against
+// 14.3 us, 95x71x34 17.5 against 17.7; 83x157x24 is past the line, 20.0 against
+// 19.8).  With TMA the z-march is never behind (64x64x24 14.3 + 11.4 against
+// the tile's 15.9 + 12.4 us, 256x256x96 96 + 36 against the split's 139 + 94).
+constexpr size_t kSplitVoxels = 8000000;
+
+int smooth_auto_variant(int nx, int ny, int nz, bool scratch) {
+    const size_t N = (size_t)nx * ny * nz;
+    if (nx % 4 == 0) return SMOOTH_MARCH;
+    if (scratch && N <= kSplitVoxels) return SMOOTH_SPLIT;
+    return N <= 250000 ? SMOOTH_TILE : SMOOTH_MARCH;
 }
 
 int smooth_default_zchunk(int nx, int ny, int nz, int ncomp, float sigma) {
@@ -1220,7 +1229,8 @@ cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int n
         return cudaGetLastError();
     }
     if (err != nullptr) {
-        if (variant == SMOOTH_AUTO && ch.zchunk == 0) variant = smooth_auto_variant(nx, ny, nz);
+        if (variant == SMOOTH_AUTO && ch.zchunk == 0)
+            variant = smooth_auto_variant(nx, ny, nz, scratch != nullptr && scratch != in && scratch != out);
         if (variant == SMOOTH_FUSED) variant = SMOOTH_TILE;     // nothing to fuse with here
         if (variant == SMOOTH_TILE) return smooth_tile(in, ncomp, t, nx, ny, nz, out, stop_flag, s);
         if (variant == SMOOTH_SPLIT && scratch != nullptr && scratch != in && scratch != out)
@@ -1236,6 +1246,7 @@ cudaError_t launch_smooth_compose(const float *du, const float *u, int mode, flo
                                   int *err, bool one_pass, SmoothChoice ch) {
     const Taps t = gauss_taps(sigma);
     if (!one_pass && t.r > 0 && err != nullptr) {
+        if (ch.variant == SMOOTH_AUTO && ch.zchunk == 0) ch.variant = smooth_auto_variant(nx, ny, nz, tmp != nullptr);
         if (ch.variant == SMOOTH_SPLIT)   // x/y pass, then the z pass with the composite update fused
             return smooth_split(du, u, mode, true, 3, t, nx, ny, nz, out, tmp, ch.zchunk, stop_flag, s);
         if (ch.variant == SMOOTH_FUSED && (size_t)nx * ny * nz < (size_t)1 << 31)   // one 3-D tile kernel

@@ -133,3 +133,24 @@ def default_zchunk(shape):
     chunks = max(1, min(nz, -(-8 * sms // tiles)))
     zc = -(-nz // chunks)
     return max(min(4, nz), zc) if nx % 4 == 0 else zc
+
+
+@pytest.mark.parametrize("shape", [(5, 7, 9), (24, 59, 53), (33, 65, 67), (40, 91, 107)])
+@pytest.mark.parametrize("sigma", [0.5, 1.0, 2.0])
+def test_rows_without_tma_take_the_split_kernels_with_the_same_bits(monkeypatch, shape, sigma):
+    """The default for nx % 4 != 0 (split kernels where there is a scratch
+    field, tiles or the z-march without one) against the z-march: every
+    variant sums its taps in one order, so the results are equal."""
+    torch.manual_seed(3)
+    du = torch.randn((3,) + shape, device="cuda")
+    u = 2 * torch.randn((3,) + shape, device="cuda")
+    got = []
+    for forced in (None, "march"):
+        if forced:
+            monkeypatch.setenv("CGDIR_SMOOTH", forced)
+        with cg.Context(0) as ctx:
+            got.append([ctx.smooth_compose(du, u, sigma=sigma), ctx.smooth(du, sigma),
+                        ctx.smooth(du[0].contiguous(), sigma)])
+            ctx.sync()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
