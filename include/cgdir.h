@@ -185,7 +185,8 @@ void cgdir_default_params(cgdir_params *p);
      CGDIR_SMOOTH=march|tile|split|fused, CGDIR_SMOOTH_ZCHUNK=n   smoothing variant
      CGDIR_FORCE_ZCHUNK=n, CGDIR_FORCE_WIDTH=1|2   force pass 2 z chunk / voxels
                                  per thread (default: 4 where nx % 4 == 0, else 2
-                                 for even nx, else 1)
+                                 for even nx, else 1; on levels of up to 1.6 M
+                                 voxels with structure terms 1 or 2)
      CGDIR_COOP_MAX=n            levels below the finest with at most n voxels
                                  run as one cooperative launch
      CGDIR_SERVE_SCHEDULE=shared|alone|auto   schedule of submitted requests
@@ -211,7 +212,7 @@ size_t cgdir_mem_in_use(const cgdir_ctx *ctx);
 
 /* Wait for all work queued on ctx's stream.  Returns CGDIR_ETIMEDOUT if a
    kernel's bounded wait for its own asynchronous (TMA) loads ran out since
-   the last check -- the kernel then wrote no output and returned -- and
+   the last check -- the kernel then returned with its output incomplete -- and
    CGDIR_ECUDA if the stream reports an error.  The blocking entry points
    (cgdir_register, and cgdir_force / cgdir_iterate with stats) do this
    check themselves. */
@@ -468,9 +469,11 @@ int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us);
  * and of the smoothing with the composite update (steps 2-4 of an
  * iteration, timed behind a force step: the 32 x 32 z-march with the
  * volume in 1 to 16 z chunks, the 32 x 16 one with 2, 4 and 8, 3-D
- * shared-memory tile, split xy + z kernels with the update in the z pass)
- * on ctx's stream and keeps the fastest, then times the fused schedule
- * against it.  Later registrations of those shapes use the choices:
+ * shared-memory tile, split xy + z kernels with the update in the z pass;
+ * fewer where nx % 4 != 0) on ctx's stream and keeps the fastest, then times
+ * the fused schedule, which has to win by 5 %.  The timings resolve about
+ * 2 %: within that the wide thread and the long chunk stand (on levels of
+ * less than a wave the short and narrow ones).  Later registrations of those shapes use the choices:
  * cgdir_register, and a request submitted on an idle GPU, the fused
  * schedule where it won; batched registrations and requests submitted while
  * others run (they share the GPU, so throughput counts) the best per-step
@@ -493,9 +496,11 @@ typedef struct {
     int   smooth_zchunk;        /* z chunk of the z-march (0 = default / n/a)       */
     int   force_zchunk;         /* z chunk of the force stencil pass                */
     float smooth_ms, force_ms;  /* best times: steps 2-4 of one iteration; force   */
-    float default_smooth_ms, default_force_ms;   /* the untuned choice's times     */
+    float default_smooth_ms, default_force_ms;   /* the untuned choice's times (those of
+                                   the fused schedule where an untuned level runs it) */
     int   force_width;          /* voxels per thread of the stencil pass: 0 = the
-                                   widest the shape allows (4 where nx % 4 == 0), 2 */
+                                   widest the shape allows (4 where nx % 4 == 0), 2;
+                                   0 with the default chunk runs the untuned pass */
 } cgdir_tuning;
 
 /* Tune every level of a `levels`-level pyramid whose finest level is
