@@ -290,7 +290,9 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
         const int nch[7] = {2, 4, 1, 3, 6, 8, 16};
         for (int q = 0; q < (nx % 4 == 0 ? 7 : 2); ++q) add(SMOOTH_MARCH, (nz + nch[q] - 1) / nch[q]);
         for (int c = 2; c <= 8 && nx % 4 == 0; c *= 2) add(SMOOTH_MARCH_NARROW, (nz + c - 1) / c);
-        add(SMOOTH_TILE, 0);
+        // without TMA the tile and, below, the fused kernels are far behind on
+        // larger volumes (per iteration 91x108x60 62 us, tile 77, fused 105)
+        if (nx % 4 == 0 || N <= 500000) add(SMOOTH_TILE, 0);
         add(SMOOTH_SPLIT, 0);
         const int dflt = smooth_auto_variant(nx, ny, nz, true);
         for (int ci = 0; ci < nc && rc == CGDIR_OK; ++ci) {
@@ -330,7 +332,7 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
     }
     // the fused schedule: force stencil pass only, then the two fused tile
     // kernels (G(du) + update; G(u') + the next warp)
-    if (rc == CGDIR_OK && fused_schedule_ok(a) && gauss_taps(sigma).r > 0) {
+    if (rc == CGDIR_OK && (nx % 4 == 0 || N <= 500000) && fused_schedule_ok(a) && gauss_taps(sigma).r > 0) {
         ForceArgs a2 = a;
         a2.skip_warp = 1;
         float f2 = 0.f, fs = 0.f;
