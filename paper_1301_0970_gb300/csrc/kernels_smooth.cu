@@ -933,30 +933,31 @@ __global__ void __launch_bounds__(NT) k_smooth_z(const float *__restrict__ in, c
     const size_t nxy = (size_t)nx * ny, N = nxy * nz, col = (size_t)y * nx + x;
     const float *src = in + (size_t)comp * N + col;
     float *dst = out + (size_t)comp * N + col;
-    float ring[NC][K];
+    // planes loaded ahead: two (u smoothed, per launch pair: 213x248x48 42 -> 37 us,
+    // 237x213x107 87 -> 73; three 38 and 77); one where the update's gathers
+    // need the registers (76 against 126: 133 -> 153 us)
+    constexpr int ZAHEAD = COMPOSE ? 1 : 2;
+    constexpr int M = K + ZAHEAD;         // planes t - 2r .. t and the loads in flight behind them
+    float ring[NC][M];
+    auto load = [&](int t, float (&v)[NC][M], int slot) {
+        const size_t zo = (size_t)clampi(zb - R + t, 0, nz - 1) * nxy;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[c][slot] = __ldg(src + c * N + zo);
+    };
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
-        for (int j = 0; j < K; ++j) ring[c][j] = 0.f;
-    float nxt[NC];
-    {
-        const size_t zo = (size_t)clampi(zb - R, 0, nz - 1) * nxy;
+        for (int j = 0; j < M; ++j) ring[c][j] = 0.f;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) nxt[c] = __ldg(src + c * N + zo);
-    }
+    for (int t = 0; t < ZAHEAD; ++t)
+        if (t < P) load(t, ring, t);
     const float fxmax = (float)(nx - 1), fymax = (float)(ny - 1), fzmax = (float)(nz - 1);
-    for (int t0 = 0; t0 < P; t0 += K) {
+    for (int t0 = 0; t0 < P; t0 += M) {
 #pragma unroll
-        for (int r = 0; r < K; ++r) {
+        for (int r = 0; r < M; ++r) {
             const int t = t0 + r;
             if (t >= P) break;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) ring[c][r] = nxt[c];
-            if (t + 1 < P) {
-                const size_t zo = (size_t)clampi(zb - R + t + 1, 0, nz - 1) * nxy;
-#pragma unroll
-                for (int c = 0; c < NC; ++c) nxt[c] = __ldg(src + c * N + zo);
-            }
+            if (t + ZAHEAD < P) load(t + ZAHEAD, ring, (r + ZAHEAD) % M);
             if (t < 2 * R) continue;
             const int z = zb + t - 2 * R;
             float sv[NC];
@@ -964,7 +965,7 @@ __global__ void __launch_bounds__(NT) k_smooth_z(const float *__restrict__ in, c
             for (int c = 0; c < NC; ++c) {
                 float acc = 0.f;
 #pragma unroll
-                for (int j = 0; j < K; ++j) acc = fmaf(taps.w[j], ring[c][(r + 1 + j) % K], acc);
+                for (int j = 0; j < K; ++j) acc = fmaf(taps.w[j], ring[c][(r + ZAHEAD + 1 + j) % M], acc);
                 sv[c] = acc;
             }
             const size_t i = (size_t)z * nxy;
@@ -1115,9 +1116,9 @@ static cudaError_t smooth_march(const float *in, float *out, int ncomp, const Ta
 // Without TMA the z-march's planes wait for one asynchronous copy after
 // another.  With a scratch field (an iteration has one) the split kernels are
 // ahead while the field between them stays in L2 (du smoothed with the update
-// plus u, per iteration: 107x91x40 24 + 20 against 33 + 25 us, 181x217x91 92 + 55
-// against 102 + 60, 301x213x113 168 + 112 against 202 + 121; 313x301x97, 9.1 M
-// voxels, is past the line, 208 + 132 against 197 + 100).
+// plus u, per iteration: 107x91x40 24 + 17 against 33 + 25 us, 181x217x91 92 + 48
+// against 102 + 60, 301x213x113 167 + 95 against 202 + 121; 313x301x97, 9.1 M
+// voxels, is past the line, 208 + 114 against 197 + 100).
 // Without one, small volumes take the one-pass tile (53x59x24 12.3 against
 // 14.3 us, 95x71x34 17.5 against 17.7; 83x157x24 is past the line, 20.0 against
 // 19.8).  With TMA the z-march is never behind (64x64x24 14.3 + 11.4 against
