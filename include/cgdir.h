@@ -470,14 +470,17 @@ int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us);
  * iteration, timed behind a force step: the 32 x 32 z-march with the
  * volume in 1 to 16 z chunks, the 32 x 16 one with 2, 4 and 8, 3-D
  * shared-memory tile, split xy + z kernels with the update in the z pass;
- * fewer where nx % 4 != 0) on ctx's stream and keeps the fastest, then times
- * the fused schedule, which has to win by 5 %.  The timings resolve about
- * 2 %: within that the wide thread and the long chunk stand (on levels of
- * less than a wave the short and narrow ones).  Later registrations of those shapes use the choices:
+ * fewer where nx % 4 != 0) on ctx's stream, those of small levels as CUDA
+ * graphs, and keeps the fastest; the untuned force pass stands unless another
+ * is ahead by more than 3 %.  Then it times the fused schedule, which has to
+ * win by 5 %.  Later registrations of those shapes use the choices:
  * cgdir_register, and a request submitted on an idle GPU, the fused
  * schedule where it won; batched registrations and requests submitted while
  * others run (they share the GPU, so throughput counts) the best per-step
- * schedule.  Only the kernels change: every choice gives the same bits.
+ * schedule.  Every choice gives the same field after the same iterations,
+ * bit for bit.  The reported rms_id are sums whose FP32 parts follow
+ * force_zchunk and force_width: another choice moves them by some 1e-8 of
+ * their value, and with them a convergence test that stands that close.
  * Blocking. */
 #define CGDIR_SMOOTH_MARCH 1
 #define CGDIR_SMOOTH_TILE  2
@@ -518,8 +521,8 @@ int cgdir_tuning_read(const cgdir_ctx *ctx, cgdir_tuning *out, int cap);
 /* Install n tuned shapes (as cgdir_tuning_read returns them, e.g. saved by
    an earlier process), replacing the context's entries for those shapes;
    later registrations use them without timing anything.  Only the kernel
-   choices are used (results do not depend on them); the times are kept for
-   reporting.  Errors: EINVAL (bad shape, variant or z chunk; nothing is
+   choices are used (cgdir_autotune says what depends on them); the times are
+   kept for reporting.  Errors: EINVAL (bad shape, variant or z chunk; nothing is
    installed then). */
 int cgdir_tuning_load(cgdir_ctx *ctx, const cgdir_tuning *in, int n);
 

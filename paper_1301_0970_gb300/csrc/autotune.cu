@@ -147,15 +147,42 @@ int force_schedule(const cgdir_ctx *ctx, ForceArgs &a, int sdt) {
     return std::max(force_zchunk_min(a.nx, a.ny, a.nz), f.zchunk);
 }
 
-// Average time of `reps` launches of `body` after two untimed ones (ms).
+// Average time of `reps` launches of `body` (ms), after two untimed ones or,
+// as one graph, after an untimed launch of that graph.  Short bodies are timed
+// as a graph, as a registration runs them: launched one by one they start at
+// the pace of the host, in steps of 2 us (128x128x40, structure terms, chunks
+// of 4 / 8 planes: 16.5 / 16.5 us one by one, 12.8 / 13.5 as graphs), and the
+// pick among them, with the grouping of the RMS-ID sums that goes with it, was
+// left to noise.
 template <typename Body>
-static int time_ms(cgdir_ctx *ctx, cudaEvent_t a, cudaEvent_t b, int reps, float *ms, Body body) {
+static int time_ms(cgdir_ctx *ctx, cudaEvent_t a, cudaEvent_t b, int reps, bool graph, float *ms, Body body) {
     cudaStream_t s = ctx->stream;
-    for (int r = 0; r < 2; ++r) CK(body(s));
-    CK(cudaEventRecord(a, s));
-    for (int r = 0; r < reps; ++r) CK(body(s));
-    CK(cudaEventRecord(b, s));
-    CK(cudaEventSynchronize(b));
+    if (graph && ctx->cap_stream) {
+        const unsigned long long before = launches_now();
+        CK(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
+        cudaError_t e = cudaSuccess;
+        for (int r = 0; r < reps && e == cudaSuccess; ++r) e = body(ctx->cap_stream);
+        cudaGraph_t g = nullptr;
+        cudaGraphExec_t ge = nullptr;
+        const cudaError_t ec = cudaStreamEndCapture(ctx->cap_stream, &g);
+        if (e == cudaSuccess) e = ec;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&ge, g, 0);
+        if (g) cudaGraphDestroy(g);
+        const unsigned n = (unsigned)(launches_now() - before);      // noted by the capture: the first launch
+        if (e == cudaSuccess) e = cudaGraphLaunch(ge, s);
+        if (e == cudaSuccess) e = cudaEventRecord(a, s);
+        if (e == cudaSuccess) { e = cudaGraphLaunch(ge, s); note_launch(n); }
+        if (e == cudaSuccess) e = cudaEventRecord(b, s);
+        if (e == cudaSuccess) e = cudaEventSynchronize(b);
+        if (ge) cudaGraphExecDestroy(ge);
+        CK(e);
+    } else {
+        for (int r = 0; r < 2; ++r) CK(body(s));
+        CK(cudaEventRecord(a, s));
+        for (int r = 0; r < reps; ++r) CK(body(s));
+        CK(cudaEventRecord(b, s));
+        CK(cudaEventSynchronize(b));
+    }
     float t = 0.f;
     CK(cudaEventElapsedTime(&t, a, b));
     *ms = t / (float)reps;
@@ -220,7 +247,9 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
     CK(cudaEventCreate(&e1));
     TunedLevel best;
     int run_zc = 0;                 // the chosen stencil pass's chunk as a registration runs it
+    const bool graph = N <= 2000000;          // kernels of up to about 30 us
     const int reps = N > ((size_t)4 << 20) ? 5 : 20;
+    const int sreps = graph ? 10 : reps;      // of the five kernels of an iteration (a graph's build time grows with them)
     int rc = CGDIR_OK;
     {
         const int d = force_default_zchunk(nx, ny, nz);
@@ -229,8 +258,7 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
         // nx % 4 == 0) or two (twice the CTAs, for small levels)
         const int widths[2] = {0, 2};
         const int nw = nx % 4 == 0 && ctx->force_width == 0 ? 2 : 1;
-        const bool wave = N > 200000;
-        float bt = 1e30f;
+        float bt = 1e30f, dms = 0.f;
         for (int wi = 0; wi < nw && rc == CGDIR_OK; ++wi) {
             a.pass2_width = ctx->force_width > 0 ? ctx->force_width : widths[wi];
             for (int ci = 0; ci < 4 && rc == CGDIR_OK; ++ci) {
@@ -238,16 +266,10 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 for (int cj = 0; cj < ci; ++cj) seen = seen || cand[cj] == cand[ci];
                 if (seen) continue;
                 float ms = 0.f;
-                rc = time_ms(ctx, e0, e1, reps, &ms,
+                rc = time_ms(ctx, e0, e1, reps, graph, &ms,
                              [&](cudaStream_t st) { return launch_force(a, cand[ci], nullptr, st, kerr(ctx)); });
-                // within the noise of these timings (2 %) the wider thread
-                // and the longer chunk (fewer CTAs and halo planes) stand; on
-                // a level of less than a wave (where the default shape, too,
-                // takes one plane per thread) the shorter and narrower ones
-                const bool preferred = wave ? cand[ci] > best.force_zchunk && widths[wi] == best.force_width
-                                            : cand[ci] < best.force_zchunk ||
-                                                  (cand[ci] == best.force_zchunk && widths[wi] > best.force_width);
-                if (rc == CGDIR_OK && ms < (preferred ? 1.02f : 0.98f) * bt) {
+                if (wi == 0 && ci == 0) dms = ms;
+                if (rc == CGDIR_OK && ms < bt) {
                     bt = ms;
                     best.force_zchunk = cand[ci];
                     best.force_width = widths[wi];
@@ -255,11 +277,18 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 }
             }
         }
+        // the first (untuned) grouping stands where the best is not ahead of it
+        // by more than timings differ from run to run
+        if (dms <= 1.03f * bt) {
+            best.force_zchunk = d;
+            best.force_width = widths[0];
+            best.force_ms = dms;
+        }
         // the untuned schedule
         ForceArgs b = a;
         const int zc = force_schedule(ctx, b, -1);
         if (rc == CGDIR_OK)
-            rc = time_ms(ctx, e0, e1, reps, &best.default_force_ms,
+            rc = time_ms(ctx, e0, e1, reps, graph, &best.default_force_ms,
                          [&](cudaStream_t st) { return launch_force(b, zc, nullptr, st, kerr(ctx)); });
         a.pass2_width = ctx->force_width > 0 ? ctx->force_width : best.force_width;
         run_zc = best.force_zchunk;
@@ -315,9 +344,9 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
             // timing the tile and split kernels in full takes the tuner half
             // as long again there (213x248x48, three levels: 65 against 55 ms)
             const bool trial = nx % 4 != 0 && ci > 0;
-            rc = time_ms(ctx, e0, e1, trial ? 4 : reps, &ms, iteration);
+            rc = time_ms(ctx, e0, e1, trial ? 4 : sreps, graph, &ms, iteration);
             if (rc == CGDIR_OK && trial && ms - best.force_ms < 1.2f * bt + 2e-3f)
-                rc = time_ms(ctx, e0, e1, reps, &ms, iteration);
+                rc = time_ms(ctx, e0, e1, sreps, graph, &ms, iteration);
             else if (trial && !untuned)
                 continue;
             ms = std::max(ms - best.force_ms, 0.f);
@@ -336,10 +365,10 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
         ForceArgs a2 = a;
         a2.skip_warp = 1;
         float f2 = 0.f, fs = 0.f;
-        rc = time_ms(ctx, e0, e1, reps, &f2,
+        rc = time_ms(ctx, e0, e1, reps, graph, &f2,
                      [&](cudaStream_t st) { return launch_force(a2, run_zc, nullptr, st, kerr(ctx)); });
         if (rc == CGDIR_OK)    // timed after the stencil pass, as in an iteration
-            rc = time_ms(ctx, e0, e1, reps, &fs, [&](cudaStream_t st) {
+            rc = time_ms(ctx, e0, e1, sreps, graph, &fs, [&](cudaStream_t st) {
                 cudaError_t e = launch_force(a2, run_zc, nullptr, st, kerr(ctx));
                 if (e != cudaSuccess) return e;
                 e = launch_fused_smooth_compose(du, u, CGDIR_COMPOSE, sigma, nx, ny, nz, out, nullptr, kerr(ctx), st);

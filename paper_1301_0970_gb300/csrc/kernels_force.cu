@@ -1584,10 +1584,10 @@ int force_default_zchunk(int nx, int ny, int nz) {
     return pick_zchunk(nz, (long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY), 4, 2);
 }
 
-// What pass 2 does that no tuning table or setting names.  The chains of the
-// RMS-ID sums are always those of the widest thread and the chunk above, so
-// the histories do not depend on the schedule, which differs from them on
-// small levels:
+// What pass 2 does where no tuning table or setting names it.  The chains of
+// the RMS-ID sums are always those of the widest thread and the chunk above,
+// so an untuned level's history does not depend on the schedule, which differs
+// from them on small levels (a table's chunk and width bring their own chains):
 //  * with structure terms a voxel at a structure border loads its P_j after
 //    its bits are known, once per voxel of the thread: one or two voxels per
 //    thread instead of four, and one plane on the smallest levels (per
