@@ -222,6 +222,10 @@ int smooth_auto_variant(int nx, int ny, int nz, bool scratch);
 cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int ny, int nz,
                           float *out, const int *stop_flag, cudaStream_t s, int *err = nullptr,
                           SmoothChoice ch = SmoothChoice(), float *scratch = nullptr);
+// Self-test: the z-march of a 32 x 32 x nz field that never gets its plane
+// `hold`, by TMA or asynchronous copies; waits end after `limit` cycles.
+cudaError_t launch_smooth_wait_selftest(const float *in, float *out, int nz, int zchunk, int hold, bool tma,
+                                        long long limit, int *err, cudaStream_t s);
 cudaError_t launch_compose(const float *u, const float *du, int mode, int nx, int ny, int nz,
                            float *out, const int *stop_flag, cudaStream_t s);
 // Algorithm A steps 2 + 3: out = G(du) + u(x + G(du)) (or u + G(du)).  By

@@ -410,10 +410,13 @@ struct MarchGeom {
     static_assert(W / 4 % 2 == 1, "odd number of 16-byte units per row");
 };
 
-template <int R, int RY, bool ASYNC>
+// SELF: the self-test's form, in which the loads of plane `hold` are never
+// issued and every wait ends after `limit` cycles.
+template <int R, int RY, bool ASYNC, bool SELF = false>
 __global__ void __launch_bounds__(MT, RY == 4 ? 4 : MarchGeom<R, RY>::CTAS)
     k_smooth_march(const __grid_constant__ CUtensorMap tin, const float *__restrict__ in, float *__restrict__ out,
-                   Taps taps, int nx, int ny, int nz, int zchunk, const int *stop_flag, int *err) {
+                   Taps taps, int nx, int ny, int nz, int zchunk, const int *stop_flag, int *err, int hold = -1,
+                   long long limit = kWaitLimitCycles) {
     if (stopped(stop_flag)) return;      // (acted on later, the kernel takes 21 registers more and a CTA less)
     using G = MarchGeom<R, RY>;
     constexpr int K = G::K, BY = G::BY, ML = G::ML, W = G::W, ST = G::ST, STAGE = G::STAGE, XB = G::XB, TPT = G::TPT;
@@ -461,6 +464,7 @@ __global__ void __launch_bounds__(MT, RY == 4 ? 4 : MarchGeom<R, RY>::CTAS)
     // (one thread; with ASYNC every thread)
     auto issue = [&](int q, int so, uint64_t *b) {
         const int z = clampi(zb - R + q, 0, nz - 1);
+        if (SELF && q == hold) return;
         if (!ASYNC) {
             mbar_expect_tx(b, (uint32_t)(BY * W * sizeof(float)));
             tma_load_4d(stage0 + so, &tin, x0 - ML, y0 - R, z, comp, b);
@@ -548,9 +552,12 @@ __global__ void __launch_bounds__(MT, RY == 4 ? 4 : MarchGeom<R, RY>::CTAS)
         *reinterpret_cast<float4 *>(d + 4) = make_float4(o[2].x, o[2].y, o[3].x, o[3].y);
     };
 
+    auto wait = [&](uint64_t *b, uint32_t parity) {
+        return SELF ? mbar_wait_bounded(b, parity, limit) : mbar_wait_bounded(b, parity);
+    };
     // tw: the plane whose wait ran out in this thread (-1: none); it skips the
-    // later waits, and the CTA leaves at the next turn of the plane loop,
-    // where its threads agree on it
+    // later waits, and the CTA leaves at the next turn of the plane loop or
+    // after the last plane, where its threads agree on it
     int tw = -1;
     bool leave = false;
     uint32_t par = 0;                   // phase parity of the current stage
@@ -562,7 +569,7 @@ __global__ void __launch_bounds__(MT, RY == 4 ? 4 : MarchGeom<R, RY>::CTAS)
         for (int r = 0; r < K; ++r) {
             const int t = t0 + r;
             if (t >= P) break;
-            if (xt[0] && tw < 0 && !mbar_wait_bounded(bcur, par)) tw = t;
+            if (xt[0] && tw < 0 && !wait(bcur, par)) tw = t;
 #pragma unroll
             for (int q = 0; q < TPT; ++q) {
                 const int xg = xdst[q] % W;
@@ -617,15 +624,16 @@ __global__ void __launch_bounds__(MT, RY == 4 ? 4 : MarchGeom<R, RY>::CTAS)
         }
         if (leave) break;
     }
+    if (!leave) leave = __syncthreads_or(tw >= 0);
     if (leave) {
-        // record it, let the loads in flight land (bounded waits), leave
-        if (ASYNC) {
-            cp_async_wait_all();
-            if (tid == 0) atomicExch(err, 1);
-        } else if (tid == kIssuer) {
+        // record it, let the loads in flight land (bounded waits), leave.  The
+        // issuer has issued the planes below qe (with ASYNC every thread has,
+        // whatever its waits did), and waited for all of them but the last ST.
+        if (ASYNC) cp_async_wait_all();
+        if (tid == kIssuer) {
             atomicExch(err, 1);
-            const int q0 = tw >= 0 ? tw : t0 + 1, q1 = min((tw >= 0 ? tw : t0) + ST, P);
-            for (int q = q0; q < q1; ++q) mbar_wait_bounded(&bar[q % ST], (uint32_t)((q / ST) & 1));
+            const int qe = min((!ASYNC && tw >= 0 ? tw : t0) + ST, P);
+            for (int q = max(qe - ST, 0); q < qe; ++q) wait(&bar[q % ST], (uint32_t)((q / ST) & 1));
         }
         __syncthreads();
     }
@@ -1093,6 +1101,30 @@ static cudaError_t smooth_march_r(const float *in, float *out, int ncomp, const 
         k_smooth_march<R, RY, false><<<grid, MT, smem, s>>>(m, in, out, t, nx, ny, nz, zc, stop_flag, err);
     else
         k_smooth_march<R, RY, true><<<grid, MT, smem, s>>>(m, in, out, t, nx, ny, nz, zc, stop_flag, err);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// The z-march of a 32 x 32 x nz field (radius 3) whose plane `hold` (counted
+// from the chunk's first halo plane) never arrives.
+cudaError_t launch_smooth_wait_selftest(const float *in, float *out, int nz, int zchunk, int hold, bool tma,
+                                        long long limit, int *err, cudaStream_t s) {
+    using G = MarchGeom<3, 4>;
+    CUtensorMap m{};
+    const uint64_t dims[4] = {32, 32, (uint64_t)nz, 1};
+    const uint32_t box[4] = {(uint32_t)G::W, (uint32_t)G::BY, 1u, 1u};
+    if (tma && !encode_tensor_map(&m, in, 4, dims, box, 4)) return cudaErrorInvalidValue;
+    const dim3 grid(1, 1, (nz + zchunk - 1) / zchunk);
+    const Taps t = gauss_taps(1.f);
+    const void *f = tma ? (const void *)k_smooth_march<3, 4, false, true> : (const void *)k_smooth_march<3, 4, true, true>;
+    cudaError_t e = ensure_smem(f, G::bytes());
+    if (e != cudaSuccess) return e;
+    if (tma)
+        k_smooth_march<3, 4, false, true><<<grid, MT, G::bytes(), s>>>(m, in, out, t, 32, 32, nz, zchunk, nullptr, err,
+                                                                       hold, limit);
+    else
+        k_smooth_march<3, 4, true, true><<<grid, MT, G::bytes(), s>>>(m, in, out, t, 32, 32, nz, zchunk, nullptr, err,
+                                                                      hold, limit);
     note_launch();
     return cudaGetLastError();
 }

@@ -154,3 +154,18 @@ def test_rows_without_tma_take_the_split_kernels_with_the_same_bits(monkeypatch,
             ctx.sync()
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("limit_us", [200, 1000])
+def test_march_reports_a_plane_that_never_arrives(limit_us):
+    """Every plane's wait is reported, also in the last turn of the plane loop
+    (the self-test withholds the first, a middle and the last plane of chunks of
+    1 and 20 planes, by TMA and by asynchronous copies), and the context and its
+    smoothing work afterwards."""
+    f = torch.randn(3, 20, 32, 32, device=DEV)
+    with cg.Context(0) as c:
+        want = c.smooth(f, 1.0)
+        assert c.selftest_wait_timeout(limit_us) == cg.CGDIR_ETIMEDOUT
+        got = c.smooth(f, 1.0)
+        c.sync()
+    assert torch.equal(got, want)
