@@ -459,9 +459,10 @@ int cgdir_profile_read(const cgdir_ctx *ctx, cgdir_kernel_time *out, int cap);
    that nothing completes; the wait runs out, the kernel records it in the
    context's error word and returns, and the call reports it as a kernel
    wait that ran out.  Then (limit at most 1 ms) the z-march smoothing runs
-   on fields one plane of which is never copied, and has to report it.
-   Returns CGDIR_ETIMEDOUT when the paths work (the context stays usable);
-   EINVAL for a bad limit; ECUDA. */
+   on fields one plane of which is never copied and the fused tile kernel on
+   tiles that are never copied (of a running and of a stopped level); both
+   have to report it.  Returns CGDIR_ETIMEDOUT when the paths work (the
+   context stays usable); EINVAL for a bad limit; ECUDA. */
 int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us);
 
 /* ---- autotuner (not in the paper: an execution choice) --------------------

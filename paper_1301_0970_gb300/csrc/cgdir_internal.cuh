@@ -249,6 +249,10 @@ cudaError_t launch_fused_smooth_compose(const float *du, const float *u, int mod
 //   next iteration's warp
 cudaError_t launch_fused_smooth_warp(const float *in, float sigma, float *u, const ForceArgs &a, int *err,
                                      cudaStream_t s);
+// Self-test: the first of these kernels on a 16 x 16 x 16 field whose tiles are
+// never loaded; waits end after `limit` cycles.
+cudaError_t launch_fused_wait_selftest(const float *field, float *out, const int *stop_flag, long long limit, int *err,
+                                       cudaStream_t s);
 // Whether the fused schedule can run for this force configuration (the
 // two-pass force with 32-bit indexing).
 bool fused_schedule_ok(const ForceArgs &a);

@@ -75,14 +75,16 @@ struct FusedTile {
 
 // G(in) over the CTA's tile into Z (smem), all three components.  Returns
 // false (every thread) if the level has stopped or the TMA wait ran out; the
-// error word is set in the second case.
+// error word is set in the second case, stopped or not.
 // With umap, the u tile's TMA copy (completing on bar[1]) is issued as soon
 // as the input box has been read.
-template <int R>
+// SELF: the self-test's form, whose input box is never loaded and whose waits
+// end after `limit` cycles.
+template <int R, bool SELF>
 __device__ __forceinline__ bool tile_smooth(const CUtensorMap *tin, bool use_tma, const float *__restrict__ in,
                                             const Taps &t, int nx, int ny, int nz, int x0, int y0, int z0,
                                             float *S, float *X, uint64_t *bar, int *err, int tid, bool stop,
-                                            const CUtensorMap *umap = nullptr) {
+                                            const CUtensorMap *umap = nullptr, long long limit = 0) {
     using G = FusedTile<R>;
     constexpr int K = 2 * R + 1, A = G::A, ML = G::ML, W = G::W, XS = G::XS, XP = G::XP, YP = G::YP;
     float2 w2[K];
@@ -93,20 +95,23 @@ __device__ __forceinline__ bool tile_smooth(const CUtensorMap *tin, bool use_tma
             mbar_init(bar, 1);
             if (umap) mbar_init(bar + 1, 1);
             fence_mbar_init();
-            mbar_expect_tx(bar, (uint32_t)(G::SN * sizeof(float)));
-            tma_load_4d(S, tin, x0 - ML, y0 - R, z0 - R, 0, bar);
+            if (!SELF) {
+                mbar_expect_tx(bar, (uint32_t)(G::SN * sizeof(float)));
+                tma_load_4d(S, tin, x0 - ML, y0 - R, z0 - R, 0, bar);
+            }
         }
         __syncthreads();
-        const bool ok = mbar_wait_bounded(bar, 0);
-        if (stop) return false;                         // the box has landed; nothing else is in flight
+        auto wait = [&] { return SELF ? mbar_wait_bounded(bar, 0, limit) : mbar_wait_bounded(bar, 0); };
+        const bool ok = wait();
         if (__syncthreads_or(!ok)) {
             if (tid == 0) {
                 atomicExch(err, 1);
-                mbar_wait_bounded(bar, 0);              // let the copy land before leaving
+                wait();                                 // let the copy land before leaving
             }
             __syncthreads();
             return false;
         }
+        if (stop) return false;                         // the box has landed; nothing else is in flight
     } else {
         if (stop) return false;
         const int nxy = nx * ny, N = nxy * nz;
@@ -247,21 +252,22 @@ struct TileSmem {
 
 constexpr int kVoxPerThread = FQ * FQ * FQ / FT;          // 2
 
-template <int R>
+template <int R, bool SELF = false>
 __global__ void __launch_bounds__(FT, 3) k_fused_smooth_compose(const __grid_constant__ CUtensorMap tin, int use_tma,
                                                               const __grid_constant__ CUtensorMap umap,
                                                               const float *__restrict__ du,
                                                               const float *__restrict__ u, int mode, Taps t,
                                                               int nx, int ny, int nz, float *__restrict__ out,
-                                                              const int *stop_flag, int *err) {
+                                                              const int *stop_flag, int *err,
+                                                              long long limit = 0) {
     const bool stop = stopped(stop_flag);
     extern __shared__ __align__(128) unsigned char smem_raw[];
     TileSmem<R> sm(smem_raw);
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * FQ, y0 = blockIdx.y * FQ, z0 = blockIdx.z * FQ;
     const bool utile = use_tma != 0 && mode != CGDIR_ADDITIVE;
-    if (!tile_smooth<R>(&tin, use_tma != 0, du, t, nx, ny, nz, x0, y0, z0, sm.S, sm.X, sm.bar, err, tid, stop,
-                        utile ? &umap : nullptr))
+    if (!tile_smooth<R, SELF>(&tin, use_tma != 0, du, t, nx, ny, nz, x0, y0, z0, sm.S, sm.X, sm.bar, err, tid, stop,
+                              utile ? &umap : nullptr, limit))
         return;
     const float *Z = sm.X;
     const int nxy = nx * ny, N = nxy * nz;
@@ -368,7 +374,7 @@ __global__ void __launch_bounds__(FT) k_fused_smooth_warp(const __grid_constant_
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * FQ, y0 = blockIdx.y * FQ, z0 = blockIdx.z * FQ;
-    if (!tile_smooth<R>(&tin, use_tma != 0, in, t, nx, ny, nz, x0, y0, z0, sm.S, sm.X, sm.bar, err, tid, stop)) return;
+    if (!tile_smooth<R, false>(&tin, use_tma != 0, in, t, nx, ny, nz, x0, y0, z0, sm.S, sm.X, sm.bar, err, tid, stop)) return;
     const float *Z = sm.X;
     const int nxy = nx * ny, N = nxy * nz;
     Cell cell[kVoxPerThread];
@@ -451,6 +457,20 @@ cudaError_t warp_r(const float *in, const Taps &t, float *u, const ForceArgs &a,
 }
 
 }  // namespace
+
+cudaError_t launch_fused_wait_selftest(const float *field, float *out, const int *stop_flag, long long limit, int *err,
+                                       cudaStream_t s) {
+    constexpr int n = 16;
+    const size_t smem = FusedTile<3>::bytes();
+    cudaError_t e = ensure_smem((const void *)k_fused_smooth_compose<3, true>, smem);
+    if (e != cudaSuccess) return e;
+    CUtensorMap m{};
+    if (!tile_map<3>(&m, field, n, n, n)) return cudaErrorInvalidValue;
+    k_fused_smooth_compose<3, true><<<dim3(n / FQ, n / FQ, n / FQ), FT, smem, s>>>(
+        m, 1, m, field, field, CGDIR_ADDITIVE, gauss_taps(1.f), n, n, n, out, stop_flag, err, limit);
+    note_launch();
+    return cudaGetLastError();
+}
 
 bool fused_schedule_ok(const ForceArgs &a) {
     return a.wfield != nullptr && (!(a.contour && a.k > 0) || a.mtex != nullptr) &&

@@ -4,7 +4,8 @@
 // timeout in the context's error word and returns -- what the TMA kernels do
 // when a copy never lands.  Then the z-march smoothing runs on fields one plane
 // of which is never copied: it has to report that plane wherever its wait runs
-// out.  Nothing faults or hangs: every wait is bounded.
+// out; and the fused tile kernel on tiles that are never copied, of a running
+// and of a stopped level.  Nothing faults or hangs: every wait is bounded.
 #include "runtime_internal.hpp"
 #include "tma.cuh"
 
@@ -46,21 +47,31 @@ extern "C" int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us) {
     const int rc = check_err_word(ctx);
     if (rc != CGDIR_ETIMEDOUT) return rc;
     constexpr int nz = 20;
+    constexpr size_t n = nz * 32 * 32;             // >= 3 x 16 x 16 x 16
     void *f = nullptr;
-    TRY(ws_get(ctx, "selftest", 2 * (size_t)nz * 32 * 32 * sizeof(float), &f));
-    float *in = (float *)f, *out = in + nz * 32 * 32;
-    CK(cudaMemsetAsync(in, 0, (size_t)nz * 32 * 32 * sizeof(float), ctx->stream));
+    TRY(ws_get(ctx, "selftest", (2 * n + 1) * sizeof(float), &f));
+    float *in = (float *)f, *out = in + n;
+    int *stop = (int *)(out + n);
+    CK(cudaMemsetAsync(in, 0, n * sizeof(float), ctx->stream));
+    const long long limit = std::min<long long>(cycles, 2100000);
     // first, middle and last plane of one turn of the plane loop (chunks of
     // one plane march 7 planes) and of a chunk whose last turn is cut short
     const int at[6][2] = {{1, 0}, {1, 3}, {1, 6}, {nz, 0}, {nz, 21}, {nz, 25}};
     for (const auto &q : at)
         for (int tma = 0; tma < 2; ++tma) {
-            CK(launch_smooth_wait_selftest(in, out, nz, q[0], q[1], tma != 0, std::min<long long>(cycles, 2100000),
-                                           ctx->err_word, ctx->stream));
+            CK(launch_smooth_wait_selftest(in, out, nz, q[0], q[1], tma != 0, limit, ctx->err_word, ctx->stream));
             CK(cudaStreamSynchronize(ctx->stream));
             const int rs = check_err_word(ctx);
             if (rs == CGDIR_OK) return fail(ctx, CGDIR_ECUDA, "selftest: the z-march lost a wait that ran out");
             if (rs != CGDIR_ETIMEDOUT) return rs;
         }
+    for (int stopped = 0; stopped < 2; ++stopped) {
+        CK(cudaMemsetAsync(stop, stopped, sizeof(int), ctx->stream));
+        CK(launch_fused_wait_selftest(in, out, stop, limit, ctx->err_word, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        const int rs = check_err_word(ctx);
+        if (rs == CGDIR_OK) return fail(ctx, CGDIR_ECUDA, "selftest: the fused tiles lost a wait that ran out");
+        if (rs != CGDIR_ETIMEDOUT) return rs;
+    }
     return rc;
 }
