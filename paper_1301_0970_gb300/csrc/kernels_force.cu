@@ -1603,7 +1603,7 @@ ForceShape force_default_shape(int nx, int ny, int nz, bool contour) {
     const int zc = force_default_zchunk(nx, ny, nz);
     ForceShape f{zc, 0, 0, 0};
     if (nx % 4 == 0) {
-        if (contour && N <= 1600000) {
+        if (contour && N <= 1600000 && nz <= 4 * 65535) {      // (its grid holds 65535 chunks)
             f.width = N > 200000 && N <= 600000 ? 1 : 2;
             f.zchunk = N <= 200000 ? 1 : std::min(4, nz);
             f.chain_w = 4;

@@ -1157,11 +1157,18 @@ static cudaError_t smooth_march(const float *in, float *out, int ncomp, const Ta
 // the tile's 15.9 + 12.4 us, 256x256x96 96 + 36 against the split's 139 + 94).
 constexpr size_t kSplitVoxels = 8000000;
 
+// Whether the grid of the split kernels or of the tile kernel, z slabs times
+// components, holds a volume this deep (the z-march's always does).
+static bool grid_holds(int variant, int nz, int ncomp) {
+    const int slab = variant == SMOOTH_SPLIT ? XYZ : variant == SMOOTH_TILE ? QZ : 0;
+    return slab == 0 || ((long)nz + slab - 1) / slab * ncomp <= 65535;
+}
+
 int smooth_auto_variant(int nx, int ny, int nz, bool scratch) {
     const size_t N = (size_t)nx * ny * nz;
     if (nx % 4 == 0) return SMOOTH_MARCH;
-    if (scratch && N <= kSplitVoxels) return SMOOTH_SPLIT;
-    return N <= 250000 ? SMOOTH_TILE : SMOOTH_MARCH;
+    if (scratch && N <= kSplitVoxels && grid_holds(SMOOTH_SPLIT, nz, 3)) return SMOOTH_SPLIT;
+    return N <= 250000 && grid_holds(SMOOTH_TILE, nz, 3) ? SMOOTH_TILE : SMOOTH_MARCH;
 }
 
 int smooth_default_zchunk(int nx, int ny, int nz, int ncomp, float sigma) {
@@ -1265,6 +1272,7 @@ cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int n
         if (variant == SMOOTH_AUTO && ch.zchunk == 0)
             variant = smooth_auto_variant(nx, ny, nz, scratch != nullptr && scratch != in && scratch != out);
         if (variant == SMOOTH_FUSED) variant = SMOOTH_TILE;     // nothing to fuse with here
+        if (!grid_holds(variant, nz, ncomp)) variant = SMOOTH_MARCH;
         if (variant == SMOOTH_TILE) return smooth_tile(in, ncomp, t, nx, ny, nz, out, stop_flag, s);
         if (variant == SMOOTH_SPLIT && scratch != nullptr && scratch != in && scratch != out)
             return smooth_split(in, nullptr, 0, false, ncomp, t, nx, ny, nz, out, scratch, ch.zchunk, stop_flag, s);
@@ -1280,7 +1288,8 @@ cudaError_t launch_smooth_compose(const float *du, const float *u, int mode, flo
     const Taps t = gauss_taps(sigma);
     if (!one_pass && t.r > 0 && err != nullptr) {
         if (ch.variant == SMOOTH_AUTO && ch.zchunk == 0) ch.variant = smooth_auto_variant(nx, ny, nz, tmp != nullptr);
-        if (ch.variant == SMOOTH_SPLIT)   // x/y pass, then the z pass with the composite update fused
+        if (ch.variant == SMOOTH_SPLIT && grid_holds(SMOOTH_SPLIT, nz, 3))   // x/y pass, then the z pass with the
+                                                                              // composite update fused
             return smooth_split(du, u, mode, true, 3, t, nx, ny, nz, out, tmp, ch.zchunk, stop_flag, s);
         if (ch.variant == SMOOTH_FUSED && (size_t)nx * ny * nz < (size_t)1 << 31)   // one 3-D tile kernel
             return launch_fused_smooth_compose(du, u, mode, sigma, nx, ny, nz, out, stop_flag, err, s);

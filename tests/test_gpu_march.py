@@ -169,3 +169,25 @@ def test_march_reports_a_plane_that_never_arrives(limit_us):
         got = c.smooth(f, 1.0)
         c.sync()
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("shape", [(100000, 1, 1), (90000, 9, 9), (200000, 1, 1), (270000, 1, 4)])
+def test_volumes_deeper_than_a_grid_of_slabs(shape, monkeypatch):
+    """Thin volumes of more z slabs than a grid's z extent holds run, with the
+    z-march's bits, in every step that smooths, and so do their force steps."""
+    torch.manual_seed(1)
+    du = torch.randn((3,) + shape, device=DEV)
+    u = torch.randn((3,) + shape, device=DEV)
+    img = torch.randn(shape, device=DEV)
+    bits = torch.randint(0, 2, shape, device=DEV, dtype=torch.uint8)
+    got = []
+    for forced in (None, "split", "march"):
+        if forced:
+            monkeypatch.setenv("CGDIR_SMOOTH", forced)
+        with cg.Context(0) as c:
+            got.append([c.smooth_compose(du, u, sigma=1.0), c.smooth(du, 1.0),
+                        c.iterate(img, img, bits, bits, [1e-3], [1], u, contour=True)])
+            c.sync()
+    for other in got[:2]:
+        for a, b in zip(other, got[2]):
+            assert torch.equal(a, b)
