@@ -1652,7 +1652,7 @@ static cudaError_t launch_force_t(const ForceArgs &a, int zchunk, dim3 grid, dim
         const bool quad = pass2_quad(a);
         const bool paired = a.nx % 2 == 0 && a.pass2_width != 1;
         ForceArgs b = a;
-        if (a.chain_w == 4 && (quad || !quad_aligned(a))) b.chain_w = b.chain_z = 0;      // the threads' own
+        if (a.chain_w == 4 && quad) b.chain_w = b.chain_z = 0;      // the threads' own
         dim3 g2 = quad ? dim3((a.nx / 4 + TX - 1) / TX, grid.y, grid.z)
                        : paired ? dim3((a.nx / 2 + TX - 1) / TX, grid.y, grid.z) : grid;
         const bool warp = !a.skip_warp;
@@ -1710,7 +1710,16 @@ static cudaError_t launch_force_t(const ForceArgs &a, int zchunk, dim3 grid, dim
     return cudaGetLastError();
 }
 
-cudaError_t launch_force(const ForceArgs &a, int zchunk, int *nblocks_out, cudaStream_t s, int *err) {
+cudaError_t launch_force(const ForceArgs &args, int zchunk, int *nblocks_out, cudaStream_t s, int *err) {
+    ForceArgs a = args;
+    // chains of quads stand for the widest thread and a chunk of chain_z; where
+    // a field's quads cannot be loaded (the fields of a coarse level under a
+    // finest one whose voxel count is no multiple of 4), that schedule itself
+    // runs, with the width that the fields allow
+    if (a.chain_w == 4 && !quad_aligned(a)) {
+        zchunk = a.chain_z;
+        a.pass2_width = a.chain_w = a.chain_z = 0;
+    }
     if (zchunk <= 0) zchunk = force_default_zchunk(a.nx, a.ny, a.nz);
     dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, (a.nz + zchunk - 1) / zchunk);
     dim3 block(TX, TY);

@@ -191,3 +191,25 @@ def test_volumes_deeper_than_a_grid_of_slabs(shape, monkeypatch):
     for other in got[:2]:
         for a, b in zip(other, got[2]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("shape", [(21, 33, 63), (43, 61, 127)])
+def test_unaligned_coarse_level_keeps_its_history(shape, monkeypatch):
+    """A coarse level with whole quads in fields that start at no quad's
+    boundary (the finest level has an odd number of voxels): its RMS-ID history
+    with structure terms is the one of the default chunk."""
+    rng = np.random.default_rng(hash_of(shape))
+    img = rng.normal(0, 300, shape).astype(np.float32)
+    mov = torch.from_numpy(img + rng.normal(0, 40, shape).astype(np.float32)).to(DEV)
+    img = torch.from_numpy(img).to(DEV)
+    masks = [torch.from_numpy((rng.random(shape) < 0.3).astype(np.uint8)).to(DEV)]
+    kw = dict(levels=2, iters=[4, 1], lam=[1e-3], sign=[1], contour_level_mask=3, stop_mode=cg.CGDIR_STOP_FIXED)
+    coarse = tuple((n + 1) // 2 for n in shape)
+    got = []
+    for zc in (None, default_zchunk(coarse)):
+        if zc:
+            monkeypatch.setenv("CGDIR_FORCE_ZCHUNK", str(zc))
+        with cg.Context(0) as c:
+            got.append(c.register(img, mov, masks, masks, **kw))
+    assert torch.equal(got[0][0], got[1][0])
+    assert got[0][1][0]["rms_id"] == got[1][1][0]["rms_id"]
