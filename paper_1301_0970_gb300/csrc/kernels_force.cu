@@ -1638,6 +1638,14 @@ static bool quad_aligned(const ForceArgs &a) {
            al(a.du, 16) && al(a.warped, 16) && al(a.uroi, 4) && al(a.sbits, 4);
 }
 static bool pass2_quad(const ForceArgs &a) { return a.pass2_width == 0 && quad_aligned(a); }
+// Two voxels per thread: even rows and fields aligned for pairs (a caller's
+// view may start anywhere; one voxel per thread takes those).
+static bool pass2_paired(const ForceArgs &a) {
+    auto al = [](const void *p, unsigned b) { return p == nullptr || ((uintptr_t)p & (b - 1)) == 0; };
+    const unsigned tb = a.img_dtype == CGDIR_F32 ? 8u : 4u;
+    return a.nx % 2 == 0 && a.pass2_width != 1 && al(a.wfield, 8) && al(a.wstate, 4) && al(a.T0, tb) &&
+           al(a.du, 8) && al(a.uroi, 2) && al(a.sbits, 2);
+}
 
 template <typename IT>
 static cudaError_t launch_force_t(const ForceArgs &a, int zchunk, dim3 grid, dim3 block, cudaStream_t s,
@@ -1650,7 +1658,7 @@ static cudaError_t launch_force_t(const ForceArgs &a, int zchunk, dim3 grid, dim
         // pass 2 marches the caller's (longer) z chunks: fewer CTAs, so fewer
         // end-of-block fences before the fused reduction
         const bool quad = pass2_quad(a);
-        const bool paired = a.nx % 2 == 0 && a.pass2_width != 1;
+        const bool paired = pass2_paired(a);
         ForceArgs b = a;
         if (a.chain_w == 4 && quad) b.chain_w = b.chain_z = 0;      // the threads' own
         dim3 g2 = quad ? dim3((a.nx / 4 + TX - 1) / TX, grid.y, grid.z)
@@ -1726,7 +1734,7 @@ cudaError_t launch_force(const ForceArgs &args, int zchunk, int *nblocks_out, cu
     if (nblocks_out) *nblocks_out = (int)(grid.x * grid.y * grid.z);
     if (nblocks_out && a.wfield != nullptr && (size_t)a.nx * a.ny * a.nz < (size_t)1 << 31) {
         if (pass2_quad(a)) *nblocks_out = (int)(((a.nx / 4 + TX - 1) / TX) * grid.y * grid.z);
-        else if (a.nx % 2 == 0 && a.pass2_width != 1)
+        else if (pass2_paired(a))
             *nblocks_out = (int)(((a.nx / 2 + TX - 1) / TX) * grid.y * grid.z);   // paired pass 2
     }
 

@@ -213,3 +213,30 @@ def test_unaligned_coarse_level_keeps_its_history(shape, monkeypatch):
             got.append(c.register(img, mov, masks, masks, **kw))
     assert torch.equal(got[0][0], got[1][0])
     assert got[0][1][0]["rms_id"] == got[1][1][0]["rms_id"]
+
+
+@pytest.mark.parametrize("nx", [6, 32, 34])
+@pytest.mark.parametrize("which", ["T0", "du", "uroi", "sbits"])
+def test_force_on_views_that_start_at_an_odd_element(ctx, nx, which):
+    """Force fields that are views one element into their storage (no pair of
+    voxels is aligned): the same du and the same count as for aligned copies,
+    the RMS sum to the rounding of its FP32 parts (a few dozen terms each)."""
+    shape = (7, 9, nx)
+    gen = torch.Generator(device=DEV).manual_seed(nx)
+    img, mov = (300 * torch.randn(shape, device=DEV, generator=gen) for _ in range(2))
+    bits = torch.randint(0, 4, shape, device=DEV, dtype=torch.uint8, generator=gen)
+    uroi = torch.randint(0, 2, shape, device=DEV, dtype=torch.uint8, generator=gen)
+    u = torch.randn((3,) + shape, device=DEV, generator=gen)
+
+    def run(odd):
+        a = {"T0": img, "du": torch.empty_like(u), "uroi": uroi, "sbits": bits}
+        if odd:
+            t = torch.empty(a[which].numel() + 1, device=DEV, dtype=a[which].dtype)[1:].view(a[which].shape)
+            a[which] = t.copy_(a[which])
+        return ctx.force(mov, a["T0"], bits, a["sbits"], [1e-3] * 2, [1, -1], u, uroi=a["uroi"], du=a["du"],
+                         want_stats=True)
+
+    (du, st), (want, wst) = run(True), run(False)
+    assert torch.equal(du, want)
+    assert st[1] == wst[1] and st[2] == wst[2]
+    assert abs(st[0] - wst[0]) <= 64 * 2.0 ** -24 * wst[0]
