@@ -107,13 +107,13 @@ bool use_level_coop(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, i
     return (long)nx * ny * nz <= ctx->coop_max_voxels;
 }
 
-// Voxels per thread of the force's stencil pass (0: the widest the shape
-// and alignment allow).
+// Voxels per thread and z chunk of the force's stencil pass as a setting or a
+// table names them, else the widest the shape and alignment allow and the
+// default chunk.
 int force_width_for(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt) {
     if (ctx->force_width > 0) return ctx->force_width;
     if (const TunedLevel *t = find_tuned(ctx, nx, ny, nz, contour, sdt)) return t->force_width;
-    if (ctx->force_zchunk > 0) return 0;
-    return force_default_shape(nx, ny, nz, contour != 0).width;
+    return 0;
 }
 
 // Never below force_zchunk_min: the registration's partial-sum buffer is
@@ -123,20 +123,21 @@ int force_zchunk_for(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, 
     if (ctx->force_zchunk > 0) return std::max(lo, std::min(ctx->force_zchunk, nz));
     if (const TunedLevel *t = find_tuned(ctx, nx, ny, nz, contour, sdt))
         if (t->force_zchunk > 0) return std::max(lo, std::min(t->force_zchunk, nz));
-    if (ctx->force_width > 0) return force_default_zchunk(nx, ny, nz);
-    return std::max(lo, force_default_shape(nx, ny, nz, contour != 0).zchunk);
+    return force_default_zchunk(nx, ny, nz);
 }
 
 // Pass 2's z chunk (returned) and its width and chains (in a) for a level.
 // A tuned level whose choice is the widest thread with the default chunk runs
 // the untuned schedule: the same sums, on more threads where the level is
-// small.
+// small.  That schedule is the two-pass kernels' own: the plain kernel warps
+// chunk + 2 planes per chunk, and neither it nor the one-pass kernel moves its
+// chains to other threads.
 int force_schedule(const cgdir_ctx *ctx, ForceArgs &a, int sdt) {
     const int contour = a.contour && a.k > 0;
     a.pass2_width = force_width_for(ctx, a.nx, a.ny, a.nz, contour, sdt);
     a.chain_w = a.chain_z = 0;
     const int zc = force_zchunk_for(ctx, a.nx, a.ny, a.nz, contour, sdt);
-    if (ctx->force_width > 0 || ctx->force_zchunk > 0) return zc;
+    if (ctx->force_width > 0 || ctx->force_zchunk > 0 || ctx->plain_kernels || ctx->fused_force) return zc;
     if (find_tuned(ctx, a.nx, a.ny, a.nz, contour, sdt) &&
         (a.pass2_width != 0 || zc != force_default_zchunk(a.nx, a.ny, a.nz)))
         return zc;

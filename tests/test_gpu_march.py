@@ -240,3 +240,28 @@ def test_force_on_views_that_start_at_an_odd_element(ctx, nx, which):
     assert torch.equal(du, want)
     assert st[1] == wst[1] and st[2] == wst[2]
     assert abs(st[0] - wst[0]) <= 64 * 2.0 ** -24 * wst[0]
+
+
+@pytest.mark.parametrize("kernels", ["plain", "fused"])
+@pytest.mark.parametrize("shape", [(9, 21, 44), (30, 40, 64), (13, 22, 45)])
+def test_other_kernel_families_keep_the_default_chunk(shape, kernels, monkeypatch):
+    """The plain and the one-pass force kernels run small levels with the
+    default chunk: histories and statistics bit for bit."""
+    rng = np.random.default_rng(hash_of(shape))
+    img = rng.normal(0, 300, shape).astype(np.float32)
+    mov = torch.from_numpy(img + rng.normal(0, 40, shape).astype(np.float32)).to(DEV)
+    img = torch.from_numpy(img).to(DEV)
+    masks = [torch.from_numpy((rng.random(shape) < 0.3).astype(np.uint8)).to(DEV)]
+    u = torch.from_numpy(rng.normal(0, 1, (3,) + shape).astype(np.float32)).to(DEV)
+    monkeypatch.setenv("CGDIR_KERNELS", kernels)
+    got = []
+    for zc in (None, default_zchunk(shape)):
+        if zc:
+            monkeypatch.setenv("CGDIR_FORCE_ZCHUNK", str(zc))
+        with cg.Context(0) as c:
+            dvf, st = c.register(img, mov, masks, masks, levels=1, iters=[4], lam=[1e-3], sign=[1],
+                                 stop_mode=cg.CGDIR_STOP_FIXED)
+            _, stats = c.force(mov, img, masks[0], masks[0], [1e-3], [1], u, want_stats=True)
+            got.append((dvf, st[0]["rms_id"], stats))
+    assert torch.equal(got[0][0], got[1][0])
+    assert got[0][1:] == got[1][1:]
