@@ -291,6 +291,10 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
         if (rc == CGDIR_OK)
             rc = time_ms(ctx, e0, e1, reps, graph, &best.default_force_ms,
                          [&](cudaStream_t st) { return launch_force(b, zc, nullptr, st, kerr(ctx)); });
+        if (ctx->force_width == 0 && best.default_force_ms <= best.force_ms) {
+            best.force_zchunk = d;
+            best.force_width = 0;
+        }
         a.pass2_width = ctx->force_width > 0 ? ctx->force_width : best.force_width;
         run_zc = best.force_zchunk;
         if (best.force_width == 0 && best.force_zchunk == d) {      // runs the untuned schedule
@@ -377,14 +381,15 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 return launch_fused_smooth_warp(out, sigma, u, a2, kerr(ctx), st);
             });
         fs = std::max(fs - f2, 0.f);
-        if (rc == CGDIR_OK && smooth_choice(ctx, nx, ny, nz, contour, -1, true, sigma).variant == SMOOTH_FUSED) {
-            best.default_smooth_ms = fs;                   // the untuned choice is the fused schedule
+        const bool dflt = smooth_choice(ctx, nx, ny, nz, contour, -1, true, sigma).variant == SMOOTH_FUSED;
+        if (rc == CGDIR_OK && dflt) {                      // the untuned choice is the fused schedule
+            best.default_smooth_ms = fs;
             best.default_force_ms = f2;
         }
-        // by 5 %: each of the four spans is timed behind another kernel and
-        // taken off it (72x184x96: estimated ahead, 95 us per iteration
-        // against 89)
-        if (rc == CGDIR_OK && f2 + fs < 0.95f * (best.force_ms + best.smooth_ms)) {
+        // the other schedule has to win by 5 % against the untuned one: each of
+        // the four spans is timed behind another kernel and taken off it
+        // (72x184x96: estimated ahead, 95 us per iteration against 89)
+        if (rc == CGDIR_OK && f2 + fs < (dflt ? 1.f / 0.95f : 0.95f) * (best.force_ms + best.smooth_ms)) {
             best.fused = 1;
             best.fused_smooth_ms = fs;
             best.fused_force_ms = f2;

@@ -58,3 +58,14 @@ def test_a_table_fixes_the_histories():
             got = register(c, data)
         assert torch.equal(got[0], want[0])
         assert got[1][0]["rms_id"] == want[1][0]["rms_id"]
+
+
+@pytest.mark.parametrize("shape", [(12, 48, 48), (24, 64, 64), (30, 60, 100), (24, 62, 54), (34, 71, 95), (40, 96, 160)])
+@pytest.mark.parametrize("k", [0, 2])
+def test_no_choice_is_slower_than_the_untuned_one(shape, k):
+    """By the tuner's own times, with and without structure terms, on levels
+    whose untuned schedule is the fused one, the split kernels or narrow force
+    threads."""
+    with cg.Context(0) as c:
+        for t in c.autotune(shape, k, 1):
+            assert t["smooth_ms"] + t["force_ms"] <= (t["default_smooth_ms"] + t["default_force_ms"]) * 1.0001 + 1e-6
