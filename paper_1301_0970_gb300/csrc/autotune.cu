@@ -76,9 +76,10 @@ static const TunedLevel *find_tuned(const cgdir_ctx *ctx, int nx, int ny, int nz
     return it == ctx->tuned.end() ? nullptr : &it->second;
 }
 
-// sigma: the larger Gaussian width of the level.
+// sigma: the larger Gaussian width of the level; tma: its fields can be loaded
+// by TMA.
 SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt, bool allow_fused,
-                           float sigma) {
+                           float sigma, bool tma) {
     SmoothChoice ch;
     // registrations that share the GPU (batched, served) cap the z-march's
     // CTAs per SM: uncapped they fill an SM's registers and starve the other
@@ -92,11 +93,11 @@ SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int con
     if (const TunedLevel *t = find_tuned(ctx, nx, ny, nz, contour, sdt)) {
         ch.variant = t->fused && allow_fused ? SMOOTH_FUSED : t->smooth_variant;
         ch.zchunk = t->fused && allow_fused ? 0 : t->smooth_zchunk;
-    } else if (allow_fused && nx % 4 == 0 && gauss_radius(sigma) <= 3 && (size_t)nx * ny * nz <= 350000) {
+    } else if (allow_fused && tma && gauss_radius(sigma) <= 3 && (size_t)nx * ny * nz <= 350000) {
         // untuned small levels: three kernels per iteration instead of five
         // (per iteration: 32x32x16 19.8 against 23.9 us, 64x64x32 23.8 against
         // 27.6, 120x80x35 33.6 against 35.3; 96x96x48 is past the line, 37.5
-        // against 35.7; without TMA, nx % 4 != 0, 58.8 against 48.3)
+        // against 35.7; without TMA 58.8 against 48.3)
         ch.variant = SMOOTH_FUSED;
     }
     return ch;
@@ -328,7 +329,7 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
         // larger volumes (per iteration 91x108x60 62 us, tile 77, fused 105)
         if (nx % 4 == 0 || N <= 500000) add(SMOOTH_TILE, 0);
         add(SMOOTH_SPLIT, 0);
-        const int dflt = smooth_auto_variant(nx, ny, nz, true);
+        const int dflt = smooth_auto_variant(du, nx, ny, nz, true);
         for (int ci = 0; ci < nc && rc == CGDIR_OK; ++ci) {
             float ms = 0.f;
             const bool untuned = cand[ci].variant == dflt && (dflt != SMOOTH_MARCH || cand[ci].zchunk == d);
@@ -381,7 +382,7 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 return launch_fused_smooth_warp(out, sigma, u, a2, kerr(ctx), st);
             });
         fs = std::max(fs - f2, 0.f);
-        const bool dflt = smooth_choice(ctx, nx, ny, nz, contour, -1, true, sigma).variant == SMOOTH_FUSED;
+        const bool dflt = smooth_choice(ctx, nx, ny, nz, contour, -1, true, sigma, nx % 4 == 0).variant == SMOOTH_FUSED;
         if (rc == CGDIR_OK && dflt) {                      // the untuned choice is the fused schedule
             best.default_smooth_ms = fs;
             best.default_force_ms = f2;

@@ -216,7 +216,7 @@ struct SmoothChoice {
 };
 int smooth_default_zchunk(int nx, int ny, int nz, int ncomp, float sigma);
 // scratch: the launch has a field of its own to hold a pass between kernels.
-int smooth_auto_variant(int nx, int ny, int nz, bool scratch);
+int smooth_auto_variant(const float *in, int nx, int ny, int nz, bool scratch);
 // err: device word set to 1 if a bounded wait inside the kernel ran out;
 // nullptr selects the plain-load kernel (no waits).
 cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int ny, int nz,

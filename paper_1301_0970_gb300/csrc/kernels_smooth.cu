@@ -1164,9 +1164,9 @@ static bool grid_holds(int variant, int nz, int ncomp) {
     return slab == 0 || ((long)nz + slab - 1) / slab * ncomp <= 65535;
 }
 
-int smooth_auto_variant(int nx, int ny, int nz, bool scratch) {
+int smooth_auto_variant(const float *in, int nx, int ny, int nz, bool scratch) {
     const size_t N = (size_t)nx * ny * nz;
-    if (nx % 4 == 0) return SMOOTH_MARCH;
+    if (nx % 4 == 0 && ((uintptr_t)in & 15) == 0) return SMOOTH_MARCH;
     if (scratch && N <= kSplitVoxels && grid_holds(SMOOTH_SPLIT, nz, 3)) return SMOOTH_SPLIT;
     return N <= 250000 && grid_holds(SMOOTH_TILE, nz, 3) ? SMOOTH_TILE : SMOOTH_MARCH;
 }
@@ -1270,7 +1270,7 @@ cudaError_t launch_smooth(const float *in, int ncomp, float sigma, int nx, int n
     }
     if (err != nullptr) {
         if (variant == SMOOTH_AUTO && ch.zchunk == 0)
-            variant = smooth_auto_variant(nx, ny, nz, scratch != nullptr && scratch != in && scratch != out);
+            variant = smooth_auto_variant(in, nx, ny, nz, scratch != nullptr && scratch != in && scratch != out);
         if (variant == SMOOTH_FUSED) variant = SMOOTH_TILE;     // nothing to fuse with here
         if (!grid_holds(variant, nz, ncomp)) variant = SMOOTH_MARCH;
         if (variant == SMOOTH_TILE) return smooth_tile(in, ncomp, t, nx, ny, nz, out, stop_flag, s);
@@ -1287,7 +1287,7 @@ cudaError_t launch_smooth_compose(const float *du, const float *u, int mode, flo
                                   int *err, bool one_pass, SmoothChoice ch) {
     const Taps t = gauss_taps(sigma);
     if (!one_pass && t.r > 0 && err != nullptr) {
-        if (ch.variant == SMOOTH_AUTO && ch.zchunk == 0) ch.variant = smooth_auto_variant(nx, ny, nz, tmp != nullptr);
+        if (ch.variant == SMOOTH_AUTO && ch.zchunk == 0) ch.variant = smooth_auto_variant(du, nx, ny, nz, tmp != nullptr);
         if (ch.variant == SMOOTH_SPLIT && grid_holds(SMOOTH_SPLIT, nz, 3))   // x/y pass, then the z pass with the
                                                                               // composite update fused
             return smooth_split(du, u, mode, true, 3, t, nx, ny, nz, out, tmp, ch.zchunk, stop_flag, s);

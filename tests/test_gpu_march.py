@@ -265,3 +265,21 @@ def test_other_kernel_families_keep_the_default_chunk(shape, kernels, monkeypatc
             got.append((dvf, st[0]["rms_id"], stats))
     assert torch.equal(got[0][0], got[1][0])
     assert got[0][1:] == got[1][1:]
+
+
+def test_unaligned_coarse_level_takes_the_split_kernels():
+    """A coarse level with nx % 4 == 0 whose fields are not 16-byte aligned (the
+    finest level has an odd number of voxels) cannot load them by TMA: six
+    kernels an iteration (two force passes, two smoothings in two) and not the
+    fused tiles' three."""
+    shape = (67, 71, 127)
+    img = torch.randn(shape, device=DEV)
+    with cg.Context(0) as c:
+        count = []
+        for n in (10, 30):
+            kw = dict(levels=2, iters=[n, 1], lam=[], sign=[], stop_mode=cg.CGDIR_STOP_FIXED)
+            c.register(img, img, [], [], **kw)
+            before = cg.launch_count()
+            c.register(img, img, [], [], **kw)
+            count.append(cg.launch_count() - before)
+    assert count[1] - count[0] == 20 * 6
