@@ -76,10 +76,10 @@ static const TunedLevel *find_tuned(const cgdir_ctx *ctx, int nx, int ny, int nz
     return it == ctx->tuned.end() ? nullptr : &it->second;
 }
 
-// sigma: the larger Gaussian width of the level; tma: its fields can be loaded
-// by TMA.
+// sigma_fluid, sigma_diff: the Gaussian widths of the level; tma: its fields can
+// be loaded by TMA.
 SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt, bool allow_fused,
-                           float sigma, bool tma) {
+                           float sigma_fluid, float sigma_diff, bool tma) {
     SmoothChoice ch;
     // registrations that share the GPU (batched, served) cap the z-march's
     // CTAs per SM: uncapped they fill an SM's registers and starve the other
@@ -93,11 +93,14 @@ SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int con
     if (const TunedLevel *t = find_tuned(ctx, nx, ny, nz, contour, sdt)) {
         ch.variant = t->fused && allow_fused ? SMOOTH_FUSED : t->smooth_variant;
         ch.zchunk = t->fused && allow_fused ? 0 : t->smooth_zchunk;
-    } else if (allow_fused && tma && gauss_radius(sigma) <= 3 && (size_t)nx * ny * nz <= 350000) {
+    } else if (allow_fused && tma && !ctx->fused_force && gauss_radius(sigma_fluid) > 0 &&
+               gauss_radius(std::max(sigma_fluid, sigma_diff)) <= 3 && (size_t)nx * ny * nz <= 350000) {
         // untuned small levels: three kernels per iteration instead of five
         // (per iteration: 32x32x16 19.8 against 23.9 us, 64x64x32 23.8 against
         // 27.6, 120x80x35 33.6 against 35.3; 96x96x48 is past the line, 37.5
-        // against 35.7; without TMA 58.8 against 48.3)
+        // against 35.7; without TMA 58.8 against 48.3).  With sigma_diff 0 steps
+        // 2 and 3 still share a tile kernel (64x64x32 19.6 against 21.8 us); with
+        // sigma_fluid 0 only a smoothing is left (24.0 against 21.2)
         ch.variant = SMOOTH_FUSED;
     }
     return ch;
@@ -382,7 +385,7 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 return launch_fused_smooth_warp(out, sigma, u, a2, kerr(ctx), st);
             });
         fs = std::max(fs - f2, 0.f);
-        const bool dflt = smooth_choice(ctx, nx, ny, nz, contour, -1, true, sigma, nx % 4 == 0).variant == SMOOTH_FUSED;
+        const bool dflt = smooth_choice(ctx, nx, ny, nz, contour, -1, true, sigma, sigma, nx % 4 == 0).variant == SMOOTH_FUSED;
         if (rc == CGDIR_OK && dflt) {                      // the untuned choice is the fused schedule
             best.default_smooth_ms = fs;
             best.default_force_ms = f2;

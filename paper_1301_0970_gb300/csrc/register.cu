@@ -346,7 +346,7 @@ int plan_enqueue(cgdir_ctx *ctx, const RegPlan &pl, cudaStream_t s, ProfList *pr
         const int zc = force_schedule(ctx, a, sdt);
         // the fields follow one another every 3 Nf floats
         const SmoothChoice sch = smooth_choice(ctx, lx, ly, lz, a.contour, sdt, !pl.shared_gpu,
-                                               std::max(P->sigma_fluid, P->sigma_diff), lx % 4 == 0 && pl.Nf % 4 == 0);
+                                               P->sigma_fluid, P->sigma_diff, lx % 4 == 0 && pl.Nf % 4 == 0);
         const int cap = P->iters[l];
         a.fin.done = done + l;
         a.fin.st = st;

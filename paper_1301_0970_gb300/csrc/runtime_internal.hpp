@@ -210,7 +210,7 @@ void launches_sub(unsigned long long n);
 // allow_fused: false for registrations that share the GPU (batches, served
 // requests), which take the best per-step schedule.
 SmoothChoice smooth_choice(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt, bool allow_fused,
-                           float sigma, bool tma);
+                           float sigma_fluid, float sigma_diff, bool tma);
 int force_zchunk_for(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt);
 int force_schedule(const cgdir_ctx *ctx, ForceArgs &a, int sdt);
 bool use_level_coop(const cgdir_ctx *ctx, int nx, int ny, int nz, int contour, int sdt);

@@ -69,3 +69,24 @@ def test_no_choice_is_slower_than_the_untuned_one(shape, k):
     with cg.Context(0) as c:
         for t in c.autotune(shape, k, 1):
             assert t["smooth_ms"] + t["force_ms"] <= (t["default_smooth_ms"] + t["default_force_ms"]) * 1.0001 + 1e-6
+
+
+@pytest.mark.parametrize("fluid, diff, kernels", [(1.0, 1.0, 3), (1.0, 0.0, 4), (0.0, 1.0, 5), (0.0, 0.0, 5)])
+def test_small_levels_without_one_smoothing(fluid, diff, kernels, monkeypatch):
+    """Kernels per iteration of a small level: the fused schedule's three; two
+    force passes, smoothing with update in one tile kernel and a copy; two
+    passes, a copy, the update and a smoothing or copy.  Same field as with the
+    z-march."""
+    data = pair((16, 32, 48))
+    kw = dict(sigma_fluid=fluid, sigma_diff=diff)
+    with cg.Context(0) as c:
+        count = []
+        for n in (4, 24):
+            register(c, data, iters=[n], **kw)
+            before = cg.launch_count()
+            got = register(c, data, iters=[n], **kw)
+            count.append(cg.launch_count() - before)
+    assert count[1] - count[0] == 20 * kernels
+    monkeypatch.setenv("CGDIR_SMOOTH", "march")
+    with cg.Context(0) as c:
+        assert torch.equal(register(c, data, iters=[24], **kw)[0], got[0])
