@@ -472,13 +472,15 @@ __global__ void k_fill_u8(uint8_t *p, size_t n, uint8_t v) {
 // plane; k_sign_sums marches along z with five planes of that in registers and
 // reads T0 only where some structure or shell is.  A thread owns V x-adjacent
 // voxels (V = 4, one 32-bit word of mask bytes, where nx % 4 == 0).  A thread
-// sums in pairs of floats (high part and rounding errors, exact to 2^-47 of the
-// sum for its 64 voxels at most), because FP64 adds take a warp 14 cycles of
-// the SM here; across threads the sums are FP64.  A structure that no thread of
-// a warp met costs it no reduction.
-// 256x256x96, 5 structures, all three kernels: 39 us; with FP64 sums per thread
-// 87 us; with three dilation launches and, per structure, an FP64 pass over T0
-// and a serial sum of its partials 742 us.
+// sums its 64 voxels at most in triples of floats (exact to 2^-64 of the sum, so
+// no less than an FP64 sum), because FP64 adds take a warp 14 cycles of the SM
+// here; across threads the sums are FP64, and a sum that overflows a float is
+// taken again in FP64.  A structure costs the voxels and warps that it does not
+// reach one test.
+// 256x256x96, 5 structures, all three kernels and the read-back: 56 us, as with
+// pairs of floats (48 bits); a third register per sum 69; FP64 sums per thread
+// about 100; three dilation launches and, per structure, an FP64 pass over T0 and
+// a serial sum of its partials 670.
 constexpr int SB = 256, SZ = 16;                  // threads (32 x 8), most planes per CTA
 // A 1-D grid of 32 V x 8 tiles, x fastest, then y, then z: no limit on ny or nz.
 struct SignTile {
@@ -491,15 +493,23 @@ struct SignTile {
         y = by * 8 + threadIdx.y;
     }
 };
-// A sum of floats as high part and the rounding errors' sum (Knuth's two-sum).
-struct PairSum {
+// A sum of floats as high part, the rounding errors' sum (both exact by Knuth's
+// two-sum) and, in *low, that sum's own rounding errors.  *low lies in shared
+// memory: values that vary as CT numbers do hardly ever reach it, and a third
+// register per sum would take the kernel from three to two CTAs per SM.
+struct TripleSum {
     float s = 0.f, e = 0.f;
-    __device__ __forceinline__ void add(float v) {
-        const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
-        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+    static __device__ __forceinline__ float two_sum(float &s, float v) {      // s += v; the rounding error
+        const float t = __fadd_rn(s, v), b = __fsub_rn(t, s), a = __fsub_rn(s, __fsub_rn(t, b));
         s = t;
+        return __fadd_rn(a, __fsub_rn(v, b));
     }
-    __device__ __forceinline__ double value() const { return isfinite(s) ? (double)s + (double)e : (double)s; }
+    __device__ __forceinline__ void add(float v, float *low) {
+        v = two_sum(s, v);
+        v = two_sum(e, v);
+        if (v != 0.f) *low += v;
+    }
+    __device__ __forceinline__ double value(const float *low) const { return (double)s + ((double)e + (double)*low); }
 };
 template <int V>
 __global__ void __launch_bounds__(SB) k_dilate_xy(const uint8_t *__restrict__ bits, int nx, int ny,
@@ -551,22 +561,25 @@ __global__ void __launch_bounds__(SB) k_sign_sums(const IT *__restrict__ T0, con
     const int x = st.x, y = st.y, zb = st.bz * zc, ze = min(zb + zc, nz);
     const int tid = threadIdx.y * 32 + threadIdx.x, bid = blockIdx.x;
     const unsigned kmask = (1u << k) - 1u;
-    PairSum sin_[kMaxMasks], ssh[kMaxMasks];
+    TripleSum sin_[kMaxMasks], ssh[kMaxMasks];
+    __shared__ float low[2][kMaxMasks][SB];       // each thread's own
+#pragma unroll
+    for (int j = 0; j < kMaxMasks; ++j) low[0][j][tid] = low[1][j][tid] = 0.f;
     int cnt[kMaxMasks] = {};                      // inside (low 16 bits) and shell: at most 4 SZ each
     unsigned seen = 0;
+    const size_t nxy = (size_t)nx * ny, col = (size_t)y * nx + x;
+    auto word = [&](const uint8_t *b, int z) -> uint32_t {           // 0 outside the volume
+        if (z < 0 || z >= nz) return 0u;
+        const uint8_t *p = b + (size_t)z * nxy + col;
+        return V == 4 ? __ldg(reinterpret_cast<const uint32_t *>(p)) : (uint32_t)__ldg(p);
+    };
     if (x < nx && y < ny) {
-        const size_t nxy = (size_t)nx * ny, col = (size_t)y * nx + x;
-        auto word = [&](const uint8_t *b, int z) -> uint32_t {       // 0 outside the volume
-            if (z < 0 || z >= nz) return 0u;
-            const uint8_t *p = b + (size_t)z * nxy + col;
-            return V == 4 ? __ldg(reinterpret_cast<const uint32_t *>(p)) : (uint32_t)__ldg(p);
-        };
         // planes z - 2 .. z + 2 of the dilated bytes, z + 3 and the next plane's own bytes in flight
         uint32_t d0 = 0, d1 = word(dxy, zb - 2), d2 = word(dxy, zb - 1), d3 = word(dxy, zb), d4 = word(dxy, zb + 1),
                  nd = word(dxy, zb + 2), nc = word(sbits, zb);
         for (int z = zb; z < ze; ++z) {
             d0 = d1; d1 = d2; d2 = d3; d3 = d4; d4 = nd;
-            const uint32_t cen = nc, all = d0 | d1 | d2 | d3 | d4;
+            const uint32_t cen = nc, all = (d0 | d1 | d2 | d3 | d4) & (kmask * 0x01010101u);
             nd = word(dxy, z + 3);
             nc = word(sbits, z + 1);
             if (all == 0u) continue;              // no structure within distance 2 of these voxels
@@ -575,18 +588,37 @@ __global__ void __launch_bounds__(SB) k_sign_sums(const IT *__restrict__ T0, con
 #pragma unroll
             for (int v = 0; v < V; ++v) tv[v] = ld_img<IT>(T0 + i + v);
 #pragma unroll
-            for (int v = 0; v < V; ++v) {
-                const unsigned in = (cen >> (8 * v)) & kmask, sh = (all >> (8 * v)) & kmask & ~in;
-                if ((in | sh) == 0u) continue;
-                seen |= in | sh;
+            for (int j = 0; j < kMaxMasks; ++j) {
+                if ((all & (0x01010101u << j)) == 0u) continue;
+                seen |= 1u << j;
 #pragma unroll
-                for (int j = 0; j < kMaxMasks; ++j) {
-                    if ((in >> j) & 1u) { sin_[j].add(tv[v]); cnt[j] += 1; }
-                    if ((sh >> j) & 1u) { ssh[j].add(tv[v]); cnt[j] += 1 << 16; }
+                for (int v = 0; v < V; ++v) {
+                    if (!((all >> (8 * v + j)) & 1u)) continue;
+                    if ((cen >> (8 * v + j)) & 1u) {
+                        sin_[j].add(tv[v], &low[0][j][tid]);
+                        cnt[j] += 1;
+                    } else {
+                        ssh[j].add(tv[v], &low[1][j][tid]);
+                        cnt[j] += 1 << 16;
+                    }
                 }
             }
         }
     }
+    // one of this thread's sums in FP64, read again
+    auto again = [&](int j, bool shell) {
+        double a = 0.0;
+        for (int z = zb; z < ze; ++z) {
+            uint32_t m = word(sbits, z);
+            if (shell) m = (word(dxy, z - 2) | word(dxy, z - 1) | word(dxy, z) | word(dxy, z + 1) | word(dxy, z + 2)) & ~m;
+            for (int v = 0; v < V; ++v)
+                if ((m >> (8 * v + j)) & 1u) a += (double)ld_img<IT>(T0 + (size_t)z * nxy + col + v);
+        }
+        return a;
+    };
+    auto total = [&](const TripleSum &t, int j, bool shell) {
+        return isfinite(t.s + t.e) ? t.value(&low[shell][j][tid]) : again(j, shell);
+    };
     // block sums in a fixed order: lanes by shuffles, then the 8 warps in turn
     __shared__ double ws[kMaxMasks][2][8];
     __shared__ int wc[kMaxMasks][2][8];
@@ -597,7 +629,7 @@ __global__ void __launch_bounds__(SB) k_sign_sums(const IT *__restrict__ T0, con
         double a = 0.0, c = 0.0;
         int ca = 0, cc = 0;
         if ((wseen >> j) & 1u) {                  // the same for the whole warp
-            a = sin_[j].value(); c = ssh[j].value();
+            a = total(sin_[j], j, false); c = total(ssh[j], j, true);
             ca = __reduce_add_sync(0xffffffffu, cnt[j] & 0xffff);
             cc = __reduce_add_sync(0xffffffffu, cnt[j] >> 16);
 #pragma unroll

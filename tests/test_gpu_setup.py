@@ -117,3 +117,33 @@ def test_prolong_tiles(ctx, fine):
     torch.cuda.synchronize()
     ref = oracle.prolong(uc, fine)
     assert np.abs(got.cpu().numpy() - ref).max() <= 1e-6 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("shape", [(17, 12, 64), (20, 10, 33)])
+def test_auto_sign_of_sums_beyond_float(ctx, shape):
+    """Values whose sum over a few voxels overflows a float have a mean all the
+    same; an infinite or NaN voxel decides as it does in FP64."""
+    m = np.zeros((1,) + shape, np.uint8)
+    m[0, 4:14, 3:9, 8:24] = 1
+    for inside, shell in ((2.0e38, 1.0e38), (1.0e38, 2.0e38), (-2.0e38, -1.0e38), (3.0e38, 3.4028235e38)):
+        for odd in (None, np.inf, -np.inf, np.nan):
+            T = np.where(m[0] != 0, inside, shell).astype(np.float32)
+            if odd is not None:
+                T[6, 5, 12] = odd
+            with np.errstate(invalid="ignore"):
+                want = oracle.auto_sign(T.astype(np.float64), m)
+            assert ctx.auto_sign(torch.from_numpy(T).to(DEV), packed(m), 1) == want
+
+
+@pytest.mark.parametrize("shape", [(16, 12, 64), (16, 12, 33)])
+def test_auto_sign_keeps_what_fp64_keeps(ctx, shape):
+    """A column of 2^48, 2^24, 1, -2^48, -2^24, 0, 0, 0 has mean 1/8 in FP64 and
+    0 in a sum of 48 bits; its shell's value lies between."""
+    m = np.zeros((1,) + shape, np.uint8)
+    m[0, 4:12, 6, 17] = 1
+    T = np.full(shape, 0.0625, np.float32)
+    T[4:12, 6, 17] = [2.0 ** 48, 2.0 ** 24, 1, -2.0 ** 48, -2.0 ** 24, 0, 0, 0]
+    want = oracle.auto_sign(T.astype(np.float64), m)
+    assert ctx.auto_sign(torch.from_numpy(T).to(DEV), packed(m), 1) == want
+    T[6, 6, 17] = 0
+    assert ctx.auto_sign(torch.from_numpy(T).to(DEV), packed(m), 1) == [-s for s in want]
