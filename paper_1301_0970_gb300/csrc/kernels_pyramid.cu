@@ -232,16 +232,20 @@ __global__ void k_restrict_bits_rows(const uint8_t *__restrict__ in, int nx, int
 // a time from the 3 x 3 x 3 coarse values around (X, Y, Z): 27 shared reads
 // for 8 outputs.  Along an axis the even voxel's corners are the first two of
 // those three values and the odd one's the last two, with k_prolong's weights
-// and order of multiply-adds (same bits); at the low border, where the clamped
-// coordinate is 0, the weights are 1 and 0 on values that are both u_c(0).
+// and terms (same bits); at the low border, where the clamped coordinate is 0 and
+// the corners are voxels 0 and 1 with weights 1 and 0, voxel 1 stands in the place
+// before voxel 0 and the weights change places.
 constexpr int PX = 64, PY = 8, PZ = 8;
 constexpr int PCX = PX / 2 + 2, PCY = PY / 2 + 2, PCZ = PZ / 2 + 2;
 // Weights (low, high corner) of fine index x on a coarse axis of c voxels.
 __device__ __forceinline__ void prolong_axis(int x, int c, float *w) {
     const float p = fminf(fmaxf((x + 0.5f) * 0.5f - 0.5f, 0.f), (float)(c - 1));
-    w[1] = p - floorf(p);
+    const float f = p - floorf(p);
+    w[1] = x > 0 ? f : 1.f;
     w[0] = 1.f - w[1];
 }
+// The coarse index staged at place i of an axis of c voxels.
+__device__ __forceinline__ int prolong_src(int i, int c) { return i < 0 ? min(1, c - 1) : min(i, c - 1); }
 __global__ void __launch_bounds__(128) k_prolong_tile(const float *__restrict__ uc, int cx, int cy, int cz, int nx,
                                                       int ny, int nz, float *__restrict__ uf) {
     __shared__ float t[3][PCZ][PCY][PCX];
@@ -250,13 +254,13 @@ __global__ void __launch_bounds__(128) k_prolong_tile(const float *__restrict__ 
     const size_t Nc = (size_t)cx * cy * cz, N = (size_t)nx * ny * nz;
     // a warp per coarse row, nine rows' loads in flight
     static_assert(3 * PCZ * PCY % 36 == 0, "4 warps x 9 rows per turn");
-    const int ca = clampi(bx + (int)threadIdx.x, 0, cx - 1), cb = clampi(bx + 32 + (int)threadIdx.x, 0, cx - 1);
+    const int ca = prolong_src(bx + (int)threadIdx.x, cx), cb = prolong_src(bx + 32 + (int)threadIdx.x, cx);
     for (int r0 = threadIdx.y; r0 < 3 * PCZ * PCY; r0 += 36) {
         float v[9], e[9];
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
             const int row = r0 + 4 * q, j = row % PCY, k = (row / PCY) % PCZ, comp = row / (PCY * PCZ);
-            const float *src = uc + comp * Nc + ((size_t)clampi(bz + k, 0, cz - 1) * cy + clampi(by + j, 0, cy - 1)) * cx;
+            const float *src = uc + comp * Nc + ((size_t)prolong_src(bz + k, cz) * cy + prolong_src(by + j, cy)) * cx;
             v[q] = __ldg(src + ca);
             e[q] = threadIdx.x < PCX - 32 ? __ldg(src + cb) : 0.f;
         }

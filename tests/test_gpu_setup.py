@@ -147,3 +147,20 @@ def test_auto_sign_keeps_what_fp64_keeps(ctx, shape):
     assert ctx.auto_sign(torch.from_numpy(T).to(DEV), packed(m), 1) == want
     T[6, 6, 17] = 0
     assert ctx.auto_sign(torch.from_numpy(T).to(DEV), packed(m), 1) == [-s for s in want]
+
+
+@pytest.mark.parametrize("fine", [(2, 3, 5), (8, 8, 64), (9, 17, 66), (1, 2, 130)])
+def test_prolong_of_values_that_are_not_finite(ctx, fine):
+    """Every corner enters with its weight, also with weight 0 at the borders: an
+    infinite or NaN coarse value spoils the fine voxels that the oracle's does."""
+    coarse = tuple((n + 1) // 2 for n in fine)
+    at = {(min(a, coarse[0] - 1), min(b, coarse[1] - 1), min(c, coarse[2] - 1))
+          for a in (0, 1, 99) for b in (0, 1, 99) for c in (0, 1, 99)}
+    for place in sorted(at):
+        for value in (np.inf, -np.inf, np.nan):
+            uc = np.ones((3,) + coarse, np.float32)
+            uc[(slice(None),) + place] = value
+            got = ctx.prolong(torch.from_numpy(uc).to(DEV), fine).cpu().numpy()
+            with np.errstate(invalid="ignore"):
+                ref = oracle.prolong(uc, fine)
+            assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref)), place
