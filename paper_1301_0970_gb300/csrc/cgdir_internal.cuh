@@ -270,7 +270,7 @@ cudaError_t launch_prolong(const float *uc, int cx, int cy, int cz, int nx, int 
                            float *uf, cudaStream_t s);
 cudaError_t launch_uroi(const uint8_t *sbits, int k, int nx, int ny, int nz, const double *spacing,
                         double margin, uint8_t *scratch, uint8_t *out, cudaStream_t s);
-size_t uroi_scratch_bytes(int nx, int ny, int nz);
+size_t uroi_scratch_bytes(int nx, int ny, int nz, double spacing_z, double margin);
 cudaError_t launch_sign_sums(const void *T0, int dtype, const uint8_t *sbits, int k, int nx, int ny, int nz,
                              uint8_t *dxy, double *partial, double *sums /* [k][4] */, cudaStream_t s);
 size_t sign_partial_rows(int nx, int ny, int nz);

@@ -463,6 +463,29 @@ __global__ void k_uroi_out(const uint32_t *__restrict__ zrows, int rz, int nx, i
     }
 }
 
+// Rows of one word (nx <= 32) without the |dz| words: the OR over dz and dy of
+// rows dilated in place.  For volumes so narrow that the words, one per row
+// however short, would outgrow byte maps (nx <= 13 at the most).
+__global__ void k_uroi_narrow(const uint32_t *__restrict__ bits, const __grid_constant__ UroiTable t, int nx, int ny,
+                              int nz, uint8_t *__restrict__ out) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (long long)ny * nz) return;
+    const int z = (int)(i / ny), y = (int)(i - (long long)z * ny);
+    uint32_t b = 0;
+    for (int dz = -t.rz; dz <= t.rz; ++dz) {
+        if (z + dz < 0 || z + dz >= nz) continue;
+        for (int dy = -t.ry; dy <= t.ry; ++dy) {
+            const int e = t.ext[dz < 0 ? -dz : dz][dy < 0 ? -dy : dy];
+            if (e < 0 || y + dy < 0 || y + dy >= ny) continue;
+            const uint32_t w = __ldg(bits + i + (long long)dz * ny + dy);
+            if (w == 0u) continue;
+            for (int q = 0; q <= e; ++q) b |= (w << q) | (w >> q);
+        }
+    }
+    uint8_t *dst = out + (size_t)i * nx;
+    for (int e = 0; e < nx; ++e) dst[e] = (uint8_t)((b >> e) & 1u);
+}
+
 __global__ void k_fill_u8(uint8_t *p, size_t n, uint8_t v) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (size_t)gridDim.x * blockDim.x)
@@ -806,6 +829,13 @@ cudaError_t launch_prolong(const float *uc, int cx, int cy, int cz, int nx, int 
     return cudaGetLastError();
 }
 
+static int uroi_radius(double margin, double spacing) { return (int)(margin / spacing); }
+// Whether the words of rows and |dz| take more than byte maps did (5 per voxel).
+static bool uroi_narrow(int nx, int ny, int nz, int rz) {
+    const size_t words = (size_t)ny * nz * ((nx + 31) / 32);
+    return nx <= 32 && 4 * words * (rz + 2) > 5 * (size_t)nx * ny * nz;
+}
+
 // scratch: uroi_scratch_bytes.
 cudaError_t launch_uroi(const uint8_t *sbits, int k, int nx, int ny, int nz, const double *spacing,
                         double margin, uint8_t *scratch, uint8_t *out, cudaStream_t s) {
@@ -817,9 +847,9 @@ cudaError_t launch_uroi(const uint8_t *sbits, int k, int nx, int ny, int nz, con
     if (!(margin >= 0.0) || !(spacing[0] > 0) || !(spacing[1] > 0) || !(spacing[2] > 0))
         return cudaErrorInvalidValue;
     UroiTable t{};
-    t.rx = (int)(margin / spacing[0]);
-    t.ry = (int)(margin / spacing[1]);
-    t.rz = (int)(margin / spacing[2]);
+    t.rx = uroi_radius(margin, spacing[0]);
+    t.ry = uroi_radius(margin, spacing[1]);
+    t.rz = uroi_radius(margin, spacing[2]);
     if (t.rx > kMaxUroiRadius || t.ry > kMaxUroiRadius || t.rz > kMaxUroiRadius)
         return cudaErrorInvalidValue;
     for (int dz = 0; dz <= t.rz; ++dz)
@@ -839,6 +869,10 @@ cudaError_t launch_uroi(const uint8_t *sbits, int k, int nx, int ny, int nz, con
     const unsigned g = (unsigned)((words + 127) / 128);
     auto aligned = [&](const void *q) { return nx % 16 == 0 && (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
     k_uroi_bits<<<g, 128, 0, s>>>(sbits, mask, nx, words, wpr, aligned(sbits), bits); note_launch();
+    if (uroi_narrow(nx, ny, nz, t.rz)) {
+        k_uroi_narrow<<<g, 128, 0, s>>>(bits, t, nx, ny, nz, out); note_launch();
+        return cudaGetLastError();
+    }
     if (t.rz < 5) k_uroi_rows<5><<<g, 128, 0, s>>>(bits, t, ny, words, wpr, zrows);
     else k_uroi_rows<kMaxUroiRadius + 1><<<g, 128, 0, s>>>(bits, t, ny, words, wpr, zrows);
     note_launch();
@@ -846,9 +880,12 @@ cudaError_t launch_uroi(const uint8_t *sbits, int k, int nx, int ny, int nz, con
     return cudaGetLastError();
 }
 
-// Bit rows, then up to kMaxUroiRadius + 1 words per bit-row word.
-size_t uroi_scratch_bytes(int nx, int ny, int nz) {
-    return (size_t)ny * nz * ((nx + 31) / 32) * 4 * (kMaxUroiRadius + 2);
+// Bit rows, then rz + 1 words per bit-row word.  (A margin or spacing that
+// launch_uroi refuses needs none.)
+size_t uroi_scratch_bytes(int nx, int ny, int nz, double spacing_z, double margin) {
+    if (!(margin >= 0.0) || !(spacing_z > 0) || margin / spacing_z >= kMaxUroiRadius + 1) return 0;
+    const int rz = uroi_radius(margin, spacing_z);
+    return (size_t)ny * nz * ((nx + 31) / 32) * 4 * (uroi_narrow(nx, ny, nz, rz) ? 1 : rz + 2);
 }
 
 static size_t sign_ctas(int nx, int ny, int nz, int v, int zc) {

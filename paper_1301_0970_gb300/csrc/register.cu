@@ -188,7 +188,11 @@ int plan_make(cgdir_ctx *ctx, const cgdir_volume *S, const cgdir_volume *M, cons
     pl.need[RegPlan::B_FIELDS] = 4 * 3 * Nf * sizeof(float);
     pl.need[RegPlan::B_PARTIAL] = std::max<size_t>(np * kPartialStride * sizeof(double), 256);
     pl.need[RegPlan::B_STATE] = pl.state_bytes;
-    pl.need[RegPlan::B_ROWDIST] = std::max<size_t>(uroi_scratch_bytes(nx, ny, nz), 256);
+    pl.need[RegPlan::B_ROWDIST] = 256;
+    for (int l = 0; l < L; ++l)
+        pl.need[RegPlan::B_ROWDIST] = std::max(
+            pl.need[RegPlan::B_ROWDIST], uroi_scratch_bytes(pl.dims[l][0], pl.dims[l][1], pl.dims[l][2],
+                                                            P->spacing_mm[2] * (1 << (L - 1 - l)), P->margin_mm));
     const bool need_stage = (S->where == CGDIR_HOST && S->dtype != pl.sdt) ||
                             (M->where == CGDIR_HOST && M->dtype != pl.sdt) ||
                             (k > 0 && (SM->where == CGDIR_HOST || MM->where == CGDIR_HOST));

@@ -604,10 +604,9 @@ int cgdir_uroi(cgdir_ctx *ctx, const uint8_t *sbits, int k, int nx, int ny, int 
         return fail(ctx, CGDIR_EINVAL, "uroi: bad arguments");
     DeviceGuard g(ctx->device);
     void *rd = nullptr;
-    TRY(ws_get(ctx, "rowdist", uroi_scratch_bytes(nx, ny, nz), &rd));
-    const double sp1[3] = {1, 1, 1};
-    cudaError_t e = launch_uroi(sbits, k, nx, ny, nz, spacing ? spacing : sp1, margin, (uint8_t *)rd, out,
-                                ctx->stream);
+    const double sp1[3] = {1, 1, 1}, *sp = spacing ? spacing : sp1;
+    TRY(ws_get(ctx, "rowdist", uroi_scratch_bytes(nx, ny, nz, sp[2], margin), &rd));
+    cudaError_t e = launch_uroi(sbits, k, nx, ny, nz, sp, margin, (uint8_t *)rd, out, ctx->stream);
     if (e == cudaErrorInvalidValue)
         return fail(ctx, CGDIR_EINVAL, "uroi: spacing must be > 0, margin >= 0, margin/spacing <= 15");
     CK(e);

@@ -164,3 +164,20 @@ def test_prolong_of_values_that_are_not_finite(ctx, fine):
             with np.errstate(invalid="ignore"):
                 ref = oracle.prolong(uc, fine)
             assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref)), place
+
+
+@pytest.mark.parametrize("nx, spacing, margin", [(1, 2.5, 10.0), (4, 2.5, 10.0), (5, 2.5, 10.0), (8, 1.0, 15.0),
+                                                 (13, 1.0, 15.0), (14, 1.0, 15.0), (33, 1.0, 15.0)])
+def test_uroi_scratch_of_narrow_volumes(nx, spacing, margin):
+    """The UROI of a context whose budget holds 5 bytes of scratch per voxel:
+    word rows where they fit, rows dilated in place where they do not."""
+    shape = (100, 700, nx)                        # 2 MB is the unit of the budget
+    m = np.zeros((1,) + shape, np.uint8)
+    m[0, 40:50, 300:340, nx // 2] = 1
+    m[0, 0, 0, 0] = m[0, -1, -1, -1] = 1
+    unit = 1 << 21
+    budget = -(-(m.size * 5 + 3) // unit) * unit
+    with cg.Context(0, mem_budget_bytes=budget) as c:
+        got = c.uroi(packed(m), 1, (spacing,) * 3, margin)
+        torch.cuda.synchronize()
+    assert np.array_equal(got.cpu().numpy(), oracle.uroi(m, shape, (spacing,) * 3, margin))
