@@ -508,16 +508,20 @@ __global__ void k_fill_u8(uint8_t *p, size_t n, uint8_t v) {
 // pairs of floats (48 bits); a third register per sum 69; FP64 sums per thread
 // about 100; three dilation launches and, per structure, an FP64 pass over T0 and
 // a serial sum of its partials 670.
-constexpr int SB = 256, SZ = 16;                  // threads (32 x 8), most planes per CTA
-// A 1-D grid of 32 V x 8 tiles, x fastest, then y, then z: no limit on ny or nz.
+constexpr int SB = 256, SZ = 16;                  // threads, planes per CTA at most (thin volumes: more)
+// A 1-D grid of SB threads of V voxels over the columns of a plane, then z: no
+// limit on any extent, and no idle threads in narrow or flat volumes.
 struct SignTile {
-    int x, y, bz;
+    size_t col;            // first voxel of the thread's columns in a plane
+    bool in;
+    int bz;
     __device__ SignTile(int nx, int ny, int v) {
-        const int tx = (nx + 32 * v - 1) / (32 * v), ty = (ny + 7) / 8, bid = blockIdx.x;
-        bz = bid / (tx * ty);
-        const int by = (bid - bz * tx * ty) / tx;
-        x = v * ((bid - (bz * ty + by) * tx) * 32 + threadIdx.x);
-        y = by * 8 + threadIdx.y;
+        const size_t cols = (size_t)nx * ny / v;
+        const unsigned tiles = (unsigned)((cols + SB - 1) / SB);
+        bz = (int)(blockIdx.x / tiles);
+        const size_t c = (size_t)(blockIdx.x - bz * tiles) * SB + threadIdx.x;
+        in = c < cols;
+        col = c * v;
     }
 };
 // A sum of floats as high part, the rounding errors' sum (both exact by Knuth's
@@ -542,8 +546,9 @@ template <int V>
 __global__ void __launch_bounds__(SB) k_dilate_xy(const uint8_t *__restrict__ bits, int nx, int ny,
                                                   uint8_t *__restrict__ out) {
     const SignTile t(nx, ny, V);
-    const int x = t.x, y = t.y;
-    if (x >= nx || y >= ny) return;
+    if (!t.in) return;
+    const int y = t.col < (1ull << 31) ? (int)((unsigned)t.col / (unsigned)nx) : (int)(t.col / nx);
+    const int x = (int)(t.col - (size_t)y * nx);
     // rows outside the volume are read at the border, which lies within
     // distance 2 as well: no branch between the loads
     uint32_t w[5][V == 4 ? 3 : 5];
@@ -585,22 +590,22 @@ __global__ void __launch_bounds__(SB) k_sign_sums(const IT *__restrict__ T0, con
                                                   const uint8_t *__restrict__ dxy, int k, int nx, int ny, int nz,
                                                   int zc, double *__restrict__ partial) {
     const SignTile st(nx, ny, V);
-    const int x = st.x, y = st.y, zb = st.bz * zc, ze = min(zb + zc, nz);
-    const int tid = threadIdx.y * 32 + threadIdx.x, bid = blockIdx.x;
+    const int zb = st.bz * zc, ze = min(zb + zc, nz);
+    const int tid = threadIdx.x, bid = blockIdx.x;
     const unsigned kmask = (1u << k) - 1u;
     TripleSum sin_[kMaxMasks], ssh[kMaxMasks];
     __shared__ float low[2][kMaxMasks][SB];       // each thread's own
 #pragma unroll
     for (int j = 0; j < kMaxMasks; ++j) low[0][j][tid] = low[1][j][tid] = 0.f;
-    int cnt[kMaxMasks] = {};                      // inside (low 16 bits) and shell: at most 4 SZ each
+    int cnt[kMaxMasks] = {};                      // inside (low 16 bits) and shell: at most V zc each
     unsigned seen = 0;
-    const size_t nxy = (size_t)nx * ny, col = (size_t)y * nx + x;
+    const size_t nxy = (size_t)nx * ny, col = st.col;
     auto word = [&](const uint8_t *b, int z) -> uint32_t {           // 0 outside the volume
         if (z < 0 || z >= nz) return 0u;
         const uint8_t *p = b + (size_t)z * nxy + col;
         return V == 4 ? __ldg(reinterpret_cast<const uint32_t *>(p)) : (uint32_t)__ldg(p);
     };
-    if (x < nx && y < ny) {
+    if (st.in) {
         // planes z - 2 .. z + 2 of the dilated bytes, z + 3 and the next plane's own bytes in flight
         uint32_t d0 = 0, d1 = word(dxy, zb - 2), d2 = word(dxy, zb - 1), d3 = word(dxy, zb), d4 = word(dxy, zb + 1),
                  nd = word(dxy, zb + 2), nc = word(sbits, zb);
@@ -889,18 +894,22 @@ size_t uroi_scratch_bytes(int nx, int ny, int nz, double spacing_z, double margi
 }
 
 static size_t sign_ctas(int nx, int ny, int nz, int v, int zc) {
-    return (size_t)((nx + 32 * v - 1) / (32 * v)) * ((ny + 7) / 8) * ((nz + zc - 1) / zc);
+    return ((size_t)nx * ny / v + SB - 1) / SB * ((nz + zc - 1) / zc);
 }
 // Planes per CTA: 16 where that gives 8 CTAs per SM (the march is bound by
-// latency), else 8 or 4 (each chunk reads 4 more planes of dilated bytes).
+// latency), else 8 or 4 (each chunk reads 4 more planes of dilated bytes).  In a
+// volume of few columns more, so that the partial sums (a row of 4 per structure
+// and CTA) take no more than a byte per voxel; a thread counts its voxels in 16
+// bits.
 static int sign_zchunk(int nx, int ny, int nz, int v) {
     int zc = SZ;
     while (zc > 4 && sign_ctas(nx, ny, nz, v, zc) < (size_t)8 * sm_count()) zc /= 2;
+    while (zc < 4096 && sign_ctas(nx, ny, nz, v, zc) * kMaxMasks * 32 > (size_t)nx * ny * nz + 16384) zc *= 2;
     return zc;
 }
 size_t sign_partial_rows(int nx, int ny, int nz) {
-    return std::max(sign_ctas(nx, ny, nz, 1, sign_zchunk(nx, ny, nz, 1)),
-                    sign_ctas(nx, ny, nz, 4, sign_zchunk(nx, ny, nz, 4)));
+    const size_t one = sign_ctas(nx, ny, nz, 1, sign_zchunk(nx, ny, nz, 1));
+    return nx % 4 == 0 ? std::max(one, sign_ctas(nx, ny, nz, 4, sign_zchunk(nx, ny, nz, 4))) : one;
 }
 
 template <typename IT>
@@ -910,7 +919,7 @@ static void sign_sums_t(const void *T0, const uint8_t *sbits, int k, int nx, int
     const bool quad = nx % 4 == 0 && (reinterpret_cast<uintptr_t>(sbits) & 3u) == 0;
     const int v = quad ? 4 : 1, zc = sign_zchunk(nx, ny, nz, v);
     const unsigned g = (unsigned)sign_ctas(nx, ny, nz, v, zc);
-    const dim3 block(32, 8);
+    const int block = SB;
     const IT *t0 = static_cast<const IT *>(T0);
     if (quad) {
         k_dilate_xy<4><<<(unsigned)sign_ctas(nx, ny, nz, 4, 1), block, 0, s>>>(sbits, nx, ny, dxy);

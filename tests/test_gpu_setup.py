@@ -181,3 +181,22 @@ def test_uroi_scratch_of_narrow_volumes(nx, spacing, margin):
         got = c.uroi(packed(m), 1, (spacing,) * 3, margin)
         torch.cuda.synchronize()
     assert np.array_equal(got.cpu().numpy(), oracle.uroi(m, shape, (spacing,) * 3, margin))
+
+
+@pytest.mark.parametrize("shape", [(300000, 1, 1), (1, 300000, 1), (1, 1, 300000), (40000, 5, 3), (75000, 1, 4)])
+def test_auto_sign_of_thin_volumes(shape):
+    """Volumes of few columns or few planes: the signs, in scratch of two buffers
+    of a byte per voxel (allocated in units of 2 MB)."""
+    rng = np.random.default_rng(shape[0])
+    m = np.zeros((8,) + shape, np.uint8)
+    for j in range(8):
+        for _ in range(4):
+            at = [int(rng.integers(0, n)) for n in shape]
+            m[j][tuple(slice(a, a + 9) for a in at)] = 1
+    T = rng.normal(0, 5, shape)
+    for j in range(8):
+        T = T + np.where(m[j] != 0, 300.0 * (j + 1) * (1 if j % 2 == 0 else -1), 0.0)
+    T = T.astype(np.float32)
+    want = oracle.auto_sign(T.astype(np.float64), m)
+    with cg.Context(0, mem_budget_bytes=2 << 21) as c:
+        assert c.auto_sign(torch.from_numpy(T).to(DEV), packed(m), 8) == want
