@@ -31,29 +31,15 @@ __global__ void k_wait_timeout(long long limit_cycles, int *err) {
     }
 }
 
-}  // namespace
+constexpr int nz = 20;
+constexpr size_t n = nz * 32 * 32;             // >= 3 x 16 x 16 x 16
 
-extern "C" int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us) {
-    if (!ctx) return CGDIR_EINVAL;
-    ctx->err.clear();
-    if (limit_us < 1 || limit_us > 2000000) return fail(ctx, CGDIR_EINVAL, "selftest: limit_us must be 1..2000000");
-    DeviceGuard g(ctx->device);
-    // at most 2.1 GHz: the wait lasts at least limit_us
-    const long long cycles = (long long)limit_us * 2100;
-    k_wait_timeout<<<1, 32, 0, ctx->stream>>>(cycles, ctx->err_word);
-    note_launch();
-    CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(ctx->stream));
-    const int rc = check_err_word(ctx);
-    if (rc != CGDIR_ETIMEDOUT) return rc;
-    constexpr int nz = 20;
-    constexpr size_t n = nz * 32 * 32;             // >= 3 x 16 x 16 x 16
-    void *f = nullptr;
-    TRY(ws_get(ctx, "selftest", (2 * n + 1) * sizeof(float), &f));
-    float *in = (float *)f, *out = in + n;
+// The kernels that wait for copies, on fields some of which never arrive.
+// f: 2 n floats and an int.
+int lost_copies(cgdir_ctx *ctx, float *f, long long limit) {
+    float *in = f, *out = in + n;
     int *stop = (int *)(out + n);
     CK(cudaMemsetAsync(in, 0, n * sizeof(float), ctx->stream));
-    const long long limit = std::min<long long>(cycles, 2100000);
     // first, middle and last plane of one turn of the plane loop (chunks of
     // one plane march 7 planes) and of a chunk whose last turn is cut short
     const int at[6][2] = {{1, 0}, {1, 3}, {1, 6}, {nz, 0}, {nz, 21}, {nz, 25}};
@@ -73,5 +59,28 @@ extern "C" int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us) {
         if (rs == CGDIR_OK) return fail(ctx, CGDIR_ECUDA, "selftest: the fused tiles lost a wait that ran out");
         if (rs != CGDIR_ETIMEDOUT) return rs;
     }
-    return rc;
+    return CGDIR_ETIMEDOUT;
+}
+
+}  // namespace
+
+extern "C" int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us) {
+    if (!ctx) return CGDIR_EINVAL;
+    ctx->err.clear();
+    if (limit_us < 1 || limit_us > 2000000) return fail(ctx, CGDIR_EINVAL, "selftest: limit_us must be 1..2000000");
+    DeviceGuard g(ctx->device);
+    // at most 2.1 GHz: the wait lasts at least limit_us
+    const long long cycles = (long long)limit_us * 2100;
+    k_wait_timeout<<<1, 32, 0, ctx->stream>>>(cycles, ctx->err_word);
+    note_launch();
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(ctx->stream));
+    const int rc = check_err_word(ctx);
+    if (rc != CGDIR_ETIMEDOUT) return rc;
+    float *f = nullptr;                        // not the context's: its budget stays
+    CK(cudaMalloc(&f, (2 * n + 1) * sizeof(float)));
+    const int rs = lost_copies(ctx, f, std::min<long long>(cycles, 2100000));
+    cudaStreamSynchronize(ctx->stream);
+    cudaFree(f);
+    return rs;
 }
