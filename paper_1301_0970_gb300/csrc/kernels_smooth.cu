@@ -1173,7 +1173,7 @@ int smooth_auto_variant(const float *in, int nx, int ny, int nz, bool scratch) {
 
 int smooth_default_zchunk(int nx, int ny, int nz, int ncomp, float sigma) {
     const int r = std::max(gauss_radius(sigma), 1), wy = r <= 4 ? 32 : 16;
-    const int res = r <= 3 ? 5 : 4;          // MarchGeom::CTAS
+    const int res = nx % 4 == 0 && r <= 3 ? 5 : 4;          // as smooth_march_r has it
     return march_zchunk_r(nz, (long)((nx + MX - 1) / MX) * ((ny + wy - 1) / wy) * ncomp, res, r);
 }
 
