@@ -474,11 +474,12 @@ int cgdir_selftest_wait_timeout(cgdir_ctx *ctx, int limit_us);
  * volume in 1 to 16 z chunks, the 32 x 16 one with 2, 4 and 8, 3-D
  * shared-memory tile, split xy + z kernels with the update in the z pass;
  * fewer where nx % 4 != 0) on ctx's stream, those of small levels as CUDA
- * graphs, and keeps the fastest; the default chunk and width of the force
- * pass stand unless others are ahead by more than 3 %, and the untuned pass
- * wherever it is not behind the choice.  Then it times the fused schedule: of
- * it and the steps apart, the one that an untuned level does not run has to
- * win by 5 %.  Later registrations of those shapes use the choices:
+ * graphs, and keeps the fastest; of force passes within 3 % of each other the
+ * one with the longer chunk (on levels of up to 200 K voxels the shorter chunk
+ * and narrower thread), and the untuned pass wherever it is not behind.  Then
+ * it times the fused schedule: of it and the steps apart, the one that an
+ * untuned level does not run has to win by 5 %.  Later registrations of those
+ * shapes use the choices:
  * cgdir_register, and a request submitted on an idle GPU, the fused
  * schedule where it won; batched registrations and requests submitted while
  * others run (they share the GPU, so throughput counts) the best per-step

@@ -263,7 +263,8 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
         // nx % 4 == 0) or two (twice the CTAs, for small levels)
         const int widths[2] = {0, 2};
         const int nw = nx % 4 == 0 && ctx->force_width == 0 ? 2 : 1;
-        float bt = 1e30f, dms = 0.f;
+        const bool wave = N > 200000;
+        float least = 1e30f;
         for (int wi = 0; wi < nw && rc == CGDIR_OK; ++wi) {
             a.pass2_width = ctx->force_width > 0 ? ctx->force_width : widths[wi];
             for (int ci = 0; ci < 4 && rc == CGDIR_OK; ++ci) {
@@ -273,21 +274,21 @@ int tune_level(cgdir_ctx *ctx, int nx, int ny, int nz, int k, int contour, int s
                 float ms = 0.f;
                 rc = time_ms(ctx, e0, e1, reps, graph, &ms,
                              [&](cudaStream_t st) { return launch_force(a, cand[ci], nullptr, st, kerr(ctx)); });
-                if (wi == 0 && ci == 0) dms = ms;
-                if (rc == CGDIR_OK && ms < bt) {
-                    bt = ms;
+                // within 3 % of the fastest (what timings of two runs may differ
+                // by, and a third of it in an iteration) the longer chunk (fewer
+                // CTAs and halo planes) stands; on a level of less than a wave
+                // (where the default shape, too, takes one plane per thread) the
+                // shorter chunk and the narrower thread
+                const bool preferred = wave ? cand[ci] > best.force_zchunk && widths[wi] == best.force_width
+                                            : cand[ci] < best.force_zchunk ||
+                                                  (cand[ci] == best.force_zchunk && widths[wi] > best.force_width);
+                if (rc == CGDIR_OK && (ms < least || (preferred && ms <= 1.03f * least))) {
                     best.force_zchunk = cand[ci];
                     best.force_width = widths[wi];
                     best.force_ms = ms;
                 }
+                least = std::min(least, ms);
             }
-        }
-        // the first (untuned) grouping stands where the best is not ahead of it
-        // by more than timings differ from run to run
-        if (dms <= 1.03f * bt) {
-            best.force_zchunk = d;
-            best.force_width = widths[0];
-            best.force_ms = dms;
         }
         // the untuned schedule
         ForceArgs b = a;

@@ -31,9 +31,10 @@ def register(ctx, data, **more):
 
 
 def test_tuned_histories_do_not_follow_timing_noise():
-    """A level without structure terms whose chunks of 4 (the default) and 8 planes are 5 % apart as a
-    registration runs them, and tie when each launch waits for the host: every
-    tuning keeps the default, and with it the untuned sums, bit for bit."""
+    """A level without structure terms whose chunks of 4 (the default) and 8
+    planes are 5 % apart as a registration runs them, and tie when each launch
+    waits for the host: every tuning keeps the default, and with it the untuned
+    sums, bit for bit."""
     data = pair((40, 128, 128))
     with cg.Context(0) as c:
         dvf, st = register(c, data, contour_level_mask=0)
