@@ -338,7 +338,8 @@ int cgdir_compose(cgdir_ctx *ctx, const float *u, const float *du, int mode, flo
    (CGDIR_ADDITIVE), G the Gaussian of sigma voxels (0 <= sigma <= 2; 0 is
    no smoothing).  The kernels are the context's forced smoothing variant
    (CGDIR_SMOOTH at creation; under CGDIR_SMOOTH=fused one 3-D tile kernel
-   for both steps), else the z-march; every choice gives the same bits.
+   for both steps), else chosen by size and row length; every choice gives
+   the same bits.
    Fields [3][nz][ny][nx] FP32 in device memory; out must not alias u or
    du.  Errors: EINVAL, ENOMEM, ECUDA. */
 int cgdir_smooth_compose(cgdir_ctx *ctx, const float *du, const float *u, int mode, float sigma,

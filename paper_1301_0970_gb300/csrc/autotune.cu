@@ -8,11 +8,12 @@
 //              update kernel), the 3-D shared-memory tile kernel (idem), and
 //              the split xy + z kernels with the update fused into the z pass;
 //   force:     the stencil pass with the default z chunk, half, a quarter
-//              and double, at four, two and (structure terms) one voxels per
-//              thread;
+//              and double, at the widest thread and, where that is four
+//              voxels, at two, and the untuned pass;
 // then the fused schedule (force stencil pass alone, 3-D tiles of G(du)
 // with the update, 3-D tiles of G(u') with the next iteration's warp)
-// against the best of those two, summed.
+// against the best of those two, summed.  Levels of up to 2 M voxels are timed
+// as CUDA graphs.
 // The fastest of each is recorded in the context and used by every later
 // registration of that shape (and baked into its CUDA graph).
 #include "runtime_internal.hpp"

@@ -112,7 +112,7 @@ __global__ void k_restrict_image_rows(const IT *__restrict__ in, int nx, int ny,
 }
 
 // The same where nx is even and rows are aligned for pairs: the two x
-// neighbours come by one load, four coarse values per thread are in flight.
+// neighbours come by one load, a coarse value's four pairs are in flight.
 template <typename IT>
 struct PairOf { using type = unsigned; };
 template <>

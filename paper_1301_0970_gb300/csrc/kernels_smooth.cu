@@ -389,7 +389,8 @@ __global__ void __launch_bounds__(NT) k_smooth_compose_tma(const __grid_constant
 // slower at 256x256x96, 32 x 16 194, a fifth warp for the x pass 189, the x pass
 // one plane ahead of the y / z passes 189.
 // RY = 2 is the 32 x 16 tile: radii 5 and 6, whose z ring would not fit four
-// rows' registers, and the MARCH32 variant.
+// rows' registers, and the MARCH32 variant.  At radius 4 the copy-fed forms
+// spill (48 bytes with RY = 4, 32 with RY = 2); no other form does.
 constexpr int MT = 128;                // threads
 constexpr int MX = 32;                 // tile width
 template <int R, int RY>

@@ -52,7 +52,7 @@ struct WsSet {
 
 // Kernel choices for one pyramid level shape, picked by timing (autotune.cu).
 struct TunedLevel {
-    int smooth_variant = 0;    // best per-step smoothing: SMOOTH_MARCH / TILE / SPLIT (0 = the z-march)
+    int smooth_variant = 0;    // best per-step smoothing: SMOOTH_MARCH / TILE / SPLIT (0 = by size and row length)
     int smooth_zchunk = 0;     // z chunk of the z-march smoothing (0 = default)
     int force_zchunk = 0;      // z chunk of the force stencil pass (0 = default)
     int force_width = 0;       // voxels per thread of the stencil pass: 0 = the widest, 2, 1
