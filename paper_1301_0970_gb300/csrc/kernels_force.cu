@@ -608,6 +608,13 @@ __device__ __forceinline__ void plane_load(const ForceArgs &a, int ic, int ip, i
     }
 }
 
+// |du|^2 with its roundings written out (a compiler's choice of contractions
+// differs between the passes): `quad` as the four-voxel pass has them, which the
+// narrower passes take where they stand for it.
+__device__ __forceinline__ float norm2(float x, float y, float z, bool quad) {
+    return fmaf(z, z, quad ? fmaf(x, x, __fmul_rn(y, y)) : fmaf(y, y, __fmul_rn(x, x)));
+}
+
 // The chain of the RMS-ID sums over the quad x .. x + 3 and the planes from z
 // on (chain_z of them at most), as the four-voxel pass runs it.  Every load is
 // issued at once.
@@ -694,7 +701,7 @@ __global__ void __launch_bounds__(NT, 3) k_force_pass(ForceArgs a, int zchunk) {
             cnt += cur.ur ? 1 : 0;
             if (cur.ur) ssd = fmaf(r0, r0, ssd);
             if (a.chain_w == 0 && a.chain_z > 0 && (z + 1) % a.chain_z == 0) { sum.add(ssd); ssd = 0.f; }
-            if (MAXDU) mx = fmaxf(mx, dux * dux + duy * duy + duz * duz);
+            if (MAXDU) mx = fmaxf(mx, norm2(dux, duy, duz, a.chain_w == 4));
             Wm = Wc; Wc = Wp; im = ic;
             if (CONTOUR) { Sm = Sc; Sc = Sp; }
             ++z;
@@ -829,7 +836,7 @@ __global__ void __launch_bounds__(NT, 2) k_force_pass2(ForceArgs a, int zchunk) 
             if (cur.ur & 0xffu) { ssd = fmaf(r00, r00, ssd); cnt += 1; }
             if (cur.ur >> 8) { ssd = fmaf(r01, r01, ssd); cnt += 1; }
             if (a.chain_w == 0 && a.chain_z > 0 && (z + 1) % a.chain_z == 0) { sum.add(ssd); ssd = 0.f; }
-            if (MAXDU) mx = fmaxf(mx, fmaxf(d0x * d0x + d0y * d0y + d0z * d0z, d1x * d1x + d1y * d1y + d1z * d1z));
+            if (MAXDU) mx = fmaxf(mx, fmaxf(norm2(d0x, d0y, d0z, a.chain_w == 4), norm2(d1x, d1y, d1z, a.chain_w == 4)));
             Wm = Wc; Wc = cur.wp; im = ic;
             Sm = Sc; Sc = cur.sp;
             ++z;
@@ -988,7 +995,7 @@ __global__ void __launch_bounds__(NT, 2) k_force_pass4(ForceArgs a, int zchunk) 
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 if ((cur.ur >> (8 * q)) & 0xffu) { ssd = fmaf(r[q], r[q], ssd); cnt += 1; }
-                if (MAXDU) mx = fmaxf(mx, dx[q] * dx[q] + dy[q] * dy[q] + dz[q] * dz[q]);
+                if (MAXDU) mx = fmaxf(mx, norm2(dx[q], dy[q], dz[q], true));
             }
             Wm = Wc; Wc = cur.wp; im = ic;
             Sm = Sc; Sc = cur.sp;

@@ -283,3 +283,22 @@ def test_unaligned_coarse_level_takes_the_split_kernels():
             c.register(img, img, [], [], **kw)
             count.append(cg.launch_count() - before)
     assert count[1] - count[0] == 20 * 6
+
+
+@pytest.mark.parametrize("shape", [(16, 94, 72), (30, 40, 64), (40, 64, 128)])
+def test_largest_step_does_not_depend_on_the_pass(shape, monkeypatch):
+    """max |du| of the force step with structure terms on small levels, whose
+    threads are narrower than the four-voxel ones they stand for: equal to that
+    pass's, bit for bit."""
+    got = []
+    for zc in (None, default_zchunk(shape)):
+        if zc:
+            monkeypatch.setenv("CGDIR_FORCE_ZCHUNK", str(zc))
+        with cg.Context(0) as c:
+            for seed in range(40):
+                gen = torch.Generator(device=DEV).manual_seed(seed)
+                img, mov = (300 * torch.randn(shape, device=DEV, generator=gen) for _ in range(2))
+                bits = torch.randint(0, 2, shape, device=DEV, dtype=torch.uint8, generator=gen)
+                u = torch.randn((3,) + shape, device=DEV, generator=gen)
+                got.append(c.force(mov, img, bits, bits, [1e-3], [1], u, want_stats=True)[1])
+    assert got[:40] == got[40:]
