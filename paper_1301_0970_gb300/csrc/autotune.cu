@@ -163,7 +163,7 @@ int force_schedule(const cgdir_ctx *ctx, ForceArgs &a, int sdt) {
 template <typename Body>
 static int time_ms(cgdir_ctx *ctx, cudaEvent_t a, cudaEvent_t b, int reps, bool graph, float *ms, Body body) {
     cudaStream_t s = ctx->stream;
-    if (graph && ctx->cap_stream) {
+    if (graph && ctx->use_graphs && ctx->cap_stream) {
         const unsigned long long before = launches_now();
         CK(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;
